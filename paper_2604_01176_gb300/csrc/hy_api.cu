@@ -143,6 +143,23 @@ struct hy_ham {
     int64_t jl_r0 = -1, jl_r1 = -1, jl_n = 0;
 };
 
+namespace {
+
+// Whole-pool screen in double of one or many molecules (hy_screen.cu): the
+// molecules' tables, the task list and the partial sums it writes, laid out
+// when a pool is created or a batch given its pools.
+struct ScreenPlan {
+    DevArena arena;
+    hy::k::ScreenMol *d_mols = nullptr;
+    int4 *d_tasks = nullptr;
+    double *d_partials = nullptr;
+    int count = 0, cfg = 0, n_tasks = 0;
+    int64_t n_partials = 0, n_ops = 0;
+    size_t smem = 0;
+};
+
+}  // namespace
+
 struct hy_pool {
     const hy_ham *h = nullptr;
     std::vector<hy::PoolOpHost> ops;
@@ -161,6 +178,12 @@ struct hy_pool {
     unsigned long long *d_bad = nullptr;
     unsigned long long *h_bad = nullptr;
     int qubit = 0;                  // HY_POOL_QEB: qubit excitations, no sign
+    // pattern ids by electrons moved (singles, doubles) per spin, and each
+    // id's place in its list, for the whole-pool screen
+    std::vector<int32_t> sing[2], dbl[2];
+    int32_t *d_sing[2] = {nullptr, nullptr}, *d_dbl[2] = {nullptr, nullptr};
+    int32_t *d_slot[2] = {nullptr, nullptr};
+    ScreenPlan screen;
 };
 
 struct hy_batch {
@@ -191,6 +214,7 @@ struct hy_batch {
     double *d_gpart = nullptr;
     int64_t n_gpart = 0;
     unsigned long long *d_gctr = nullptr, *d_gbad = nullptr, *h_gbad = nullptr;
+    ScreenPlan screen;
 };
 
 namespace {
@@ -476,10 +500,138 @@ hy_status energy_t(hy_ham *h, const T *psi, const T *sigma, double *e, cudaStrea
     return dot_t<T>(h, psi, sigma, e, st);
 }
 
+// The screen plan of `count` molecules: pool m at state offset offs[m], its
+// operators from gbase[m].  A group is what a task stages at a time; kinds are
+// dealt to tasks in proportion to the work of their groups, about eight tasks
+// per SM in all (two to four run at once, so the last wave is a small part of
+// the launch), largest molecules first.
+hy_status build_screen_plan(ScreenPlan &sp, const hy_pool *const *pools, const int64_t *offs,
+                            const int64_t *gbase, int count, int num_sms)
+{
+    sp.arena.release();
+    sp = ScreenPlan{};
+    int64_t M = 0, nR = 0;
+    for (int m = 0; m < count; ++m) {
+        M = std::max({M, pools[m]->h->Na, pools[m]->h->Nb});
+        nR = std::max({nR, int64_t(pools[m]->dbl[0].size()), int64_t(pools[m]->dbl[1].size())});
+        sp.n_ops += int64_t(pools[m]->ops.size());
+    }
+    // strings x vectors staged: two CTAs per SM (113 KB each, less the launch's
+    // own kilobyte), one CTA per SM (227 KB), or the narrow planes
+    const int64_t acc_bytes = (nR + 3) / 4 * 32;
+    sp.cfg = 64 * M + acc_bytes <= 114 * 1000 ? 0 : 32 * M + acc_bytes <= 226 * 1024 ? 1 : 2;
+    const int64_t Q = sp.cfg == 0 ? 4 : sp.cfg == 1 ? 2 : 1;
+    std::vector<hy::k::ScreenMol> mols(count);
+    std::vector<int4> tasks;
+    std::vector<int> order(count);
+    for (int m = 0; m < count; ++m) order[m] = m;
+    std::stable_sort(order.begin(), order.end(),
+                     [&](int x, int y) { return pools[x]->h->N > pools[y]->h->N; });
+    // groups of a kind (per alpha single; alpha identity; alpha and beta
+    // doubles) and the work of one: pairs summed, and the staging
+    struct Kind { int64_t groups; double cost; };
+    auto kinds = [&](const hy_pool *p, Kind k[4]) {
+        const hy_ham *h = p->h;
+        const int64_t cb = p->sing[1].empty() ? 0 : p->pb.cnt[p->sing[1][0]];
+        const double ab = double(p->sing[1].size()) * double(cb) + 2.0 * double(h->Nb);
+        k[0] = {p->sing[0].empty() ? 0 : p->pa.cnt[p->sing[0][0]], ab};
+        k[1] = {h->Na, ab};
+        auto doubles = [&](int spin, const hy::PatternLists &pl, int64_t strs, int64_t vecs) {
+            const auto &d = p->dbl[spin];
+            if (d.empty()) return Kind{0, 0.0};
+            return Kind{(vecs + Q - 1) / Q,
+                        double(Q) * (double(d.size()) * double(pl.cnt[d[0]]) + 2.0 * double(strs))};
+        };
+        k[2] = doubles(0, p->pa, h->Na, h->Nb);
+        k[3] = doubles(1, p->pb, h->Nb, h->Na);
+    };
+    double total = 0.0;
+    for (int m = 0; m < count; ++m) {
+        Kind k[4];
+        kinds(pools[m], k);
+        total += double(pools[m]->sing[0].size()) * double(k[0].groups) * k[0].cost;
+        for (int j = 1; j < 4; ++j) total += double(k[j].groups) * k[j].cost;
+    }
+    const double per_task = std::max(total / (8.0 * num_sms), 1.0);
+    auto deal = [&](const Kind &k) {
+        const int64_t c = int64_t(std::ceil(double(k.groups) * k.cost / per_task));
+        return int(std::max<int64_t>(1, std::min(c, k.groups)));
+    };
+    for (int m : order) {
+        const hy_pool *p = pools[m];
+        const hy_ham *h = p->h;
+        hy::k::ScreenMol &q = mols[m];
+        Kind k[4];
+        kinds(p, k);
+        q.opd = p->d_op; q.cons = p->d_cons;
+        q.aent = p->d_aent; q.bent = p->d_bent;
+        q.aoff = p->d_aoff; q.acnt = p->d_acnt; q.boff = p->d_boff; q.bcnt = p->d_bcnt;
+        q.la = p->d_sing[0]; q.lb = p->d_sing[1];
+        q.ra = p->d_dbl[0]; q.rb = p->d_dbl[1];
+        q.aslot = p->d_slot[0]; q.bslot = p->d_slot[1];
+        q.off = offs[m];
+        q.gbase = gbase[m];
+        q.Na = int(h->Na); q.Nb = int(h->Nb);
+        q.nA = int(p->sing[0].size()); q.nB = int(p->sing[1].size());
+        q.nRa = int(p->dbl[0].size()); q.nRb = int(p->dbl[1].size());
+        // the identity (first in the list, a few times a single's pairs) shares
+        // the singles' chunk count
+        q.ch[0] = q.nA ? deal(k[0]) : deal(k[1]);
+        q.base[0] = sp.n_partials;
+        sp.n_partials += int64_t(q.nA + 1) * q.ch[0] * (q.nB + 1);
+        for (int ia = q.nA; ia >= 0; --ia)
+            for (int c = 0; c < q.ch[0]; ++c) tasks.push_back(make_int4(m, 0, ia, c));
+        sp.smem = std::max(sp.smem, size_t(2) * q.Nb * (sp.cfg < 2 ? 16 : 8));
+        for (int kind = 1; kind <= 2; ++kind) {
+            const int nr = kind == 1 ? q.nRa : q.nRb;
+            q.ch[kind] = nr ? deal(k[kind + 1]) : 0;
+            q.base[kind] = sp.n_partials;
+            sp.n_partials += int64_t(q.ch[kind]) * nr;
+            for (int c = 0; c < q.ch[kind]; ++c) tasks.push_back(make_int4(m, kind, 0, c));
+            if (nr)
+                sp.smem = std::max(sp.smem, size_t(Q) * (kind == 1 ? q.Na : q.Nb) * 16 +
+                                                size_t(nr + 3) / 4 * 32);
+        }
+    }
+    sp.count = count;
+    sp.n_tasks = int(tasks.size());
+    HY_CUDA(sp.arena.upload(&sp.d_mols, mols.data(), mols.size()), "upload screen plan");
+    HY_CUDA(sp.arena.upload(&sp.d_tasks, tasks.data(), tasks.size()), "upload screen tasks");
+    HY_CUDA(sp.arena.alloc(&sp.d_partials, size_t(sp.n_partials)), "screen partials");
+    return HY_OK;
+}
+
+hy_status screen_run(const ScreenPlan &sp, const double *psi, const double *sigma, double *partials,
+                     double *g, cudaStream_t st)
+{
+    hy::k::ScreenArgs a;
+    a.mols = sp.d_mols;
+    a.tasks = sp.d_tasks;
+    a.psi = psi;
+    a.sigma = sigma;
+    a.partials = partials;
+    HY_CUDA(hy::k::screen_all(a, sp.cfg, sp.n_tasks, sp.smem, sp.count, sp.n_ops, g, st),
+            "pool gradients");
+    return HY_OK;
+}
+
 template <typename T>
 hy_status grad_t(hy_ham *h, const hy_pool *p, const T *psi, const T *sigma,
                  const int32_t *ops, int64_t n_ops, double *g, cudaStream_t st)
 {
+    double bytes = 0.0;     // pairs of the listed operators (known for the whole pool)
+    if (!ops)
+        for (const auto &od : p->opd)
+            for (int q = 0; q < od.nc; ++q) {
+                const hy::k::ConsDev &cd = p->cons[q == 0 ? od.c0 : od.c1];
+                const double nr = cd.ap < 0 ? double(h->Na) : double(p->pa.cnt[cd.ap]);
+                const double nc = cd.bp < 0 ? double(h->Nb) : double(p->pb.cnt[cd.bp]);
+                bytes += 4.0 * nr * nc * sizeof(T);
+            }
+    hy::ProfScope prof(HY_PROF_SCREEN, st, bytes);
+    // whole pools in double by pattern; lists and float sums per operator
+    if constexpr (sizeof(T) == sizeof(double))
+        if (!ops) return screen_run(p->screen, psi, sigma, p->screen.d_partials, g, st);
     const WsLayout L = ws_layout(h, n_partials_needed(h, n_ops), sizeof(T));
     hy_status s = ensure_ws(h, L.total);
     if (s != HY_OK) return s;
@@ -503,16 +655,6 @@ hy_status grad_t(hy_ham *h, const hy_pool *p, const T *psi, const T *sigma,
     a.g = g;
     a.K = int64_t(p->ops.size());
     a.bad = p->d_bad;
-    double bytes = 0.0;     // pairs of the listed operators (known for the whole pool)
-    if (!ops)
-        for (const auto &od : p->opd)
-            for (int q = 0; q < od.nc; ++q) {
-                const hy::k::ConsDev &cd = p->cons[q == 0 ? od.c0 : od.c1];
-                const double nr = cd.ap < 0 ? double(h->Na) : double(p->pa.cnt[cd.ap]);
-                const double nc = cd.bp < 0 ? double(h->Nb) : double(p->pb.cnt[cd.bp]);
-                bytes += 4.0 * nr * nc * sizeof(T);
-            }
-    hy::ProfScope prof(HY_PROF_SCREEN, st, bytes);
     HY_CUDA(hy::k::grad<T>(a, st), "pool gradients");
     return HY_OK;
 }
@@ -1185,6 +1327,16 @@ hy_status hy_pool_create(const hy_ham *h, hy_pool_kind kind, hy_pool **out)
     }
     p->pa.finalize(h->A);
     p->pb.finalize(h->B);
+    std::vector<int32_t> slot[2];
+    for (int spin = 0; spin < 2; ++spin) {
+        const hy::PatternLists &pl = spin ? p->pb : p->pa;
+        for (size_t i = 0; i < pl.keys.size(); ++i) {
+            const bool single = pl.keys[i].nops == 2;
+            auto &l = single ? p->sing[spin] : p->dbl[spin];
+            slot[spin].push_back(single ? int32_t(l.size()) : -1 - int32_t(l.size()));
+            l.push_back(int32_t(i));
+        }
+    }
     hy_status s = HY_OK;
     auto up = [&](cudaError_t err, const char *what) {
         if (s == HY_OK && err != cudaSuccess) s = cuda_fail(err, what);
@@ -1208,6 +1360,15 @@ hy_status hy_pool_create(const hy_ham *h, hy_pool_kind kind, hy_pool **out)
         up(cudaMallocHost(&p->h_bad, sizeof(unsigned long long)), "list-check mirror");
         if (p->h_bad) *p->h_bad = none;
     }
+    for (int spin = 0; spin < 2; ++spin) {
+        up(ar.upload(&p->d_sing[spin], p->sing[spin].data(), p->sing[spin].size()), "upload singles");
+        up(ar.upload(&p->d_dbl[spin], p->dbl[spin].data(), p->dbl[spin].size()), "upload doubles");
+        up(ar.upload(&p->d_slot[spin], slot[spin].data(), slot[spin].size()), "upload slots");
+    }
+    if (s == HY_OK) {
+        const int64_t zero = 0;
+        s = build_screen_plan(p->screen, &p, &zero, &zero, 1, h->num_sms);
+    }
     if (s != HY_OK) {
         std::string msg = g_err;
         hy_pool_destroy(p);
@@ -1223,6 +1384,7 @@ hy_status hy_pool_destroy(hy_pool *p)
     if (!p) return HY_OK;
     if (p->h_bad) cudaFreeHost(p->h_bad);
     p->arena.release();
+    p->screen.arena.release();
     delete p;
     return HY_OK;
 }
@@ -1401,6 +1563,11 @@ hy_status grad_noalloc_t(hy_ham *h, const hy_pool *p, const T *psi, const T *sig
                          const int32_t *ops, int64_t n_ops, double *g, double *scratch,
                          cudaStream_t st)
 {
+    // the whole pool in double: the plan's partial sums fit the array at every
+    // size the library takes (at most ~220 k at 16 orbitals)
+    if constexpr (sizeof(T) == sizeof(double))
+        if (!ops && p->screen.n_partials <= kNoAllocPartials)
+            return screen_run(p->screen, psi, sigma, scratch, g, st);
     hy::k::GradArgs<T> a;
     a.psi = psi;
     a.sigma = sigma;
@@ -1915,6 +2082,7 @@ hy_status hy_batch_destroy(hy_batch *b)
     cudaFree(b->d_gctr);
     cudaFree(b->d_gbad);
     cudaFreeHost(b->h_gbad);
+    b->screen.arena.release();
     delete b;
     return HY_OK;
 }
@@ -1952,6 +2120,10 @@ hy_status hy_batch_set_pools(hy_batch *b, const hy_pool *const *pools)
                        cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(b->d_gbad, 0xFF, sizeof(unsigned long long));
     if (e != cudaSuccess) return cuda_fail(e, "batch pools");
+    b->pools.clear();
+    hy_status s = build_screen_plan(b->screen, pools, b->offsets.data(), base.data(), count,
+                                    b->num_sms);
+    if (s != HY_OK) return s;
     *b->h_gbad = ~0ull;
     b->pools.assign(pools, pools + count);
     b->pool_base = base;
@@ -1986,6 +2158,10 @@ hy_status hy_batch_gradients(hy_batch *b, const void *psi, const void *sigma, co
     const int64_t n = ops ? n_entries : b->pool_base.back();
     if (n == 0) return HY_OK;
     cudaStream_t st = as_stream(stream);
+    hy::ProfScope prof(HY_PROF_SCREEN, stream, 0.0);
+    if (!ops && dt == HY_F64)
+        return screen_run(b->screen, static_cast<const double *>(psi),
+                          static_cast<const double *>(sigma), b->screen.d_partials, g, st);
     int64_t ch = (int64_t(8) * b->num_sms + n - 1) / n;
     if (ch < 1) ch = 1;
     if (ch > 256) ch = 256;
@@ -1998,7 +2174,6 @@ hy_status hy_batch_gradients(hy_batch *b, const void *psi, const void *sigma, co
         HY_CUDA(cudaMalloc(&b->d_gpart, size_t(n * ch) * sizeof(double)), "cudaMalloc(partials)");
         b->n_gpart = n * ch;
     }
-    hy::ProfScope prof(HY_PROF_SCREEN, stream, 0.0);
     auto run = [&](auto *tag) -> cudaError_t {
         using T = std::remove_pointer_t<decltype(tag)>;
         hy::k::BatchGradArgs<T> a;

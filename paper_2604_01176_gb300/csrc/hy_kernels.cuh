@@ -541,6 +541,31 @@ cudaError_t fold_rows(const FoldArgs &a, int num_sms, cudaStream_t st);
 cudaError_t fold_compact(const FoldArgs &a, int32_t *ptr, int32_t *col, double *val64,
                          float *val32, int num_sms, cudaStream_t st);
 
+// Screen of whole pools in double, one or many molecules (hy_screen.cu).
+// Kinds of tasks: 0 alpha-beta (and every single), 1 alpha doubles, 2 beta
+// doubles.
+struct ScreenMol {
+    const OpDev *opd;
+    const ConsDev *cons;
+    const uint32_t *aent, *bent;                 // pattern pairs, as in GradArgs
+    const int64_t *aoff, *acnt, *boff, *bcnt;
+    const int32_t *la, *lb, *ra, *rb;            // ids of the singles / doubles of each spin
+    const int32_t *aslot, *bslot;                // pattern id -> place in l (>= 0), -1 - place in r
+    int64_t off;                                 // first amplitude of psi and sigma
+    int64_t gbase;                               // first operator in g
+    int64_t base[3];                             // partials of each kind
+    int ch[3];                                   // tasks a kind's groups are dealt to
+    int Na, Nb, nA, nB, nRa, nRb;
+};
+struct ScreenArgs {
+    const ScreenMol *mols;
+    const int4 *tasks;                           // (molecule, kind, alpha pattern, chunk)
+    const double *psi, *sigma;
+    double *partials;
+};
+cudaError_t screen_all(const ScreenArgs &a, int cfg, int n_tasks, size_t smem, int count,
+                       int64_t n_ops, double *g, cudaStream_t st);
+
 // Batched pool-gradient screen: per molecule its pool's pair tables (as in
 // GradArgs) and its place in the packed state buffers
 struct BatchPool {
