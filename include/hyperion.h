@@ -471,7 +471,7 @@ hy_status hy_normalize(const hy_ham *h, void *psi, hy_dtype dt, void *stream);
  * groups of tile.gsize threads; each group takes the next (molecule, alpha
  * row) task from a device work-list (largest molecules first) and computes
  * that output row completely, then writes its <psi|sigma> partial, which a
- * second small kernel sums per molecule in row order.  Intended for
+ * second small kernel sums per molecule in a fixed order.  Intended for
  * molecules of up to 12 orbitals (their tables stay in L2); larger ones are
  * correct but slow.  States are packed: molecule m's amplitudes start at
  * element offsets[m] of one buffer (offsets are multiples of 32). */

@@ -188,16 +188,18 @@ k_batch_rows(BatchArgs<T> a)
     }
 }
 
-// energies[m] = sum of molecule m's row partials, in row order
+// energies[m] = sum of molecule m's row partials in a fixed order: a warp per
+// molecule (one thread walked up to 924 rows in 84 us)
 __global__ void k_batch_energy(const double *__restrict__ row_energy,
                                const int64_t *__restrict__ base, const int64_t *__restrict__ rows,
                                int count, double *__restrict__ energies)
 {
-    const int mol = blockIdx.x * blockDim.x + threadIdx.x;
+    const int mol = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (mol >= count) return;
     double s = 0.0;
-    for (int64_t r = 0; r < rows[mol]; ++r) s += row_energy[base[mol] + r];
-    energies[mol] = s;
+    for (int64_t r = threadIdx.x & 31; r < rows[mol]; r += 32) s += row_energy[base[mol] + r];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) energies[mol] = s;
 }
 
 // ---------------------------------------------------------------------------
@@ -349,7 +351,7 @@ cudaError_t batch_occupancy(const BatchArgs<T> &a, int *per_sm)
 cudaError_t batch_energy(const double *row_energy, const int64_t *base, const int64_t *rows,
                          int count, double *energies, cudaStream_t st)
 {
-    k_batch_energy<<<(count + 63) / 64, 64, 0, st>>>(row_energy, base, rows, count, energies); hy::count_launch();
+    k_batch_energy<<<(count + 7) / 8, 256, 0, st>>>(row_energy, base, rows, count, energies); hy::count_launch();
     return cudaGetLastError();
 }
 

@@ -517,15 +517,18 @@ k_grad_sparse(SparseGradArgs<T> a)
     if (threadIdx.x == 0) a.partials[i * gridDim.y + blockIdx.y] = tot;
 }
 
+// a warp per operator: a single operator (the reverse sweep) has up to 608
+// chunks, a 26 us chain of loads for one thread
 __global__ void __launch_bounds__(256)
 k_grad_sparse_final(const double *__restrict__ partials, int chunks, int64_t n_ops,
                     double *__restrict__ g)
 {
-    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    const int64_t i = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     if (i >= n_ops) return;
     double s = 0.0;
-    for (int c = 0; c < chunks; ++c) s += partials[i * chunks + c];
-    g[i] = 2.0 * s;
+    for (int c = threadIdx.x & 31; c < chunks; c += 32) s += partials[i * chunks + c];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) g[i] = 2.0 * s;
 }
 
 // ---------------------------------------------------------------------------
@@ -2106,8 +2109,8 @@ cudaError_t grad_sparse(const SparseGradArgs<T> &a, int num_sms, cudaStream_t st
     if (a.n_ops == 0) return cudaSuccess;
     k_grad_sparse<T><<<dim3(unsigned(a.n_ops), unsigned(a.chunks)), 256, 0, st>>>(a);
     hy::count_launch();
-    k_grad_sparse_final<<<unsigned((a.n_ops + 255) / 256), 256, 0, st>>>(a.partials, a.chunks,
-                                                                       a.n_ops, a.g);
+    k_grad_sparse_final<<<unsigned((a.n_ops + 7) / 8), 256, 0, st>>>(a.partials, a.chunks,
+                                                                     a.n_ops, a.g);
     hy::count_launch();
     return cudaGetLastError();
 }

@@ -198,15 +198,19 @@ k_grad_partial(GradArgs<T> a)
     if (threadIdx.x == 0) a.partials[i * a.CH + chunk] = tot;
 }
 
+// A warp per operator, lanes over its chunks: one operator alone (the reverse
+// sweep asks for one at a time) has 608 of them, a 41 us chain of loads for a
+// single thread, 3 us for a warp.
 __global__ void __launch_bounds__(256)
 k_grad_final(const double *__restrict__ partials, int CH, int64_t n_ops,
              double *__restrict__ g)
 {
-    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    const int64_t i = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     if (i >= n_ops) return;
     double s = 0.0;
-    for (int c = 0; c < CH; ++c) s += partials[i * CH + c];
-    g[i] = 2.0 * s;
+    for (int c = threadIdx.x & 31; c < CH; c += 32) s += partials[i * CH + c];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) g[i] = 2.0 * s;
 }
 
 template <typename T>
@@ -215,8 +219,7 @@ cudaError_t grad(const GradArgs<T> &a, cudaStream_t st)
     if (a.n_ops == 0) return cudaSuccess;
     dim3 grid(unsigned(a.n_ops), unsigned(a.CH));
     k_grad_partial<T><<<grid, 256, 0, st>>>(a); hy::count_launch();
-    k_grad_final<<<unsigned((a.n_ops + 255) / 256), 256, 0, st>>>(a.partials, a.CH,
-                                                                 a.n_ops, a.g); hy::count_launch();
+    k_grad_final<<<unsigned((a.n_ops + 7) / 8), 256, 0, st>>>(a.partials, a.CH, a.n_ops, a.g); hy::count_launch();
     return cudaGetLastError();
 }
 
