@@ -178,7 +178,8 @@ hy_status hy_ham_info(const hy_ham *h, int64_t *n_det, int64_t *n_alpha_str,
                       int64_t *n_terms);
 
 /* With enable != 0, every later hy_apply_h records a pair of CUDA events on
- * its stream around the alpha-beta coupling kernel(s); hy_ham_coupling_ms
+ * its stream around the alpha-beta coupling kernel(s) (HY_F64 with up to
+ * 1,716 beta strings: around the one kernel of the sweep); hy_ham_coupling_ms
  * waits for the last pair and returns the elapsed milliseconds (host).  Off
  * by default; the events cost nothing when off. */
 hy_status hy_ham_profile(hy_ham *h, int enable);
@@ -467,11 +468,14 @@ hy_status hy_normalize(const hy_ham *h, void *psi, hy_dtype dt, void *stream);
 /* ---------------------------------------------------------------------- */
 
 /* A batch runs sigma = H psi (and the energies <psi|sigma>) for many
- * molecules of uneven size in one persistent launch: CTAs are split into
- * groups of tile.gsize threads; each group takes the next (molecule, alpha
- * row) task from a device work-list (largest molecules first) and computes
- * that output row completely, then writes its <psi|sigma> partial, which a
- * second small kernel sums per molecule in a fixed order.  Intended for
+ * molecules of uneven size in one launch over their output rows, largest
+ * molecules first; each task also writes its <psi|sigma> partial, which a
+ * second small kernel sums per molecule in a fixed order.  HY_F32, and
+ * HY_F64 when a molecule has more than 1,716 beta strings: a persistent
+ * launch whose CTAs are split into groups of tile.gsize threads, each taking
+ * the next (molecule, alpha row) from a device work-list.  HY_F64 otherwise:
+ * a CTA per row and chunk of columns, whatever the tile (hy_batch_tune then
+ * times it once and keeps the tile).  Intended for
  * molecules of up to 12 orbitals (their tables stay in L2); larger ones are
  * correct but slow.  States are packed: molecule m's amplitudes start at
  * element offsets[m] of one buffer (offsets are multiples of 32). */

@@ -110,6 +110,9 @@ struct hy_ham {
     uint16_t *d_rank16 = nullptr;   // [1 << n] colex rank of every n-bit string
     DevCsr<double> Ma64, Mb64;
     DevCsr<float> Ma32, Mb32;
+    // Mb64 by column, for spaces of up to kRowsMaxNb beta strings (hy_rows64.cu)
+    double *d_mbv = nullptr;
+    uint16_t *d_mbc = nullptr;
     double *d_V64 = nullptr;
     float *d_V32 = nullptr;
     double *d_h1 = nullptr, *d_eri = nullptr;   // integrals (ranker features)
@@ -196,6 +199,13 @@ struct hy_batch {
     hy::k::BatchMol<double> *d_mols64 = nullptr;
     hy::k::BatchMol<float> *d_mols32 = nullptr;
     int2 *d_tasks = nullptr;
+    // double: rows x column chunks of every molecule in one plain launch, when
+    // all of them have at most kRowsMaxNb beta strings
+    hy::k::Rows64Mol *d_rows64 = nullptr;
+    int2 *d_tasks64 = nullptr;
+    int64_t n_tasks64 = 0;
+    size_t smem64 = 0;
+    int64_t *d_base64 = nullptr, *d_rows64n = nullptr;   // row_energy spans per molecule
     int *d_counter = nullptr;
     double *d_row_energy = nullptr;
     int64_t *d_base = nullptr, *d_rows = nullptr;
@@ -351,6 +361,45 @@ hy_status coupling_jlist(hy_ham *h, int64_t r0, int64_t r1, const int32_t **list
     return HY_OK;
 }
 
+// Tables of one molecule for the batched kernels; offset and task_base are the
+// caller's.
+template <typename T>
+hy::k::BatchMol<T> batch_mol(const hy_ham *h)
+{
+    hy::k::BatchMol<T> m{};
+    m.Na = h->Na;
+    m.Nb = h->Nb;
+    m.n = h->n;
+    m.nexa = h->A.nex;
+    m.nexb = h->B.nex;
+    const DevCsr<T> *Ma, *Mb;
+    if constexpr (sizeof(T) == sizeof(double)) {
+        Ma = &h->Ma64; Mb = &h->Mb64; m.V = h->d_V64;
+    } else {
+        Ma = &h->Ma32; Mb = &h->Mb32; m.V = h->d_V32;
+    }
+    m.Ma_ptr = Ma->ptr; m.Ma_col = Ma->col; m.Ma_val = Ma->val;
+    m.Mb_ptr = Mb->ptr; m.Mb_col = Mb->col; m.Mb_val = Mb->val;
+    m.aex = h->d_aex; m.bexT = h->d_bexT; m.astr = h->d_astr; m.bstr = h->d_bstr;
+    return m;
+}
+
+// columns per chunk: as even as the chunks can be
+int rows64_chunks(const hy_ham *h, int cols)
+{
+    return int(std::max<int64_t>(1, (h->Nb + cols - 1) / cols));
+}
+
+hy::k::Rows64Mol rows64_mol(const hy_ham *h, int cols)
+{
+    hy::k::Rows64Mol r{};
+    r.m = batch_mol<double>(h);
+    r.Mb_colv = h->d_mbv;
+    r.Mb_colc = h->d_mbc;
+    r.chunks = rows64_chunks(h, cols);
+    return r;
+}
+
 // sigma rows [r0, r1) (alpha strings) of H psi; sigma holds those rows only.
 // Every output element is formed by the same arithmetic in the same order
 // whatever the range, so shards concatenate to the full sigma bit for bit.
@@ -359,6 +408,26 @@ hy_status apply_h_t(hy_ham *h, const T *psi, T *sigma, cudaStream_t st, int64_t 
 {
     const int64_t nr = r1 - r0;
     if (nr <= 0) return HY_OK;
+    if constexpr (sizeof(T) == sizeof(double)) {
+        // one launch where a few partner rows fit an SM twice over
+        if (h->d_mbv) {
+            const double rows_det = double(nr) * double(h->Nb);
+            hy::ProfScope prof(HY_PROF_HPSI, st, 2.0 * rows_det * sizeof(T),
+                               2.0 * double(hy::ham_connections(h)) * rows_det);
+            hy::k::Rows64Args a{};
+            a.psi = psi;
+            a.sigma = sigma;
+            const int slices = h->N <= hy::k::kRowsSmallN ? hy::k::kRowsSlices : 1;
+            a.mol = rows64_mol(h, slices > 1 ? hy::k::kRowsColsSmall : hy::k::kRowsCols);
+            a.mol.row0 = r0;
+            const int64_t width = (h->Nb + a.mol.chunks - 1) / a.mol.chunks;
+            if (h->prof) cudaEventRecord(h->ev0, st);
+            HY_CUDA(hy::k::rows64(a, nr * a.mol.chunks, slices, int((width + 31) / 32 * 32),
+                                  hy::k::rows64_smem(h->Nb, h->n, slices), st), "H psi rows");
+            if (h->prof) cudaEventRecord(h->ev1, st);
+            return HY_OK;
+        }
+    }
     const WsLayout L = ws_layout(h, n_partials_needed(h, 0), sizeof(T));
     // float: room for the dense coupling's intermediate T after the state
     // buffers, sized before any launch; without it the direct kernel runs
@@ -848,6 +917,13 @@ hy_status fold_same_spin(hy_ham *h)
         if (e == cudaSuccess)
             e = cudaMemcpy(&nnz, M64.ptr + N, sizeof(int32_t), cudaMemcpyDeviceToHost);
         (spin == 0 ? h->nnz_a : h->nnz_b) = nnz;
+        if (spin == 1 && N <= hy::k::kRowsMaxNb && e == cudaSuccess) {
+            e = ar.alloc(&h->d_mbv, size_t(cap > 0 ? cap : 1));
+            if (e == cudaSuccess) e = ar.alloc(&h->d_mbc, size_t(cap > 0 ? cap : 1));
+            if (e == cudaSuccess)
+                e = hy::k::rows64_table(M64.ptr, M64.col, M64.val, int(N), h->d_mbv, h->d_mbc,
+                                        nullptr);
+        }
     }
     done();
     if (e != cudaSuccess) return cuda_fail(e, "same-spin tables");
@@ -1949,6 +2025,21 @@ hy_status batch_apply_t(hy_batch *b, const void *psi, void *sigma, double *energ
                         cudaStream_t st)
 {
     if (!tile_ok(b, b->tile, sizeof(T))) return fail(HY_ERR_ARG, "tile shape does not fit");
+    if constexpr (sizeof(T) == sizeof(double)) {
+        if (b->d_rows64) {
+            hy::k::Rows64Args r{};
+            r.psi = static_cast<const double *>(psi);
+            r.sigma = static_cast<double *>(sigma);
+            r.mols = b->d_rows64;
+            r.tasks = b->d_tasks64;
+            r.row_energy = energies ? b->d_row_energy : nullptr;
+            HY_CUDA(hy::k::rows64(r, b->n_tasks64, 1, hy::k::kRowsCols, b->smem64, st), "batch rows");
+            if (energies)
+                HY_CUDA(hy::k::batch_energy(b->d_row_energy, b->d_base64, b->d_rows64n,
+                                            int(b->hams.size()), energies, st), "batch energies");
+            return HY_OK;
+        }
+    }
     hy::k::BatchArgs<T> a = batch_args<T>(b, psi, sigma, energies ? b->d_row_energy : nullptr);
     int per_sm = 0;
     HY_CUDA(hy::k::batch_occupancy<T>(a, &per_sm), "batch occupancy");
@@ -2010,26 +2101,24 @@ hy_status hy_batch_create(const hy_ham *const *hams, int count, hy_batch **out)
     b->total = off;
     std::vector<hy::k::BatchMol<double>> m64(count);
     std::vector<hy::k::BatchMol<float>> m32(count);
-    std::vector<int64_t> base(count), rows(count);
-    int64_t tb = 0;
+    std::vector<hy::k::Rows64Mol> r64(count);
+    std::vector<int64_t> base(count), rows(count), base64(count), rows64(count);
+    int64_t tb = 0, tb64 = 0;
+    bool small64 = true;
     for (int i = 0; i < count; ++i) {
         const hy_ham *h = hams[i];
-        auto fill = [&](auto &m, const auto &Ma, const auto &Mb, const auto *V) {
-            m.offset = b->offsets[i];
-            m.Na = h->Na;
-            m.Nb = h->Nb;
-            m.task_base = tb;
-            m.n = h->n;
-            m.nexa = h->A.nex;
-            m.nexb = h->B.nex;
-            m.pad = 0;
-            m.Ma_ptr = Ma.ptr; m.Ma_col = Ma.col; m.Ma_val = Ma.val;
-            m.Mb_ptr = Mb.ptr; m.Mb_col = Mb.col; m.Mb_val = Mb.val;
-            m.V = V;
-            m.aex = h->d_aex; m.bexT = h->d_bexT; m.astr = h->d_astr; m.bstr = h->d_bstr;
-        };
-        fill(m64[i], h->Ma64, h->Mb64, h->d_V64);
-        fill(m32[i], h->Ma32, h->Mb32, h->d_V32);
+        m64[i] = batch_mol<double>(h);
+        m32[i] = batch_mol<float>(h);
+        m64[i].offset = m32[i].offset = b->offsets[i];
+        m64[i].task_base = m32[i].task_base = tb;
+        r64[i] = rows64_mol(h, hy::k::kRowsCols);
+        r64[i].m.offset = b->offsets[i];
+        r64[i].task_base = tb64;
+        small64 = small64 && h->d_mbv;
+        base64[i] = tb64;
+        rows64[i] = h->Na * r64[i].chunks;
+        tb64 += rows64[i];
+        b->smem64 = std::max(b->smem64, hy::k::rows64_smem(h->Nb, h->n, 1));
         base[i] = tb;
         rows[i] = h->Na;
         tb += h->Na;
@@ -2038,6 +2127,11 @@ hy_status hy_batch_create(const hy_ham *const *hams, int count, hy_batch **out)
     for (int i : b->order)
         for (int64_t r = 0; r < hams[i]->Na; ++r) tasks.push_back(make_int2(i, int(r)));
     b->n_tasks = int64_t(tasks.size());
+    std::vector<int2> tasks64;
+    if (small64)
+        for (int i : b->order)
+            for (int64_t t = 0; t < rows64[i]; ++t) tasks64.push_back(make_int2(i, int(t)));
+    b->n_tasks64 = int64_t(tasks64.size());
     hy_status s = HY_OK;
     auto up = [&](cudaError_t err, const char *what) {
         if (s == HY_OK && err != cudaSuccess) s = cuda_fail(err, what);
@@ -2052,7 +2146,14 @@ hy_status hy_batch_create(const hy_ham *const *hams, int count, hy_batch **out)
     put(&b->d_mols32, m32.data(), m32.size(), "batch tables");
     put(&b->d_tasks, tasks.data(), tasks.size(), "batch tasks");
     put(&b->d_counter, static_cast<const int *>(nullptr), 1, "batch counter");
-    put(&b->d_row_energy, static_cast<const double *>(nullptr), size_t(tb), "batch partials");
+    put(&b->d_row_energy, static_cast<const double *>(nullptr), size_t(std::max(tb, tb64)),
+        "batch partials");
+    if (small64) {
+        put(&b->d_rows64, r64.data(), r64.size(), "batch tables");
+        put(&b->d_tasks64, tasks64.data(), tasks64.size(), "batch tasks");
+        put(&b->d_base64, base64.data(), base64.size(), "batch tables");
+        put(&b->d_rows64n, rows64.data(), rows64.size(), "batch tables");
+    }
     put(&b->d_base, base.data(), base.size(), "batch tables");
     put(&b->d_rows, rows.data(), rows.size(), "batch tables");
     if (s != HY_OK) {
@@ -2072,6 +2173,10 @@ hy_status hy_batch_destroy(hy_batch *b)
     cudaFree(b->d_mols64);
     cudaFree(b->d_mols32);
     cudaFree(b->d_tasks);
+    cudaFree(b->d_rows64);
+    cudaFree(b->d_tasks64);
+    cudaFree(b->d_base64);
+    cudaFree(b->d_rows64n);
     cudaFree(b->d_counter);
     cudaFree(b->d_row_energy);
     cudaFree(b->d_base);
@@ -2303,10 +2408,13 @@ hy_status hy_batch_tune(hy_batch *b, const void *psi, void *sigma, hy_dtype dt,
     hy_batch_tile win = saved;
     double win_ms = 1e300;
     hy_status s = HY_OK;
+    // double batches of small molecules run without the tile: time it as it is
+    const bool fixed = dt == HY_F64 && b->d_rows64;
     for (int gsize = 32; gsize <= 512 && s == HY_OK; gsize *= 2)
         for (int groups = 1; groups <= 8 && s == HY_OK; groups *= 2) {
             hy_batch_tile t{gsize, groups, 0};
-            if (!tile_ok(b, t, elem)) continue;
+            if (fixed) t = saved;
+            if (!tile_ok(b, t, elem) || (fixed && win_ms < 1e300)) continue;
             b->tile = t;
             for (int w = 0; w < 2 && s == HY_OK; ++w) s = batch_apply(b, psi, sigma, dt, nullptr, st);
             if (s != HY_OK) break;

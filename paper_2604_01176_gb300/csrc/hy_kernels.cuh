@@ -516,6 +516,41 @@ template <typename T>
 cudaError_t batch_rows(const BatchArgs<T> &a, int grid, cudaStream_t st);
 template <typename T>
 cudaError_t batch_occupancy(const BatchArgs<T> &a, int *per_sm);
+// H psi in double over small beta string spaces, one or many molecules
+// (hy_rows64.cu), the beta table by column: entry k of string b at
+// [k * Nb + b].
+// kRowsMaxNb: 13 orbitals at half filling, 15.3 ms -> 13.2 ms there; at 14
+// (3,432 strings) the two tie, 73.8 against 74.6 ms, and the table by column
+// would take 17 MB.  kRowsCols: 308 of 320 lanes work at 12 orbitals (256: 3.20
+// ms, 320: 3.03, 480: 3.12).  Up to kRowsSmallN determinants there are fewer
+// than about four warps of columns per quarter SM: kRowsSlices slices of
+// kRowsColsSmall columns (8 orbitals: 25 us, 33 with two slices, 41 with none;
+// 11 orbitals, 213 k determinants: 657 us against 647 without).
+constexpr int kRowsCols = 320, kRowsColsSmall = 64, kRowsSlices = 4;
+constexpr int64_t kRowsSmallN = 131072;
+constexpr int64_t kRowsMaxNb = 1716;
+struct Rows64Mol {
+    BatchMol<double> m;
+    const double *Mb_colv;
+    const uint16_t *Mb_colc;
+    int64_t row0;            // first output row (sigma holds row row0 first)
+    int64_t task_base;       // first entry of row_energy
+    int chunks;              // column chunks per row
+};
+struct Rows64Args {
+    const double *psi;
+    double *sigma;
+    const Rows64Mol *mols;   // or nullptr: the molecule below
+    const int2 *tasks;       // (molecule, row * chunks + chunk), or nullptr
+    double *row_energy;      // per-task <psi|sigma> partials or nullptr
+    Rows64Mol mol;
+};
+size_t rows64_smem(int64_t Nb, int n, int slices);
+cudaError_t rows64(const Rows64Args &a, int64_t n_tasks, int slices, int cols, size_t smem,
+                   cudaStream_t st);
+cudaError_t rows64_table(const int32_t *ptr, const int32_t *col, const double *val, int Nb,
+                         double *cv, uint16_t *cc, cudaStream_t st);
+
 // Same-spin kernel table of one spin folded on the device from the Pauli
 // table (hy_fold.cu): candidates of row r = the diagonal, the singles and the
 // doubles of str[r]; element = the Pauli group with X-mask K ^ J evaluated on J
