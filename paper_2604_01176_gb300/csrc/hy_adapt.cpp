@@ -203,6 +203,19 @@ const int64_t kHssMaxEntries = int64_t(1) << 29;
 // bound) and 1.24 ns (float, tensor-core coupling) per determinant
 const double kScatterPerDense[2] = {20.0, 135.0};
 
+// cos, sin of the angles to the device (the staging slot's previous copy was
+// waited for by the evaluation that made it)
+hy_status upload_angles(hy_adapt *a, const std::vector<double> &th, cudaStream_t st)
+{
+    for (size_t l = 0; l < th.size(); ++l) {
+        a->h_cs[2 * l] = std::cos(th[l]);
+        a->h_cs[2 * l + 1] = std::sin(th[l]);
+    }
+    if (th.empty()) return HY_OK;
+    return xfer(a, a->d_cs, a->h_cs, th.size() * 2 * sizeof(double), cudaMemcpyHostToDevice, st,
+                "angles");
+}
+
 // The sparse evaluation: psi = U(theta)|HF> as a sparse vector (rotations
 // cost O(support)), renormalised over its support in double (float states),
 // sigma = H psi by the scatter, E = <psi|sigma> over the support.  *ok =
@@ -221,14 +234,7 @@ hy_status energy_sparse(hy_adapt *a, const std::vector<double> &th, hy_dtype dt,
                           a->prog_ops == a->ops;
     bool prog_build = false;
     int64_t steps = 0;
-    if (a->prep_small) {
-        for (size_t l = 0; l < L; ++l) {
-            a->h_cs[2 * l] = std::cos(th[l]);
-            a->h_cs[2 * l + 1] = std::sin(th[l]);
-        }
-        if (L) HY_TRY(xfer(a, a->d_cs, a->h_cs, L * 2 * sizeof(double), cudaMemcpyHostToDevice, st,
-                           "angles"));
-    }
+    if (a->prep_small) HY_TRY(upload_angles(a, th, st));
     if (prog_run) {
         HY_TRY(hy::prog_prepare(a->prog, S, a->p, a->d_ops, a->d_cs, int64_t(L), dt == HY_F32,
                                 a->d_n2, st));
@@ -385,6 +391,21 @@ hy_status energy_sparse(hy_adapt *a, const std::vector<double> &th, hy_dtype dt,
     return HY_OK;
 }
 
+// sigma = H psi and E = <psi|sigma> of the dense state in buf[dt][0]
+hy_status dense_energy(hy_adapt *a, const std::vector<double> &th, hy_dtype dt, cudaStream_t st,
+                       double *e)
+{
+    const int d = di(dt);
+    void *psi = a->buf[d][0], *sigma = a->buf[d][1];
+    HY_TRY(hy_apply_h(a->h, psi, sigma, dt, st));
+    a->sigma_full[d] = true;
+    HY_TRY(hy_energy(a->h, psi, sigma, dt, a->d_e, st));
+    HY_TRY(xfer(a, a->h_e, a->d_e, sizeof(double), cudaMemcpyDeviceToHost, st, "energy readback"));
+    HY_TRY(cu(cudaStreamSynchronize(st), "sync"));
+    *e = a->h_e[0];
+    return finish_energy(a, th, dt);
+}
+
 // psi = U(theta) |HF>, sigma = H psi, returns E = <psi|sigma>; speculate:
 // the caller will most likely ask for the gradient at th next
 hy_status energy(hy_adapt *a, const std::vector<double> &th, hy_dtype dt,
@@ -400,12 +421,18 @@ hy_status energy(hy_adapt *a, const std::vector<double> &th, hy_dtype dt,
         if (ok) return finish_energy(a, th, dt);
         a->sparse_fail_len[d] = a->ops.size();
     }
-    void *psi = a->buf[d][0], *sigma = a->buf[d][1];
+    void *psi = a->buf[d][0];
     a->ss_clean[d][0] = false;
     a->ss_clean[d][3] = false;
     a->sig_listed[d] = false;
     a->sig_support[d] = false;
     a->prog_support[d] = false;
+    if (hy::dense_chain_ok(a->h, dt, int64_t(a->ops.size()))) {
+        HY_TRY(upload_angles(a, th, st));
+        HY_TRY(hy::dense_chain_prepare(a->h, a->p, a->d_ops, a->d_cs, int64_t(a->ops.size()), psi,
+                                       dt, a->d_n2, st));
+        return dense_energy(a, th, dt, st, e);
+    }
     HY_TRY(set_hf(a, psi, dt, st));
     // float states: the squared norm is tracked through the rotations in
     // double and the state renormalised once after the last one (equal to
@@ -420,12 +447,7 @@ hy_status energy(hy_adapt *a, const std::vector<double> &th, hy_dtype dt,
             HY_TRY(hy_apply_excitation(a->h, a->p, a->ops[l], th[l], psi, dt, 0, st));
     }
     if (track) HY_TRY(hy_renormalize(a->h, psi, dt, a->d_n2, st));
-    HY_TRY(hy_apply_h(a->h, psi, sigma, dt, st));
-    a->sigma_full[d] = true;
-    HY_TRY(hy_energy(a->h, psi, sigma, dt, a->d_e, st));
-    HY_TRY(xfer(a, e, a->d_e, sizeof(double), cudaMemcpyDeviceToHost, st, "energy readback"));
-    HY_TRY(cu(cudaStreamSynchronize(st), "sync"));
-    return finish_energy(a, th, dt);
+    return dense_energy(a, th, dt, st, e);
 }
 
 // adjoint gradient at the point of the last energy() call in dt
@@ -438,17 +460,26 @@ hy_status gradient_dense(hy_adapt *a, const std::vector<double> &th, hy_dtype dt
     void *phi = a->buf[d][2], *lam = a->buf[d][3];
     a->ss_clean[d][1] = false;
     a->ss_clean[d][2] = false;
-    HY_TRY(cu(cudaMemcpyAsync(phi, psi, size_t(a->N) * es, cudaMemcpyDeviceToDevice, st), "copy"));
-    HY_TRY(cu(cudaMemcpyAsync(lam, sigma, size_t(a->N) * es, cudaMemcpyDeviceToDevice, st), "copy"));
-    for (size_t l = j; l-- > 0;) {
-        HY_TRY(hy::pool_gradients_unchecked(a->h, a->p, phi, lam, a->d_ops + l, 1, a->d_ga + l, dt, st));
-        if (l == 0) break;
-        HY_TRY(hy_apply_excitation(a->h, a->p, a->ops[l], -th[l], phi, dt, 0, st));
-        HY_TRY(hy_apply_excitation(a->h, a->p, a->ops[l], -th[l], lam, dt, 0, st));
+    if (hy::dense_chain_ok(a->h, dt, int64_t(j))) {
+        HY_TRY(upload_angles(a, th, st));
+        HY_TRY(hy::dense_chain_gradient(a->h, a->p, a->d_ops, a->d_cs, int64_t(j), psi, sigma, dt,
+                                        a->d_ga, st));
+    } else {
+        HY_TRY(cu(cudaMemcpyAsync(phi, psi, size_t(a->N) * es, cudaMemcpyDeviceToDevice, st), "copy"));
+        HY_TRY(cu(cudaMemcpyAsync(lam, sigma, size_t(a->N) * es, cudaMemcpyDeviceToDevice, st), "copy"));
+        for (size_t l = j; l-- > 0;) {
+            HY_TRY(hy::pool_gradients_unchecked(a->h, a->p, phi, lam, a->d_ops + l, 1, a->d_ga + l, dt,
+                                                st));
+            if (l == 0) break;
+            HY_TRY(hy_apply_excitation(a->h, a->p, a->ops[l], -th[l], phi, dt, 0, st));
+            HY_TRY(hy_apply_excitation(a->h, a->p, a->ops[l], -th[l], lam, dt, 0, st));
+        }
     }
-    HY_TRY(xfer(a, g.data(), a->d_ga, j * sizeof(double), cudaMemcpyDeviceToHost, st,
+    HY_TRY(xfer(a, a->h_g, a->d_ga, j * sizeof(double), cudaMemcpyDeviceToHost, st,
                 "gradient readback"));
-    return cu(cudaStreamSynchronize(st), "sync");
+    HY_TRY(cu(cudaStreamSynchronize(st), "sync"));
+    std::copy(a->h_g, a->h_g + j, g.begin());
+    return HY_OK;
 }
 
 // sigma = H psi in full for the sparse psi of the last evaluation in dt (whose

@@ -1535,6 +1535,52 @@ hy_status pool_gradients_unchecked(const hy_ham *hc, const hy_pool *p, const voi
                          as_stream(stream));
 }
 
+bool dense_chain_ok(const hy_ham *h, hy_dtype dt, int64_t L)
+{
+    if (h->N > k::kDenseMaxN || L > k::kDenseMaxOps) return false;
+    // float: one operator's screen deals its rows to 4 chunks per SM of 256
+    // columns, so up to these counts no thread of it adds two pairs in float
+    return dt == HY_F64 || (h->Na <= int64_t(4) * h->num_sms && h->Nb <= 256);
+}
+
+namespace {
+k::DensePool dense_pool(const hy_ham *h, const hy_pool *p)
+{
+    return {p->d_op, p->d_cons, p->d_aent, p->d_bent, p->d_aoff, p->d_acnt, p->d_boff, p->d_bcnt,
+            int(h->Na), int(h->Nb)};
+}
+}  // namespace
+
+hy_status dense_chain_prepare(const hy_ham *h, const hy_pool *p, const int32_t *ops,
+                              const double *cs, int64_t L, void *psi, hy_dtype dt, double *norm2,
+                              void *stream)
+{
+    ProfScope prof(HY_PROF_EXCITE, stream, 0.0);
+    const k::DensePool d = dense_pool(h, p);
+    HY_CUDA(dt == HY_F64 ? k::dense_prepare<double>(d, ops, cs, int(L), static_cast<double *>(psi),
+                                                    norm2, as_stream(stream))
+                         : k::dense_prepare<float>(d, ops, cs, int(L), static_cast<float *>(psi),
+                                                   norm2, as_stream(stream)),
+            "ansatz preparation");
+    return HY_OK;
+}
+
+hy_status dense_chain_gradient(const hy_ham *h, const hy_pool *p, const int32_t *ops,
+                               const double *cs, int64_t L, const void *psi, const void *sigma,
+                               hy_dtype dt, double *g, void *stream)
+{
+    ProfScope prof(HY_PROF_SCREEN, stream, 0.0);
+    const k::DensePool d = dense_pool(h, p);
+    cudaStream_t st = as_stream(stream);
+    HY_CUDA(dt == HY_F64
+                ? k::dense_gradient<double>(d, ops, cs, int(L), static_cast<const double *>(psi),
+                                            static_cast<const double *>(sigma), g, st)
+                : k::dense_gradient<float>(d, ops, cs, int(L), static_cast<const float *>(psi),
+                                           static_cast<const float *>(sigma), g, st),
+            "ansatz gradient");
+    return HY_OK;
+}
+
 // Operator lists of the public screens.  A list in pageable host memory (the
 // caller wrote it on the host) is range-checked here, before any launch; a
 // device, pinned or managed list may still be written by work queued on the

@@ -145,6 +145,18 @@ class ProfScope {
     void *a_;
 };
 
+// The rotations of an ansatz on a small dense state, and its gradient, in one
+// launch each (hy_dense.cu); false where the per-rotation launches serve:
+// more than kDenseMaxN determinants, a longer ansatz, or float string counts
+// whose per-operator screens add several pairs in float
+bool dense_chain_ok(const hy_ham *h, hy_dtype dt, int64_t L);
+hy_status dense_chain_prepare(const hy_ham *h, const hy_pool *p, const int32_t *ops,
+                              const double *cs, int64_t L, void *psi, hy_dtype dt, double *norm2,
+                              void *stream);
+hy_status dense_chain_gradient(const hy_ham *h, const hy_pool *p, const int32_t *ops,
+                               const double *cs, int64_t L, const void *psi, const void *sigma,
+                               hy_dtype dt, double *g, void *stream);
+
 // ---------------------------------------------------------------------------
 // Sparse state vectors for the ADAPT driver (implemented in hy_api.cu over
 // the kernels of hy_sparse.cu).  A SparseState owns a support list of

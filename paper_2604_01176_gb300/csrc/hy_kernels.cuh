@@ -196,6 +196,25 @@ struct ProdAcc<double> {
     __device__ __forceinline__ double total() { return d; }
 };
 
+// preparation and gradient of an ansatz on a small dense state, one cluster
+// launch each (hy_dense.cu): ops and cs[2l], cs[2l+1] = cos, sin theta_l on
+// the device
+constexpr int64_t kDenseMaxN = 65536;
+constexpr int kDenseMaxOps = 192;            // shared memory of the gradient: 448 bytes each
+struct DensePool {
+    const OpDev *opd;
+    const ConsDev *cons;
+    const uint32_t *aent, *bent;
+    const int64_t *aoff, *acnt, *boff, *bcnt;
+    int Na, Nb;
+};
+template <typename T>
+cudaError_t dense_prepare(const DensePool &p, const int32_t *ops, const double *cs, int L, T *psi,
+                          double *norm2, cudaStream_t st);
+template <typename T>
+cudaError_t dense_gradient(const DensePool &p, const int32_t *ops, const double *cs, int L,
+                           const T *psi, const T *sigma, double *g, cudaStream_t st);
+
 // learned ranker (hy_ranker.cu)
 constexpr int kRankerFeatures = 16;
 constexpr int kTopKMax = 8192;
