@@ -698,9 +698,10 @@ hy_status grad_t(hy_ham *h, const hy_pool *p, const T *psi, const T *sigma,
                 bytes += 4.0 * nr * nc * sizeof(T);
             }
     hy::ProfScope prof(HY_PROF_SCREEN, st, bytes);
-    // whole pools in double by pattern; lists and float sums per operator
+    // whole pools in double by pattern, from kScreenMinN determinants; lists,
+    // small states and float sums per operator
     if constexpr (sizeof(T) == sizeof(double))
-        if (!ops) return screen_run(p->screen, psi, sigma, p->screen.d_partials, g, st);
+        if (!ops && h->N >= hy::k::kScreenMinN) return screen_run(p->screen, psi, sigma, p->screen.d_partials, g, st);
     const WsLayout L = ws_layout(h, n_partials_needed(h, n_ops), sizeof(T));
     hy_status s = ensure_ws(h, L.total);
     if (s != HY_OK) return s;
@@ -1443,7 +1444,8 @@ hy_status hy_pool_create(const hy_ham *h, hy_pool_kind kind, hy_pool **out)
     }
     if (s == HY_OK) {
         const int64_t zero = 0;
-        s = build_screen_plan(p->screen, &p, &zero, &zero, 1, h->num_sms);
+        if (h->N >= hy::k::kScreenMinN)
+            s = build_screen_plan(p->screen, &p, &zero, &zero, 1, h->num_sms);
     }
     if (s != HY_OK) {
         std::string msg = g_err;
@@ -1688,7 +1690,7 @@ hy_status grad_noalloc_t(hy_ham *h, const hy_pool *p, const T *psi, const T *sig
     // the whole pool in double: the plan's partial sums fit the array at every
     // size the library takes (at most ~220 k at 16 orbitals)
     if constexpr (sizeof(T) == sizeof(double))
-        if (!ops && p->screen.n_partials <= kNoAllocPartials)
+        if (!ops && h->N >= hy::k::kScreenMinN && p->screen.n_partials <= kNoAllocPartials)
             return screen_run(p->screen, psi, sigma, scratch, g, st);
     hy::k::GradArgs<T> a;
     a.psi = psi;

@@ -597,7 +597,11 @@ cudaError_t fold_compact(const FoldArgs &a, int32_t *ptr, int32_t *col, double *
 
 // Screen of whole pools in double, one or many molecules (hy_screen.cu).
 // Kinds of tasks: 0 alpha-beta (and every single), 1 alpha doubles, 2 beta
-// doubles.
+// doubles.  One molecule alone takes it from kScreenMinN determinants: a task's
+// staged groups follow one another, so below that the per-operator kernel's
+// single short pass is quicker (400 determinants 12 against 19 us, 4,900 26
+// against 29, 15,876 a tie at 50, 63,504 138 against 71).
+constexpr int64_t kScreenMinN = 16384;
 struct ScreenMol {
     const OpDev *opd;
     const ConsDev *cons;

@@ -61,3 +61,24 @@ def test_packed_molecules_match_their_own_screens():
         if len(every):
             ref = pools[m].gradients(x, y, ops=every)
             assert torch.max(torch.abs(g[lo:hi] - ref)).item() <= 1e-12
+
+
+@pytest.mark.parametrize("kind", ["sd", "qeb"])
+@pytest.mark.parametrize("cfg", CFGS[:9], ids=[f"n{n}a{a}b{b}" for n, a, b in CFGS[:9]])
+def test_small_molecule_in_a_batch(cfg, kind):
+    """Below 16,384 determinants a molecule alone is screened per operator; in a
+    batch it takes the screen by pattern."""
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2604_01176_gb300 as hy
+    n, na, nb = cfg
+    ham = hy.Hamiltonian(*synth.integrals(n, 50 + n), n, na, nb)
+    pool = hy.Pool(ham, kind)
+    batch = hy.Batch([ham])
+    batch.set_pools([pool])
+    psi = torch.from_numpy(synth.random_state(ham.n_det, 3)).cuda()
+    sigma = torch.from_numpy(synth.random_state(ham.n_det, 4)).cuda()
+    whole = batch.gradients(batch.pack([psi]), batch.pack([sigma]))
+    every = torch.arange(len(pool), dtype=torch.int32, device="cuda")
+    listed = pool.gradients(psi, sigma, ops=every)
+    assert torch.max(torch.abs(whole - listed)).item() <= 1e-12
