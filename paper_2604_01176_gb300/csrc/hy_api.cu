@@ -186,7 +186,8 @@ struct hy_pool {
     std::vector<int32_t> sing[2], dbl[2];
     int32_t *d_sing[2] = {nullptr, nullptr}, *d_dbl[2] = {nullptr, nullptr};
     int32_t *d_slot[2] = {nullptr, nullptr};
-    ScreenPlan screen;
+    ScreenPlan screen;              // double
+    double *d_part32 = nullptr;     // float: partial sums
 };
 
 struct hy_batch {
@@ -684,6 +685,44 @@ hy_status screen_run(const ScreenPlan &sp, const double *psi, const double *sigm
     return HY_OK;
 }
 
+// pairs of a beta single pattern (the same for all of them)
+int beta_single_pairs(const hy_pool *p)
+{
+    return p->sing[1].empty() ? 0 : int(p->pb.cnt[p->sing[1][0]]);
+}
+
+// whether whole pools of this molecule alone are screened by pattern
+bool screen_by_pattern(const hy_pool *p, bool f32)
+{
+    return p->h->N >= hy::k::kScreenMinN && (!f32 || beta_single_pairs(p) <= hy::k::kScreen32MaxPairs);
+}
+
+// partial sums of the float screen of a whole pool
+int64_t screen32_partials(const hy_ham *h, const hy_pool *p)
+{
+    return (int64_t(p->sing[0].size() * p->sing[1].size()) + int64_t(p->pa.keys.size()) +
+            int64_t(p->pb.keys.size())) * grad_chunks(h, int64_t(p->ops.size()));
+}
+
+hy_status screen32_run(const hy_ham *h, const hy_pool *p, const float *psi, const float *sigma,
+                       double *partials, double *g, cudaStream_t st)
+{
+    hy::k::Screen32Args a{};
+    a.psi = psi;
+    a.sigma = sigma;
+    a.aent = p->d_aent; a.bent = p->d_bent;
+    a.aoff = p->d_aoff; a.acnt = p->d_acnt; a.boff = p->d_boff; a.bcnt = p->d_bcnt;
+    a.la = p->d_sing[0]; a.lb = p->d_sing[1];
+    a.Na = int(h->Na); a.Nb = int(h->Nb);
+    a.nA = int(p->sing[0].size()); a.nB = int(p->sing[1].size());
+    a.npA = int(p->pa.keys.size()); a.npB = int(p->pb.keys.size());
+    a.CH = grad_chunks(h, int64_t(p->ops.size()));
+    a.partials = partials;
+    HY_CUDA(hy::k::screen32(a, beta_single_pairs(p), p->d_op, p->d_cons, p->d_slot[0], p->d_slot[1],
+                            int64_t(p->ops.size()), g, st), "pool gradients");
+    return HY_OK;
+}
+
 template <typename T>
 hy_status grad_t(hy_ham *h, const hy_pool *p, const T *psi, const T *sigma,
                  const int32_t *ops, int64_t n_ops, double *g, cudaStream_t st)
@@ -698,10 +737,13 @@ hy_status grad_t(hy_ham *h, const hy_pool *p, const T *psi, const T *sigma,
                 bytes += 4.0 * nr * nc * sizeof(T);
             }
     hy::ProfScope prof(HY_PROF_SCREEN, st, bytes);
-    // whole pools in double by pattern, from kScreenMinN determinants; lists,
-    // small states and float sums per operator
-    if constexpr (sizeof(T) == sizeof(double))
-        if (!ops && h->N >= hy::k::kScreenMinN) return screen_run(p->screen, psi, sigma, p->screen.d_partials, g, st);
+    // whole pools by pattern where that is the quicker; lists per operator
+    if (!ops && screen_by_pattern(p, sizeof(T) == sizeof(float))) {
+        if constexpr (sizeof(T) == sizeof(double))
+            return screen_run(p->screen, psi, sigma, p->screen.d_partials, g, st);
+        else
+            return screen32_run(h, p, psi, sigma, p->d_part32, g, st);
+    }
     const WsLayout L = ws_layout(h, n_partials_needed(h, n_ops), sizeof(T));
     hy_status s = ensure_ws(h, L.total);
     if (s != HY_OK) return s;
@@ -1444,8 +1486,10 @@ hy_status hy_pool_create(const hy_ham *h, hy_pool_kind kind, hy_pool **out)
     }
     if (s == HY_OK) {
         const int64_t zero = 0;
-        if (h->N >= hy::k::kScreenMinN)
+        if (h->N >= hy::k::kScreenMinN) {
             s = build_screen_plan(p->screen, &p, &zero, &zero, 1, h->num_sms);
+            up(ar.alloc(&p->d_part32, size_t(screen32_partials(h, p))), "screen partials");
+        }
     }
     if (s != HY_OK) {
         std::string msg = g_err;
@@ -1687,11 +1731,16 @@ hy_status grad_noalloc_t(hy_ham *h, const hy_pool *p, const T *psi, const T *sig
                          const int32_t *ops, int64_t n_ops, double *g, double *scratch,
                          cudaStream_t st)
 {
-    // the whole pool in double: the plan's partial sums fit the array at every
-    // size the library takes (at most ~220 k at 16 orbitals)
-    if constexpr (sizeof(T) == sizeof(double))
-        if (!ops && h->N >= hy::k::kScreenMinN && p->screen.n_partials <= kNoAllocPartials)
-            return screen_run(p->screen, psi, sigma, scratch, g, st);
+    // whole pools: the partial sums fit the array at every size the library
+    // takes (at most ~220 k at 16 orbitals in double, ~6 k in float)
+    if (!ops && screen_by_pattern(p, sizeof(T) == sizeof(float))) {
+        if constexpr (sizeof(T) == sizeof(double)) {
+            if (p->screen.n_partials <= kNoAllocPartials)
+                return screen_run(p->screen, psi, sigma, scratch, g, st);
+        } else if (screen32_partials(h, p) <= kNoAllocPartials) {
+            return screen32_run(h, p, psi, sigma, scratch, g, st);
+        }
+    }
     hy::k::GradArgs<T> a;
     a.psi = psi;
     a.sigma = sigma;

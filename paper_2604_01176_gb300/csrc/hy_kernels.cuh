@@ -624,6 +624,23 @@ struct ScreenArgs {
 cudaError_t screen_all(const ScreenArgs &a, int cfg, int n_tasks, size_t smem, int count,
                        int64_t n_ops, double *g, cudaStream_t st);
 
+// Screen of a whole pool on a float state (hy_screen32.cu), CH row chunks as in
+// GradArgs.  partials: (nA nB + npA + npB) x CH doubles
+struct Screen32Args {
+    const float *psi, *sigma;
+    const uint32_t *aent, *bent;
+    const int64_t *aoff, *acnt, *boff, *bcnt;    // by pattern id
+    const int32_t *la, *lb;                      // ids of the singles of each spin
+    int Na, Nb, nA, nB, npA, npB, CH;
+    int n_pg, n_ab;                              // set by the launch
+    double *partials;
+};
+// bs_cnt: pairs of a beta single pattern, at most kScreen32MaxPairs
+constexpr int kScreen32MaxPairs = 7 * 256;
+cudaError_t screen32(Screen32Args a, int bs_cnt, const OpDev *opd, const ConsDev *cons,
+                     const int32_t *aslot, const int32_t *bslot, int64_t n_ops, double *g,
+                     cudaStream_t st);
+
 // Batched pool-gradient screen: per molecule its pool's pair tables (as in
 // GradArgs) and its place in the packed state buffers
 struct BatchPool {

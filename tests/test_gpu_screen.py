@@ -82,3 +82,32 @@ def test_small_molecule_in_a_batch(cfg, kind):
     every = torch.arange(len(pool), dtype=torch.int32, device="cuda")
     listed = pool.gradients(psi, sigma, ops=every)
     assert torch.max(torch.abs(whole - listed)).item() <= 1e-12
+
+
+@pytest.mark.parametrize("kind", ["sd", "qeb"])
+@pytest.mark.parametrize("cfg", [(10, 5, 5), (11, 6, 5), (12, 9, 4), (13, 4, 9), (13, 7, 5), (14, 7, 7),
+                                 (15, 8, 7), (16, 4, 8), (16, 8, 8)],
+                         ids=lambda c: "n%da%db%d" % c)
+def test_float_pool_keeps_the_operator_lists_sums(cfg, kind):
+    """Float: the same float sums per thread as the per-operator kernel (same
+    row chunks for a list of the whole pool), so only the double sums of 256
+    threads differ: 1e-13 of them, |g| <= 4 on normalised vectors.  Sizes: one to
+    fourteen table entries per thread and pattern, both stagings, several chunks
+    (small pools), shares of patterns that do not divide."""
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2604_01176_gb300 as hy
+    n, na, nb = cfg
+    if n == 16 and (kind == "qeb") != (na == 4):
+        pytest.skip("one pool per 16-orbital size")
+    ham = hy.Hamiltonian(*synth.integrals(n, 50 + n), n, na, nb)
+    pool = hy.Pool(ham, kind)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n + na)
+    v = torch.randn((2, ham.n_det), dtype=torch.float32, device="cuda", generator=g)
+    psi, sigma = v[0] / v[0].norm(), v[1] / v[1].norm()
+    every = torch.arange(len(pool), dtype=torch.int32, device="cuda")
+    whole = torch.full((len(pool),), np.nan, dtype=torch.float64, device="cuda")
+    pool.gradients(psi, sigma, out=whole)
+    listed = pool.gradients(psi, sigma, ops=every)
+    assert torch.max(torch.abs(whole - listed)).item() <= 1e-13
