@@ -121,8 +121,8 @@ struct hy_ham {
     float *d_pairB = nullptr;                   // [2][Na][n^2] touched-weight partials
     float *d_pairRs = nullptr;                  // [2][Na]
     float *d_pairD = nullptr;                   // [2][n^4] touched weights (psi, sigma)
-    float *d_pairP = nullptr;                   // [splits][n^4] contraction partials
-    int32_t *d_pairRows = nullptr;              // [Na + 1] nonzero alpha rows
+    float *d_pairP = nullptr;                   // [2][splits][n^4] contraction partials
+    int32_t *d_pairRows = nullptr;              // [2][Na + 1] nonzero alpha rows
     double *d_occw = nullptr;                   // [34] occupations-from-weights scratch
     int occ_blocks = 0;
     // workspace (grown on demand; growth synchronises the device)
@@ -1066,9 +1066,9 @@ hy_status finish_ham(hy_ham *h, hy_ham **out)
         up(ar.alloc(&h->d_pairB, 2 * size_t(h->Na) * nn, true), "touched-weight partials");
         up(ar.alloc(&h->d_pairRs, 2 * size_t(h->Na), true), "touched-weight partials");
         up(ar.alloc(&h->d_pairD, 2 * nn * nn, true), "touched weights");
-        up(ar.alloc(&h->d_pairP, size_t(hy::k::pair_splits()) * nn * nn, true),
+        up(ar.alloc(&h->d_pairP, 2 * size_t(hy::k::pair_splits()) * nn * nn, true),
            "touched-weight partials");
-        up(ar.alloc(&h->d_pairRows, size_t(h->Na) + 1, true), "touched-weight rows");
+        up(ar.alloc(&h->d_pairRows, 2 * (size_t(h->Na) + 1), true), "touched-weight rows");
         up(ar.alloc(&h->d_occw, size_t(34), true), "occupation scratch");
     }
     if (s == HY_OK) s = fold_same_spin(h);
@@ -1991,13 +1991,13 @@ hy_status hy_touched_weights(const hy_ham *h, const void *psi, hy_dtype dt, floa
     if (!h || !psi || !D || !valid_dtype(dt)) return fail(HY_ERR_ARG, "bad arguments");
     cudaStream_t st = as_stream(stream);
     if (dt == HY_F64)
-        HY_CUDA(hy::k::touched_weights<double>(static_cast<const double *>(psi), h->Na, h->Nb,
+        HY_CUDA(hy::k::touched_weights<double>(static_cast<const double *>(psi), nullptr, h->Na, h->Nb,
                                                h->d_astr, h->d_bstr, h->n, h->d_pairB,
                                                h->d_pairRs, h->d_pairRows, h->d_pairP, D,
                                                h->num_sms, st),
                 "touched weights");
     else
-        HY_CUDA(hy::k::touched_weights<float>(static_cast<const float *>(psi), h->Na, h->Nb,
+        HY_CUDA(hy::k::touched_weights<float>(static_cast<const float *>(psi), nullptr, h->Na, h->Nb,
                                               h->d_astr, h->d_bstr, h->n, h->d_pairB,
                                               h->d_pairRs, h->d_pairRows, h->d_pairP, D,
                                               h->num_sms, st),
@@ -3320,16 +3320,23 @@ hy_status ranker_features_impl(const hy_ham *h, const hy_pool *p, const void *ps
                             h->Na, h->Nb, h->d_astr, h->d_bstr, h->n, B, rs, h->d_pairRows,
                             h->d_pairP, D, h->tw, h->num_sms, st),
                         "touched weights (list)");
-        } else if (dt == HY_F64) {
-            HY_CUDA(hy::k::touched_weights<double>(static_cast<const double *>(vecs[v]), h->Na,
-                                                   h->Nb, h->d_astr, h->d_bstr, h->n, B, rs,
-                                                   h->d_pairRows, h->d_pairP, D, h->num_sms, st),
-                    "touched weights");
         } else {
-            HY_CUDA(hy::k::touched_weights<float>(static_cast<const float *>(vecs[v]), h->Na,
-                                                  h->Nb, h->d_astr, h->d_bstr, h->n, B, rs,
-                                                  h->d_pairRows, h->d_pairP, D, h->num_sms, st),
-                    "touched weights");
+            // psi and sigma both dense: in the same launches
+            const bool both = v == 0 && vecs[1] && !states[1];
+            const void *second = both ? vecs[1] : nullptr;
+            if (dt == HY_F64)
+                HY_CUDA(hy::k::touched_weights<double>(
+                            static_cast<const double *>(vecs[v]), static_cast<const double *>(second),
+                            h->Na, h->Nb, h->d_astr, h->d_bstr, h->n, B, rs, h->d_pairRows,
+                            h->d_pairP, D, h->num_sms, st),
+                        "touched weights");
+            else
+                HY_CUDA(hy::k::touched_weights<float>(
+                            static_cast<const float *>(vecs[v]), static_cast<const float *>(second),
+                            h->Na, h->Nb, h->d_astr, h->d_bstr, h->n, B, rs, h->d_pairRows,
+                            h->d_pairP, D, h->num_sms, st),
+                        "touched weights");
+            if (both) break;
         }
     }
     // occupations from psi's touched-weight partials: no further pass over psi

@@ -230,10 +230,11 @@ cudaError_t occupations_from_weights(const float *Bw, const float *rs, const uin
 cudaError_t features(const int32_t *desc, int64_t K, int n, const double *h1,
                      const double *eri, const float *occ, const float *extra, const float *Dpsi,
                      const float *Dsig, float *feat, cudaStream_t st);
-// part: pair_splits() x n^4 floats of scratch; rows: Na + 1 ints of scratch
+// scratch per vector: part pair_splits() x n^4 floats, rows Na + 1 ints; psi1
+// (or null): a second vector, its Bw, rs, rows, part and D behind the first's
 int pair_splits();
 template <typename T>
-cudaError_t touched_weights(const T *psi, int64_t Na, int64_t Nb, const uint32_t *astr,
+cudaError_t touched_weights(const T *psi, const T *psi1, int64_t Na, int64_t Nb, const uint32_t *astr,
                             const uint32_t *bstr, int n, float *Bw, float *rs, int32_t *rows,
                             float *part, float *D, int num_sms, cudaStream_t st);
 // scratch that groups a listed state's entries by alpha row: counts and

@@ -1,0 +1,63 @@
+"""The ranker's forward pass at widths and row counts around its tile edges
+(8 rows, 32 inputs, 256 units, 512 the widest single-launch width) against the
+same network in 64 bits, and touched weights of one vector and of two in the
+same launches against brute force.
+
+Tolerance: a score sums at most 600 float products per layer over four layers
+(the rounding of 600 terms, 600 x 2^-24 = 4e-5 of their absolute sum, typically
+a twentieth of it): 1e-4 of the largest score.
+"""
+import numpy as np
+import pytest
+
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("hidden", [16, 40, 255, 256, 300, 512, 600])
+@pytest.mark.parametrize("rows", [1, 7, 8, 65, 1107])
+def test_forward_shapes(hidden, rows):
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2604_01176_gb300 as hy
+    r = hy.Ranker(hidden=hidden, seed=3)
+    w = r.params().astype(np.float64)
+    x = np.random.default_rng(rows).standard_normal((rows, 16)).astype(np.float32)
+    got = r.predict(torch.from_numpy(x).cuda()).cpu().numpy()
+    z, fin, o = x.astype(np.float64), 16, 0
+    for out in (hidden, hidden, hidden, 1):
+        W = w[o:o + out * fin].reshape(out, fin)
+        o += out * fin
+        b = w[o:o + out]
+        o += out
+        z = z @ W.T + b
+        if out != 1:
+            z = np.maximum(z, 0.0)
+        fin = out
+    assert o == len(w)
+    assert np.abs(got - z[:, 0]).max() <= 1e-4 * max(np.abs(z).max(), 1e-3)
+
+
+@pytest.mark.parametrize("cfg", [(3, 1, 2), (6, 3, 3), (9, 5, 4), (12, 6, 6)])
+def test_two_vectors_share_launches(cfg):
+    """Features of (psi, sigma) use both vectors' weights from shared launches:
+    the same as the features of psi with sigma's weights from its own call."""
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2604_01176_gb300 as hy
+    n, na, nb = cfg
+    ham = hy.Hamiltonian(*synth.integrals(n, 5), n, na, nb)
+    pool = hy.Pool(ham)
+    psi = torch.from_numpy(synth.random_state(ham.n_det, 1)).cuda()
+    sigma = torch.from_numpy(synth.random_state(ham.n_det, 2)).cuda()
+    both = hy.ranker_features(ham, pool, psi, sigma=sigma)
+    again = hy.ranker_features(ham, pool, psi, sigma=sigma)
+    assert torch.equal(both, again)
+    swapped = hy.ranker_features(ham, pool, sigma, sigma=psi)
+    alone = hy.ranker_features(ham, pool, psi)
+    assert torch.isfinite(both).all() and torch.isfinite(swapped).all() and torch.isfinite(alone).all()
+    d1, d2 = hy.touched_weights(ham, psi), hy.touched_weights(ham, sigma)
+    w1, w2 = d1[0, 0].item(), d2[0, 0].item()
+    assert abs(w1 - 1.0) <= 1e-5 and abs(w2 - 1.0) <= 1e-5
