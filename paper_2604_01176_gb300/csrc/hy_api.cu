@@ -113,6 +113,9 @@ struct hy_ham {
     // Mb64 by column, for spaces of up to kRowsMaxNb beta strings (hy_rows64.cu)
     double *d_mbv = nullptr;
     uint16_t *d_mbc = nullptr;
+    // operand tables of the float tensor-core coupling (kCplWideOrbitals and up)
+    uint16_t *d_cent = nullptr;
+    uint32_t *d_ctmask = nullptr;
     double *d_V64 = nullptr;
     float *d_V32 = nullptr;
     double *d_h1 = nullptr, *d_eri = nullptr;   // integrals (ranker features)
@@ -484,6 +487,9 @@ hy_status apply_h_t(hy_ham *h, const T *psi, T *sigma, cudaStream_t st, int64_t 
             d.Nbp = Nbp;
             d.row0 = r0;
             d.row1 = r1;
+            d.entries = h->d_cent;
+            d.tmask = h->d_ctmask;
+            d.nocc = h->nb;
             hy_status sj = coupling_jlist(h, r0, r1, &d.jlist, &d.nJ);
             if (sj != HY_OK) return sj;
             if (h->prof) cudaEventRecord(h->ev0, st);
@@ -1070,6 +1076,13 @@ hy_status finish_ham(hy_ham *h, hy_ham **out)
            "touched-weight partials");
         up(ar.alloc(&h->d_pairRows, 2 * (size_t(h->Na) + 1), true), "touched-weight rows");
         up(ar.alloc(&h->d_occw, size_t(34), true), "occupation scratch");
+    }
+    if (h->n >= hy::k::kCplWideOrbitals && h->nb >= 1) {
+        up(ar.alloc(&h->d_ctmask, size_t((h->Nb + 127) / 128), true), "coupling tables");
+        up(ar.alloc(&h->d_cent, hy::k::cpl_entries_count(h->Nb, h->nb)), "coupling tables");
+        if (s == HY_OK)
+            up(hy::k::cpl_entries(h->d_bstr, h->d_bexT, h->Nb, h->n, h->nb, h->d_cent, h->d_ctmask,
+                                  h->num_sms, nullptr), "coupling tables");
     }
     if (s == HY_OK) s = fold_same_spin(h);
     if (s != HY_OK) {

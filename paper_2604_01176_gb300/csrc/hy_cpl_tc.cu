@@ -30,6 +30,8 @@
 // tensor memory and returns.
 #include "hy_kernels.cuh"
 
+#include <algorithm>
+
 namespace hy {
 namespace k {
 
@@ -366,11 +368,461 @@ k_cpl_tc(CplDenseArgs a, int *status, long long spin_limit, int issue)
                      ::"r"(tmem), "r"(kTmemCols));
 }
 
+// ---------------------------------------------------------------------------
+// The same contraction for wider beta spaces (k_cpl_tcw): W_J stays in shared
+// memory for all column tiles of J, already split (n x 8 KB), an operand stage
+// is the 16 types of one r, and the roles run apart, joined by mbarriers only:
+//   * two groups of eight warps build alternate stages.  A thread owns a column
+//     and eight s; its eight partners' indices and signs are one 16-byte load
+//     from a table made when the Hamiltonian is (cpl_entries: 16 bits each,
+//     absent pairs point at a zero behind psi's row), so a stage is eight
+//     gathers, splits and four 16-byte stores;
+//   * one warp issues the MMAs of a stage (six) and commits it;
+//   * four warps read finished accumulators (two in tensor memory, used in turn)
+//     while the next tile is multiplied.
+// r that no column of a tile holds is skipped.  k_cpl_tc's block-wide barrier
+// per chunk left it at 3,600 clocks per 32 types, 768 of them tensor time.
+// Bound by the hand-over of stages (build, fence, arrive, issue, commit): with
+// gathers, stores or MMAs left out one at a time it loses 0-13 %, with all of them
+// half.  Stages of 8 types (twice the hand-overs) cost 30 %, four groups of four
+// warps, a column's 16 types to a thread, 6-20 %.  Measured, whole float H|psi>:
+// 16 orbitals, 8+8 (66 of 129 ms left of the coupling's) 205 -> 143 ms; 13
+// orbitals, 7+6: 2,989 -> 1,713 us; 11 orbitals, 6+5: 285 -> 183 us; also with few
+// strings: 12 orbitals, 2+2: 62.6 -> 55.9 us.
+// ---------------------------------------------------------------------------
+namespace {
+
+constexpr int kTwBuilders = 512, kTwThreads = kTwBuilders + 128 + 32;
+constexpr int kTwIssueWarp = 20;
+constexpr uint32_t kTwSbo = 512;                        // 16 types of 8 rows
+constexpr size_t kTwA = size_t(kTcM) * 16 * 4;          // one r of W_J, hi or lo: 4 KB
+constexpr size_t kTwB = size_t(kTcN) * 16 * 4;          // one r of a tile, hi or lo: 8 KB
+constexpr int kTwMaxStages = 4;
+
+// small block of barriers and flags at the front of shared memory
+struct TwCtl {
+    uint64_t full[kTwMaxStages], empty[kTwMaxStages], acc_full[2], acc_empty[2], fin;
+    uint32_t tmem;
+    int dead;                                           // a wait ran out somewhere
+};
+
+__device__ __forceinline__ void arrive(uint64_t *bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(bar)) : "memory");
+}
+
+// whether the phase with parity `par` has completed: a plain test, as
+// try_wait's suspended thread wakes late
+__device__ __forceinline__ bool test_bar(uint64_t *bar, uint32_t par)
+{
+    uint32_t done;
+    asm volatile("{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+                 "selp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(done) : "r"(saddr(bar)), "r"(par) : "memory");
+    return done != 0;
+}
+
+// bounded wait that also ends when another role has given up
+__device__ __forceinline__ bool tw_wait(TwCtl *c, uint64_t *bar, uint32_t par, long long limit,
+                                        int *status)
+{
+    for (long long it = 0; it < limit; ++it) {
+        if (test_bar(bar, par)) return true;
+        if (*reinterpret_cast<volatile int *>(&c->dead)) return false;
+    }
+    *reinterpret_cast<volatile int *>(&c->dead) = 1;
+    atomicExch(status, 1);
+    return false;
+}
+
+// the same for a whole warp: one lane polls (32 lanes of 20 warps polling slow
+// the barrier unit down for everyone)
+__device__ __forceinline__ bool tw_wait_warp(TwCtl *c, uint64_t *bar, uint32_t par, long long limit,
+                                             int *status)
+{
+    int ok = 1;
+    if ((threadIdx.x & 31) == 0) ok = tw_wait(c, bar, par, limit, status);
+    return __shfl_sync(0xffffffffu, ok, 0) != 0;
+}
+
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(p));
+    return p != 0;
+}
+
+// barrier of the builders (all of them, always); whether v holds in every one
+__device__ __forceinline__ bool builders_and(bool v)
+{
+    int r;
+    __syncwarp();
+    asm volatile("{\n.reg .pred p, q;\nsetp.ne.s32 p, %1, 0;\n"
+                 "bar.red.and.pred q, 1, %2, p;\nselp.s32 %0, 1, 0, q;\n}"
+                 : "=r"(r) : "r"(int(v)), "n"(kTwBuilders) : "memory");
+    return r != 0;
+}
+
+}  // namespace
+
+size_t cpl_tcw_smem(int64_t Nb, int n, int stages)
+{
+    // control | W_J hi, lo | stages | Wd | diagonal partials [2][4][128] | psi row and a zero
+    return 256 + size_t(n) * 2 * kTwA + stages * 2 * kTwB + 256 * 4 + 2 * 4 * kTcN * 4 +
+           size_t((Nb + 1 + 3) / 4 * 16);
+}
+
+__global__ void __launch_bounds__(kTwThreads, 1)
+k_cpl_tcw(CplDenseArgs a, int nst, int *status, long long spin_limit, int issue)
+{
+    extern __shared__ __align__(1024) unsigned char sm[];
+    TwCtl *ctl = reinterpret_cast<TwCtl *>(sm);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int n = a.n, nn = n * n, nexa = a.nexa, slots = nexa + 1;
+    const int Nb = int(a.Nb), tiles = (Nb + kTcN - 1) / kTcN;
+    unsigned char *Wa = sm + 256;                           // [n][hi, lo][64 x 16]
+    unsigned char *stg = Wa + size_t(n) * 2 * kTwA;         // [nst][hi, lo][128 x 16]
+    float *Wd = reinterpret_cast<float *>(stg + size_t(nst) * 2 * kTwB);  // [16][16]
+    float *dpart = Wd + 256;                                // [2][4][128]
+    float *prow = dpart + 2 * 4 * kTcN;                     // [Nb + 1]
+
+    if (tid == 0) {
+        auto init = [](uint64_t *b, int cnt) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(saddr(b)), "r"(cnt));
+        };
+        for (int i = 0; i < nst; ++i) {
+            init(&ctl->full[i], 8);
+            init(&ctl->empty[i], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            init(&ctl->acc_full[i], 1);
+            init(&ctl->acc_empty[i], 4);
+        }
+        init(&ctl->fin, 1);
+        ctl->dead = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(saddr(&ctl->tmem)), "r"(2 * kTmemCols));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = ctl->tmem;
+
+    if (tid < kTwBuilders) {
+        // ---- builders ----------------------------------------------------
+        // two groups of eight warps take the r in turn; r number i goes to stage
+        // i % nst, a thread fills half of a column's types
+        const int par = warp >> 3, half = (warp >> 2) & 1, col = tid & (kTcN - 1);
+        const uint32_t none = uint32_t(Nb) | (uint32_t(Nb) << 16);
+        const uint32_t off = kmaj(col, half * 8, kTwSbo);
+        uint32_t it = 0;            // r of all tiles so far
+        int slot = par, use = 0;    // where this group's next r goes, how often used
+        uint32_t tile_no = 0;
+        bool ok = true;
+        // this group's r of a tile whose first r has number i: every second set bit
+        auto own = [&](uint32_t tm, uint32_t i) {
+            return ((i ^ uint32_t(par)) & 1u) ? tm & (tm - 1) : tm;
+        };
+        auto load = [&](int tile, uint32_t m, int r) {
+            return ((m >> r) & 1u)
+                ? __ldg(reinterpret_cast<const uint4 *>(a.entries) +
+                        ((size_t(tile) * a.nocc + __popc(m & ((1u << r) - 1u))) * kTcN + col) * 2 + half)
+                : make_uint4(none, none, none, none);
+        };
+        auto mask = [&](int tile) {
+            const int b = tile * kTcN + col;
+            return b < Nb ? __ldg(a.bstr + b) : 0u;
+        };
+        // tables run ahead across tiles and J: e the entry of the next own stage,
+        // bm the column's string in this tile, bn in the next
+        uint32_t bm = mask(0), bn = mask(tiles > 1 ? 1 : 0), tm = __ldg(a.tmask);
+        uint4 e = make_uint4(none, none, none, none);
+        if (own(tm, 0)) e = load(0, bm, __ffs(own(tm, 0)) - 1);
+        for (int64_t jj = blockIdx.x; jj < a.nJ; jj += gridDim.x) {
+            const int64_t J = a.jlist ? int64_t(a.jlist[jj]) : jj;
+            // the previous J: its row is read by all builders, its W_J by the MMAs
+            // (the last of them done, all are).  A builder whose wait ran out comes
+            // here too: the block's builders stop together
+            if (it && ok) {
+                const uint32_t last = it - 1;
+                ok = tw_wait_warp(ctl, &ctl->empty[last % nst], (last / nst) & 1u, spin_limit, status);
+            }
+            ok = builders_and(ok);
+            if (!ok) break;
+            const float *src = a.psi + J * Nb;
+            for (int i = tid; i < Nb; i += kTwBuilders) prow[i] = __ldg(src + i);
+            if (tid == 0) prow[Nb] = 0.0f;
+            const uint32_t jm = a.astr[J];
+            for (int i = tid; i < n * kTcM * 4; i += kTwBuilders) {
+                const int m = i & 63, k4 = (i >> 6) & 3, r = i >> 8;
+                float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                if (m < nexa) {
+                    const uint32_t u = a.aex[J * nexa + m];
+                    const int pj = (u >> 16) & 15, qj = (u >> 20) & 15;
+                    const float *V = a.V + size_t(qj * n + pj) * nn + r * n;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (4 * k4 + q < n) v[q] = (u >> 31) ? -__ldg(V + 4 * k4 + q) : __ldg(V + 4 * k4 + q);
+                }
+                float4 h, l;
+                split(v[0], h.x, l.x);
+                split(v[1], h.y, l.y);
+                split(v[2], h.z, l.z);
+                split(v[3], h.w, l.w);
+                unsigned char *dst = Wa + size_t(r) * 2 * kTwA + kmaj(m, 4 * k4, kTwSbo);
+                *reinterpret_cast<float4 *>(dst) = h;
+                *reinterpret_cast<float4 *>(dst + kTwA) = l;
+            }
+            for (int i = tid; i < 256; i += kTwBuilders) {
+                const int r = i >> 4, s = i & 15;
+                float v = 0.0f;
+                if (r < n && s < n)
+                    for (uint32_t mm = jm; mm; mm &= mm - 1) {
+                        const int p = __ffs(mm) - 1;
+                        v += a.V[size_t(p * n + p) * nn + r * n + s];
+                    }
+                Wd[i] = v;
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            builders_and(true);
+            for (int tile = 0; tile < tiles && ok; ++tile, ++tile_no) {
+                const int next = tile + 1 < tiles ? tile + 1 : 0;
+                const uint32_t tn = __ldg(a.tmask + next), stages = __popc(tm);
+                const uint32_t bnn = mask(next + 1 < tiles ? next + 1 : 0);
+                uint32_t left = own(tm, it);
+                float dsum = 0.0f;
+                while (left && ok) {
+                    const int r = __ffs(left) - 1;
+                    left &= left - 1;
+                    if (left) left &= left - 1;
+                    // the next own stage's entries, here or in the next tile
+                    uint4 nx = e;
+                    if (left) {
+                        nx = load(tile, bm, __ffs(left) - 1);
+                    } else {
+                        const uint32_t on = own(tn, it + stages);
+                        if (on) nx = load(next, bn, __ffs(on) - 1);
+                    }
+                    const uint32_t w[4] = {e.x, e.y, e.z, e.w};
+                    float h[8], l[8];
+                    const float4 c0 = *reinterpret_cast<const float4 *>(Wd + r * 16 + half * 8);
+                    const float4 c1 = *reinterpret_cast<const float4 *>(Wd + r * 16 + half * 8 + 4);
+                    const float c[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        const uint32_t x = q & 1 ? w[q >> 1] >> 16 : w[q >> 1] & 0xFFFFu;
+                        const float v = __uint_as_float(__float_as_uint(prow[x & 0x7FFFu]) ^
+                                                        ((x & 0x8000u) << 16));
+                        dsum = fmaf(c[q], v, dsum);
+                        split(v, h[q], l[q]);
+                    }
+                    // the MMAs that read this stage last
+                    if (use)
+                        ok = tw_wait_warp(ctl, &ctl->empty[slot], (use - 1) & 1u, spin_limit, status);
+                    if (!ok) break;
+                    unsigned char *Bh = stg + size_t(slot) * 2 * kTwB, *Bl = Bh + kTwB;
+                    *reinterpret_cast<float4 *>(Bh + off) = make_float4(h[0], h[1], h[2], h[3]);
+                    *reinterpret_cast<float4 *>(Bh + off + 128) = make_float4(h[4], h[5], h[6], h[7]);
+                    *reinterpret_cast<float4 *>(Bl + off) = make_float4(l[0], l[1], l[2], l[3]);
+                    *reinterpret_cast<float4 *>(Bl + off + 128) = make_float4(l[4], l[5], l[6], l[7]);
+                    if (!left) {
+                        // the tile's last stage of this group: its part of the
+                        // diagonal slot, once that tile's place has been read
+                        const uint32_t buf = tile_no & 1u, used = tile_no >> 1;
+                        if (used)
+                            ok = tw_wait_warp(ctl, &ctl->acc_empty[buf], (used - 1) & 1u, spin_limit,
+                                      status);
+                        if (!ok) break;
+                        dpart[(buf * 4 + par * 2 + half) * kTcN + col] = dsum;
+                    }
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) arrive(&ctl->full[slot]);
+                    for (slot += 2; slot >= nst; slot -= nst) ++use;
+                    e = nx;
+                }
+                // a tile without a stage of this group leaves e for the one after it
+                if (!own(tm, it)) {
+                    const uint32_t on = own(tn, it + stages);
+                    if (on) e = load(next, bn, __ffs(on) - 1);
+                }
+                it += stages;
+                bm = bn;
+                bn = bnn;
+                tm = tn;
+            }
+        }
+    } else if (warp == kTwIssueWarp) {
+        // ---- MMA issue -----------------------------------------------------
+        // the whole warp walks the stages (uniform registers hold the operand
+        // descriptors), one elected lane issues
+        uint32_t tile_no = 0;
+        int slot = 0, use = 0;
+        bool ok = true;
+        const uint32_t wa = saddr(Wa), sa = saddr(stg);
+        for (int64_t jj = blockIdx.x; jj < a.nJ && ok; jj += gridDim.x)
+            for (int tile = 0; tile < tiles && ok; ++tile, ++tile_no) {
+                const uint32_t buf = tile_no & 1u, used = tile_no >> 1;
+                if (used) ok = tw_wait(ctl, &ctl->acc_empty[buf], (used - 1) & 1u, spin_limit, status);
+                const uint32_t d = tmem + buf * kTmemCols;
+                uint32_t acc = 0;
+                for (uint32_t left = __ldg(a.tmask + tile); left && ok; left &= left - 1) {
+                    ok = tw_wait(ctl, &ctl->full[slot], use & 1u, spin_limit, status);
+                    if (ok && issue) {
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        const uint32_t ah = wa + uint32_t(__ffs(left) - 1) * uint32_t(2 * kTwA);
+                        const uint32_t bh = sa + uint32_t(slot) * uint32_t(2 * kTwB);
+                        if (elect_one()) {
+#pragma unroll
+                            for (int ks = 0; ks < 2; ++ks) {
+                                const uint64_t da = sdesc(ah + ks * 256u, kTwSbo);
+                                const uint64_t db = sdesc(bh + ks * 256u, kTwSbo);
+                                mma(d, da, db, acc);
+                                mma(d, da, db + (kTwB >> 4), 1u);
+                                mma(d, da + (kTwA >> 4), db, 1u);
+                                acc = 1u;
+                            }
+                            commit(&ctl->empty[slot]);
+                        }
+                        acc = 1u;
+                        __syncwarp();
+                    }
+                    if (++slot == nst) {
+                        slot = 0;
+                        ++use;
+                    }
+                }
+                if (ok && issue && elect_one()) commit(&ctl->acc_full[buf]);
+                __syncwarp();
+            }
+        // every MMA issued is done before the tensor memory goes back
+        if (issue) {
+            if (elect_one()) commit(&ctl->fin);
+            __syncwarp();
+            wait_bar(&ctl->fin, 0, spin_limit);
+        }
+        __syncwarp();
+    } else {
+        // ---- epilogue --------------------------------------------------------
+        const int ew = warp - kTwBuilders / 32;        // sub-partition: warp % 4
+        uint32_t it = 0, tile_no = 0;
+        bool ok = true;
+        for (int64_t jj = blockIdx.x; jj < a.nJ && ok; jj += gridDim.x) {
+            const int64_t J = a.jlist ? int64_t(a.jlist[jj]) : jj;
+            for (int tile = 0; tile < tiles && ok; ++tile, ++tile_no) {
+                const uint32_t buf = tile_no & 1u, stages = __popc(__ldg(a.tmask + tile));
+                const uint32_t g1 = (it & 1u) * 2;      // parts of the first stage's group
+                it += stages;
+                ok = tw_wait_warp(ctl, &ctl->acc_full[buf], (tile_no >> 1) & 1u, spin_limit, status);
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const int b0 = tile * kTcN, m = ew * 16 + lane;
+                const uint32_t rowaddr = tmem + buf * kTmemCols + (uint32_t(ew * 32) << 16);
+                float *dst = a.T + (J * slots + m) * a.Nbp + b0;
+#pragma unroll
+                for (int cb = 0; cb < kTcN / 32; ++cb) {
+                    float v[32];
+                    tmem_ld32(rowaddr + uint32_t(cb * 32), v);
+                    if (lane < 16 && m < nexa) {
+#pragma unroll
+                        for (int i = 0; i < 32; i += 4)
+                            if (b0 + cb * 32 + i < int(a.Nbp))      // Nbp: Nb rounded up to 64
+                                *reinterpret_cast<float4 *>(dst + cb * 32 + i) =
+                                    make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+                    }
+                }
+                // the diagonal slot: 32 columns a warp; a group without a stage in
+                // this tile (one r only) has left nothing
+                const int c = ew * 32 + lane;
+                if (b0 + c < Nb) {
+                    const float *d = dpart + buf * 4 * kTcN + c;
+                    const float s = stages >= 2 ? (d[0] + d[kTcN]) + (d[2 * kTcN] + d[3 * kTcN])
+                                                : d[g1 * kTcN] + d[(g1 + 1) * kTcN];
+                    a.T[(J * slots + nexa) * a.Nbp + b0 + c] = s;
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) arrive(&ctl->acc_empty[buf]);
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;"
+                     ::"r"(tmem), "r"(2 * kTmemCols));
+}
+
+// entries and the r each tile holds (k_cpl_tcw), from the packed beta
+// excitations: entry (tile, i, column, s) belongs to the i-th occupied orbital r
+// of the column's string: its partner with r -> s (s empty), itself (s = r), or
+// the zero behind psi's row; bit 15: sign
+__global__ void __launch_bounds__(256)
+k_cpl_entries(const uint32_t *__restrict__ bstr, const uint32_t *__restrict__ bexT, int Nb, int n,
+              int nocc, int tiles, uint16_t *__restrict__ entries, uint32_t *__restrict__ tmask)
+{
+    const int64_t total = int64_t(tiles) * nocc * kTcN * 16;
+    for (int64_t id = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; id < total;
+         id += int64_t(gridDim.x) * blockDim.x) {
+        const int s = int(id & 15), col = int(id >> 4) & (kTcN - 1);
+        const int ti = int(id / (16 * kTcN)), i = ti % nocc, tile = ti / nocc, b = tile * kTcN + col;
+        uint32_t e = uint32_t(Nb);
+        if (b < Nb) {
+            const uint32_t m = bstr[b];
+            uint32_t mm = m;
+            for (int k = 0; k < i; ++k) mm &= mm - 1;
+            const int r = __ffs(mm) - 1;
+            if (s == r) {
+                e = uint32_t(b);
+            } else if (s < n && !((m >> s) & 1u)) {
+                const int f = i * (n - nocc) + s - __popc(m & ((1u << s) - 1u));
+                const uint32_t u = bexT[size_t(f) * Nb + b];
+                e = (u & 0x7FFFu) | ((u >> 31) << 15);
+            }
+            if (s == 0 && i == 0) atomicOr(tmask + tile, m);
+        }
+        entries[id] = uint16_t(e);
+    }
+}
+
+size_t cpl_entries_count(int64_t Nb, int nocc)
+{
+    return size_t((Nb + kTcN - 1) / kTcN) * nocc * kTcN * 16;
+}
+
+// tmask: (Nb + 127) / 128 words, zeroed
+cudaError_t cpl_entries(const uint32_t *bstr, const uint32_t *bexT, int64_t Nb, int n, int nocc,
+                        uint16_t *entries, uint32_t *tmask, int num_sms, cudaStream_t st)
+{
+    const int tiles = int((Nb + kTcN - 1) / kTcN);
+    k_cpl_entries<<<unsigned(8 * num_sms), 256, 0, st>>>(bstr, bexT, int(Nb), n, nocc, tiles, entries,
+                                                        tmask);
+    hy::count_launch();
+    return cudaGetLastError();
+}
+
 cudaError_t coupling_tc(const CplDenseArgs &a, int *status, long long spin_limit, int issue,
                         int num_sms, cudaStream_t st)
 {
     if (a.Na == 0 || a.Nb == 0) return cudaSuccess;
     if (a.nexa > kTcM || a.n > 16) return cudaErrorInvalidValue;
+    if (a.entries) {
+        int nst = kTwMaxStages;
+        while (nst > 2 && cpl_tcw_smem(a.Nb, a.n, nst) > 227 * 1024) --nst;
+        const size_t smem = cpl_tcw_smem(a.Nb, a.n, nst);
+        const cudaError_t e = cudaFuncSetAttribute(
+            k_cpl_tcw, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+        if (e != cudaSuccess) return e;
+        if (a.nJ == 0) return cudaSuccess;
+        k_cpl_tcw<<<unsigned(std::min<int64_t>(num_sms, a.nJ)), kTwThreads, smem, st>>>(
+            a, nst, status, spin_limit, issue);
+        hy::count_launch();
+        return cudaGetLastError();
+    }
     const size_t smem = cpl_tc_smem(a.Nb);
     cudaError_t err = cudaFuncSetAttribute(k_cpl_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            int(smem));

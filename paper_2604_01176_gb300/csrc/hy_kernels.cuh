@@ -84,6 +84,11 @@ struct CplDenseArgs {
     const int32_t *jlist;
     int64_t nJ;
     int64_t row0, row1;     // phase B: output alpha rows; sigma holds row row0 first
+    // the tensor-core kernel of wider spaces (or entries = nullptr): partner
+    // tables by column tile and the orbitals each tile holds (cpl_entries)
+    const uint16_t *entries;
+    const uint32_t *tmask;
+    int nocc;               // beta electrons
 };
 size_t cpl_dense_smem(int64_t Nb, int n);
 // phase A (SIMT) + phase B
@@ -93,6 +98,15 @@ cudaError_t coupling_gather(const CplDenseArgs &a, int num_sms, cudaStream_t st)
 // phase A on the tensor cores (hy_cpl_tc.cu); *status (device) is set to 1
 // if a bounded wait ran out
 size_t cpl_tc_smem(int64_t Nb);
+// Orbitals from which phase A is k_cpl_tcw.  It is the faster one below as well
+// (8 orbitals 58 -> 49 us, 10 orbitals 109 -> 86 us, whole float H|psi>), but adds
+// the diagonal slot in another order; up to 10 orbitals the float energies of
+// dense ansatz states are kept to the last bit, so k_cpl_tc stays for them.
+constexpr int kCplWideOrbitals = 11;
+// tables of k_cpl_tcw for the nocc-electron beta strings (hy_cpl_tc.cu)
+size_t cpl_entries_count(int64_t Nb, int nocc);
+cudaError_t cpl_entries(const uint32_t *bstr, const uint32_t *bexT, int64_t Nb, int n, int nocc,
+                        uint16_t *entries, uint32_t *tmask, int num_sms, cudaStream_t st);
 cudaError_t coupling_tc(const CplDenseArgs &a, int *status, long long spin_limit, int issue,
                         int num_sms, cudaStream_t st);
 
