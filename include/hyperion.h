@@ -25,8 +25,9 @@
  *     of N_det = N_alpha * N_beta amplitudes in that order.
  *   - Precision: HY_F64 computes in double; HY_F32 keeps amplitudes and the
  *     bulk arithmetic in float with float accumulation (the float coupling
- *     of H psi runs on the tensor cores as TF32 products of split operands,
- *     FP32 accuracy; hy_ham_set_coupling).  Energies, norms, dot products
+ *     of H psi, and from 512 strings of each spin its same-spin parts, run on
+ *     the tensor cores as TF32 products of split operands, FP32 accuracy;
+ *     hy_ham_set_coupling).  Energies, norms, dot products
  *     and gradients are always returned in double and reduced with FP64
  *     accuracy (see hy_dot).
  *   - Ownership: the caller owns every state vector and output buffer passed
@@ -187,8 +188,11 @@ hy_status hy_ham_profile(hy_ham *h, int enable);
 /* Float H|psi>: phase A of the alpha-beta coupling (the dense per-string
  * product T_J = W_J G_J) on the tensor cores (impl = 0, the default:
  * tcgen05 TF32 MMAs with split hi/lo operands, FP32 accuracy) or on the FP32
- * SIMT pipes (impl = 1).  Both feed the same phase B.  A bounded wait of the
- * tensor-core kernel that runs out is returned as HY_ERR_TIMEOUT by the next
+ * SIMT pipes (impl = 1).  Both feed the same phase B.  The same-spin parts
+ * follow the choice where both spins have 512 strings or more and one is not
+ * built without the memory for its operands (1 GB a spin for 12,870 strings);
+ * else they run on the FP32 pipes.  A bounded wait of a tensor-core kernel
+ * that runs out is returned as HY_ERR_TIMEOUT by the next
  * hy_apply_h on this handle (the kernel itself gives up, releases its tensor
  * memory and returns; the context stays usable).  impl = 2 is a test of that
  * path: the tensor-core kernel runs with its MMAs withheld, so no stage
@@ -197,7 +201,7 @@ hy_status hy_ham_profile(hy_ham *h, int enable);
 hy_status hy_ham_set_coupling(hy_ham *h, int impl);
 hy_status hy_ham_coupling_ms(const hy_ham *h, float *ms);
 
-/* Polls of an mbarrier before a wait of the tensor-core coupling gives up
+/* Polls of an mbarrier before a wait of a tensor-core kernel gives up
  * (default 2^26, seconds of waiting; >= 1). */
 hy_status hy_ham_set_wait_limit(hy_ham *h, int64_t polls);
 
@@ -293,8 +297,9 @@ hy_status hy_apply_h(const hy_ham *h, const void *psi, void *sigma,
  * blocks (or an all-reduce of the scalars formed from them) completes the
  * operation.  Every element is computed by the same arithmetic in the same
  * order as in hy_apply_h, so blocks of any split concatenate to hy_apply_h's
- * sigma bit for bit.  The same-spin parts and the FP64 coupling cost the
- * range's share of the full sweep; the float tensor-core coupling forms its
+ * sigma bit for bit.  The same-spin parts (on the tensor cores in blocks of
+ * 256 rows) and the FP64 coupling cost the range's share of the full sweep;
+ * the float tensor-core coupling forms its
  * per-string products for the range's strings and their single-excitation
  * partners (for a contiguous range of more than a few rows, nearly all).
  * 0 <= row_begin <= row_end <= N_alpha, else HY_ERR_ARG. */

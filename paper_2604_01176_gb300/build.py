@@ -19,7 +19,7 @@ LIB = os.path.join(PKG, "libhyperion.so")
 SOURCES = ["hy_build.cpp", "hy_api.cu", "hy_sigma.cu", "hy_sweeps.cu",
            "hy_adapt.cpp", "hy_ranker.cu", "hy_batch.cu", "hy_sparse.cu", "hy_profile.cpp",
            "hy_cpl_tc.cu", "hy_hmat.cu", "hy_fold.cu", "hy_screen.cu",
-           "hy_rows64.cu", "hy_dense.cu", "hy_screen32.cu"]
+           "hy_rows64.cu", "hy_dense.cu", "hy_screen32.cu", "hy_same.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler",
                 "-fPIC,-fopenmp,-O3", "-I", INCLUDE, "-I", CSRC]

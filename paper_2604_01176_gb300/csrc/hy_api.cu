@@ -116,6 +116,10 @@ struct hy_ham {
     // operand tables of the float tensor-core coupling (kCplWideOrbitals and up)
     uint16_t *d_cent = nullptr;
     uint32_t *d_ctmask = nullptr;
+    // off-diagonal same-spin tables as tensor-core operands (hy_same.cu; pack
+    // null: the CSR kernel runs), by spin, and the CTA pairs that run at once
+    hy::k::SameArgs same[2] = {};
+    int same_pairs = 0;
     double *d_V64 = nullptr;
     float *d_V32 = nullptr;
     double *d_h1 = nullptr, *d_eri = nullptr;   // integrals (ranker features)
@@ -438,8 +442,14 @@ hy_status apply_h_t(hy_ham *h, const T *psi, T *sigma, cudaStream_t st, int64_t 
     const int64_t Nbp = (h->Nb + 63) / 64 * 64;
     const size_t tbytes = sizeof(T) == sizeof(float)
         ? size_t(h->Na) * size_t(h->A.nex + 1) * size_t(Nbp) * sizeof(float) : 0;
-    bool dense = false;
-    if (tbytes && ensure_ws(h, L.total + tbytes) == HY_OK) {
+    // the tensor-core same-spin part takes the same place before it
+    size_t xbytes = 0;
+    if (sizeof(T) == sizeof(float) && h->same[0].pack && h->same[1].pack && h->cpl_impl != 1 && h->d_status)
+        xbytes = std::max(hy::k::same_x_bytes(h->Na, h->Nb), hy::k::same_x_bytes(h->Nb, nr));
+    bool dense = false, same = false;
+    if (xbytes && ensure_ws(h, L.total + std::max(tbytes, xbytes)) == HY_OK) {
+        dense = same = true;
+    } else if (tbytes && (cudaGetLastError(), ensure_ws(h, L.total + tbytes) == HY_OK)) {
         dense = true;
     } else {
         cudaGetLastError();   // clear a failed allocation
@@ -461,11 +471,40 @@ hy_status apply_h_t(hy_ham *h, const T *psi, T *sigma, cudaStream_t st, int64_t 
     const double rows_det = double(nr) * double(h->Nb);
     hy::ProfScope prof(HY_PROF_HPSI, st, 2.0 * rows_det * sizeof(T),
                        2.0 * double(hy::ham_connections(h)) * rows_det);
-    HY_CUDA(hy::k::spmm<T>(Ma->ptr + r0, Ma->col, Ma->val, nr, psi, sigma, h->Nb,
-                           false, st), "alpha part");
-    HY_CUDA(hy::k::transpose<T>(psi + r0 * h->Nb, psiT, nr, h->Nb, st), "transpose");
-    HY_CUDA(hy::k::spmm<T>(Mb->ptr, Mb->col, Mb->val, h->Nb, psiT, tau, nr,
-                           false, st), "beta part");
+    bool tc = false;            // a kernel ran that may report a timeout
+    auto status_back = [&]() {
+        if (tc)
+            HY_CUDA(cudaMemcpyAsync(h->h_status, h->d_status, sizeof(int), cudaMemcpyDeviceToHost, st),
+                    "status copy");
+        return HY_OK;
+    };
+    if constexpr (sizeof(T) == sizeof(float)) {
+        if (same) {
+            // the coupling's intermediate is written later
+            hy::k::SameArgs a = h->same[0], b = h->same[1];
+            a.xpack = b.xpack = reinterpret_cast<unsigned char *>(ws + L.total);
+            a.Y = sigma;
+            a.ncols = h->Nb;
+            a.row0 = r0;
+            a.row1 = r1;
+            HY_CUDA(hy::k::same(a, psi, h->Nb, false, h->same_pairs, h->d_status, h->tc_spin_limit, st),
+                    "alpha part");
+            b.Y = tau;
+            b.ncols = nr;
+            b.row0 = 0;
+            b.row1 = h->Nb;
+            HY_CUDA(hy::k::same(b, psi + r0 * h->Nb, h->Nb, true, h->same_pairs, h->d_status,
+                                h->tc_spin_limit, st), "beta part");
+            tc = true;
+        }
+    }
+    if (!same) {
+        HY_CUDA(hy::k::spmm<T>(Ma->ptr + r0, Ma->col, Ma->val, nr, psi, sigma, h->Nb,
+                               false, st), "alpha part");
+        HY_CUDA(hy::k::transpose<T>(psi + r0 * h->Nb, psiT, nr, h->Nb, st), "transpose");
+        HY_CUDA(hy::k::spmm<T>(Mb->ptr, Mb->col, Mb->val, h->Nb, psiT, tau, nr,
+                               false, st), "beta part");
+    }
     HY_CUDA(hy::k::add_transposed<T>(tau, sigma, nr, h->Nb, st), "beta add");
     if constexpr (sizeof(T) == sizeof(float)) {
         if (dense) {
@@ -499,9 +538,7 @@ hy_status apply_h_t(hy_ham *h, const T *psi, T *sigma, cudaStream_t st, int64_t 
                                                          h->cpl_impl == 0 ? 1 : 0, h->num_sms, st);
                 if (e == cudaSuccess) {
                     HY_CUDA(hy::k::coupling_gather(d, h->num_sms, st), "alpha-beta gather");
-                    HY_CUDA(cudaMemcpyAsync(h->h_status, h->d_status, sizeof(int),
-                                            cudaMemcpyDeviceToHost, st), "status copy");
-                    done = true;
+                    done = tc = true;
                 } else if (e != cudaErrorInvalidValue) {
                     return cuda_fail(e, "alpha-beta coupling (tensor cores)");
                 }
@@ -509,7 +546,7 @@ hy_status apply_h_t(hy_ham *h, const T *psi, T *sigma, cudaStream_t st, int64_t 
             if (!done)
                 HY_CUDA(hy::k::coupling_dense(d, h->num_sms, st), "alpha-beta coupling (dense)");
             if (h->prof) cudaEventRecord(h->ev1, st);
-            return HY_OK;
+            return status_back();
         }
     }
     hy::k::CouplingArgs<T> a;
@@ -530,7 +567,7 @@ hy_status apply_h_t(hy_ham *h, const T *psi, T *sigma, cudaStream_t st, int64_t 
     if (h->prof) cudaEventRecord(h->ev0, st);
     HY_CUDA(hy::k::coupling<T>(a, h->num_sms, st), "alpha-beta coupling");
     if (h->prof) cudaEventRecord(h->ev1, st);
-    return HY_OK;
+    return status_back();
 }
 
 template <typename T>
@@ -979,6 +1016,53 @@ hy_status fold_same_spin(hy_ham *h)
     return HY_OK;
 }
 
+// the float same-spin table of one spin as tensor-core operands; without the
+// memory for it the CSR kernel stays in use
+hy_status pack_same_spin(hy_ham *h, int spin)
+{
+    const int64_t N = spin == 0 ? h->Na : h->Nb;
+    const DevCsr<float> &M = spin == 0 ? h->Ma32 : h->Mb32;
+    const int nrb = hy::k::same_row_blocks(N), nch = hy::k::same_chunks(N);
+    DevArena tmp, ar;
+    uint32_t *place = nullptr;
+    int32_t *count = nullptr;
+    std::vector<int32_t> cnt(size_t(nrb), 0);
+    cudaError_t e = tmp.alloc(&place, size_t(nrb) * nch, true);
+    if (e == cudaSuccess) e = tmp.alloc(&count, size_t(nrb));
+    if (e == cudaSuccess) e = hy::k::same_used(M.ptr, M.col, N, place, count, nullptr);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(cnt.data(), count, cnt.size() * sizeof(int32_t), cudaMemcpyDeviceToHost);
+    std::vector<int64_t> base(size_t(nrb) + 1, 0);
+    for (int i = 0; i < nrb; ++i) base[i + 1] = base[i] + cnt[i];
+    int64_t *d_base = nullptr;
+    uint16_t *list = nullptr;
+    unsigned char *pack = nullptr;
+    float *diag = nullptr;
+    if (e == cudaSuccess) e = ar.upload(&d_base, base.data(), base.size());
+    if (e == cudaSuccess) e = ar.alloc(&list, size_t(base[nrb]));
+    if (e == cudaSuccess) e = ar.alloc(&diag, size_t(N), true);
+    if (e == cudaSuccess) e = ar.alloc(&pack, size_t(base[nrb]) * hy::k::same_block_bytes(), true);
+    if (e == cudaSuccess && pack)
+        e = hy::k::same_fill(M.ptr, M.col, M.val, N, place, d_base, list, pack, diag, nullptr);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    tmp.release();
+    if (e != cudaSuccess || !pack) {
+        ar.release();
+        if (e != cudaSuccess && e != cudaErrorMemoryAllocation) return cuda_fail(e, "same-spin operands");
+        cudaGetLastError();
+        return HY_OK;
+    }
+    h->arena.ptrs.insert(h->arena.ptrs.end(), ar.ptrs.begin(), ar.ptrs.end());
+    h->arena.uploaded += ar.uploaded;
+    hy::k::SameArgs &a = h->same[spin];
+    a.N = N;
+    a.pack = pack;
+    a.base = d_base;
+    a.list = list;
+    a.diag = diag;
+    return HY_OK;
+}
+
 // host copies of the same-spin tables, for host consumers (the explicit-H
 // builder); copied once from the device
 hy_status ensure_host_csr(hy_ham *h)
@@ -1085,6 +1169,10 @@ hy_status finish_ham(hy_ham *h, hy_ham **out)
                                   h->num_sms, nullptr), "coupling tables");
     }
     if (s == HY_OK) s = fold_same_spin(h);
+    if (s == HY_OK && std::min(h->Na, h->Nb) >= hy::k::kSameStrings) {
+        h->same_pairs = hy::k::same_pairs();
+        for (int spin = 0; spin < 2 && s == HY_OK && h->same_pairs > 0; ++spin) s = pack_same_spin(h, spin);
+    }
     if (s != HY_OK) {
         std::string msg = g_err;
         hy_ham_destroy(h);

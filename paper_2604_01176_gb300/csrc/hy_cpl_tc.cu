@@ -29,6 +29,7 @@
 // kernel records it in *status, waits (bounded) for its own MMAs, frees its
 // tensor memory and returns.
 #include "hy_kernels.cuh"
+#include "hy_tc.cuh"
 
 #include <algorithm>
 
@@ -53,24 +54,6 @@ constexpr size_t kWBytes = size_t(kTcM) * kWRow * 4;       // W_J in FP32, 65 KB
 constexpr size_t kABytes = size_t(kTcM) * kTcKc * 4;       // one A chunk, 8 KB
 constexpr size_t kBBytes = size_t(kTcN) * kTcKc * 4;       // one G chunk, 16 KB
 constexpr size_t kStage = 2 * kABytes + 2 * kBBytes;       // hi, lo of both
-
-__device__ __forceinline__ uint32_t saddr(const void *p)
-{
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-// byte offset of element (row, k) in a K-major no-swizzle operand
-__device__ __forceinline__ uint32_t kmaj(int row, int k, uint32_t sbo)
-{
-    return uint32_t(row >> 3) * sbo + uint32_t(k >> 2) * 128u + uint32_t(row & 7) * 16u +
-           uint32_t(k & 3) * 4u;
-}
-
-__device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t sbo)
-{
-    return uint64_t((addr >> 4) & 0x3FFFu) | (uint64_t(128u >> 4) << 16) |
-           (uint64_t((sbo >> 4) & 0x3FFFu) << 32) | (uint64_t(1) << 46);
-}
 
 // kind::tf32, FP32 accumulate, K-major A and B, M = 64, N = 128
 constexpr uint32_t kIdesc = (1u << 4) | (2u << 7) | (2u << 10) | (uint32_t(kTcN >> 3) << 17) |
@@ -101,12 +84,6 @@ __device__ __forceinline__ bool wait_bar(uint64_t *bar, uint32_t par, long long 
         if (done) return true;
     }
     return false;
-}
-
-__device__ __forceinline__ void split(float x, float &hi, float &lo)
-{
-    hi = __uint_as_float(__float_as_uint(x) & 0xFFFFE000u);
-    lo = x - hi;
 }
 
 __device__ __forceinline__ void tmem_ld32(uint32_t addr, float *v)
@@ -445,13 +422,6 @@ __device__ __forceinline__ bool tw_wait_warp(TwCtl *c, uint64_t *bar, uint32_t p
     return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
-__device__ __forceinline__ bool elect_one()
-{
-    uint32_t p;
-    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(p));
-    return p != 0;
-}
-
 // barrier of the builders (all of them, always); whether v holds in every one
 __device__ __forceinline__ bool builders_and(bool v)
 {
@@ -703,7 +673,7 @@ k_cpl_tcw(CplDenseArgs a, int nst, int *status, long long spin_limit, int issue)
         if (issue) {
             if (elect_one()) commit(&ctl->fin);
             __syncwarp();
-            wait_bar(&ctl->fin, 0, spin_limit);
+            wait_bar(&ctl->fin, 0, spin_limit > (1ll << 24) ? spin_limit : 1ll << 24);
         }
         __syncwarp();
     } else {

@@ -110,6 +110,37 @@ cudaError_t cpl_entries(const uint32_t *bstr, const uint32_t *bexT, int64_t Nb, 
 cudaError_t coupling_tc(const CplDenseArgs &a, int *status, long long spin_limit, int issue,
                         int num_sms, cudaStream_t st);
 
+// same-spin part on the tensor cores (hy_same.cu): Y = M X for output rows
+// [row0, row1), Y holding row row0 first; M as MMA operands by blocks of 256 rows
+// (same_used, same_fill: place and pack zeroed before, base the sums of count)
+// Strings of each spin from which it is used (of the Hamiltonian, not of the rows at
+// hand: a range of rows gives the full sweep's sums).  Below, a launch costs more
+// than the rows do: 462 strings 184 us by rows, 194 so (whole float H|psi>, 11
+// orbitals, 6+5); 560 strings 286 -> 269, 792 420 -> 387, 1,820 2,211 -> 1,599.
+constexpr int kSameStrings = 512;
+struct SameArgs {
+    unsigned char *xpack;       // same_x_bytes of scratch: X as operands
+    float *Y;
+    int64_t N, ncols, row0, row1;
+    const unsigned char *pack;
+    const int64_t *base;        // [row blocks + 1] first block of each
+    const uint16_t *list;       // columns / 32 of each block
+    const float *diag;
+};
+int same_row_blocks(int64_t N);
+int same_chunks(int64_t N);
+size_t same_block_bytes();
+cudaError_t same_used(const int32_t *ptr, const int32_t *col, int64_t N, uint32_t *place,
+                      int32_t *count, cudaStream_t st);
+cudaError_t same_fill(const int32_t *ptr, const int32_t *col, const float *val, int64_t N,
+                      const uint32_t *place, const int64_t *base, uint16_t *list,
+                      unsigned char *pack, float *diag, cudaStream_t st);
+int same_pairs();
+size_t same_x_bytes(int64_t N, int64_t ncols);
+// element (J, c) of X: src[c * stride + J] if trans, else src[J * stride + c]
+cudaError_t same(const SameArgs &a, const float *src, int64_t stride, bool trans, int pairs, int *status,
+                 long long spin_limit, cudaStream_t st);
+
 template <typename T>
 cudaError_t spmm(const int32_t *ptr, const int32_t *col, const T *val,
                  int64_t rows, const T *X, T *Y, int64_t ncols, bool accumulate,
