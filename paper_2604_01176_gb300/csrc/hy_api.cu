@@ -2663,6 +2663,7 @@ struct hy::SparseState {
     int32_t *ralpha = nullptr, *blist = nullptr;
     uint8_t *flags = nullptr;
     unsigned long long *ctr = nullptr;
+    void *sup_tables = nullptr;          // its tables in double (SupRowsArgs)
 };
 
 namespace {
@@ -2736,6 +2737,7 @@ void sstate_destroy(SparseState *s)
     cudaFree(s->partials);
     cudaFree(s->blk);
     cudaFree(s->runs);
+    cudaFree(s->sup_tables);
     cudaFree(s->ralpha);
     cudaFree(s->blist);
     cudaFree(s->flags);
@@ -3308,6 +3310,21 @@ hy_status sstate_apply_h_support(const SparseState *s, SparseState *sig, void *s
         hy::k::SupRowsArgs<double> a;
         a.s = sparse_args<double>(h, s->v, sigma, sig->list, 0);
         run(a);
+        // the tables lie one behind the other, the widest first
+        const size_t nb = size_t(h->Nb), nn = size_t(h->n) * h->n;
+        const size_t nnz = nb * size_t(hy::k::fold_candidates(h->n, h->nb));
+        if (!sig->sup_tables) {
+            const cudaError_t e =
+                cudaMalloc(&sig->sup_tables, (nnz + nn * nb) * 8 + (64 + 3) * nb * 4 + nnz * 2);
+            if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(support rows)");
+        }
+        a.mval = static_cast<double *>(sig->sup_tables);
+        a.dbeta = a.mval + nnz;
+        a.fex = reinterpret_cast<uint32_t *>(a.dbeta + nn * nb);
+        a.number = reinterpret_cast<int32_t *>(a.fex + 64 * nb);
+        a.nfex = a.number + nb;
+        a.nm = a.nfex + nb;
+        a.mcol = reinterpret_cast<uint16_t *>(a.nm + nb);
         HY_CUDA(hy::k::hpsi_support<double>(a, h->num_sms, st), "support H psi");
     } else {
         hy::k::SupRowsArgs<float> a;

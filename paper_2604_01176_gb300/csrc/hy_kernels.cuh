@@ -374,6 +374,12 @@ struct SupRowsArgs {
     uint8_t *flagA, *flagB;
     int32_t *blist;
     unsigned long long *ctr;
+    // double only: by beta string or its number in S (number: Nb, nfex, nm: Nb;
+    // fex: 64 Nb; mcol, mval: Nb times M_beta's longest row; dbeta: n^2 Nb)
+    int32_t *number, *nfex, *nm;
+    uint32_t *fex;
+    uint16_t *mcol;
+    double *mval, *dbeta;
 };
 template <typename T>
 cudaError_t hpsi_support(const SupRowsArgs<T> &a, int num_sms, cudaStream_t st);

@@ -251,8 +251,7 @@ __device__ __forceinline__ void stage_row(T *row, const T *src, int64_t Nb)
 // The alpha-beta part runs a thread per row (A, B): the row's beta
 // excitations stay in registers, and each staged row A_e costs it one fused
 // multiply-add per beta excitation (plus one per occupied beta orbital, the
-// diagonal beta part) and no cross-lane reduction -- in double precision the
-// GB300's FP64 pipe is the bound, so every FP64 instruction is useful work.
+// diagonal beta part) and no cross-lane reduction.
 // The same-alpha part (CSR rows of ~n^4/4 entries) keeps a warp per row with
 // its lanes over the entries, reduced once per row.
 template <typename T>
@@ -403,6 +402,242 @@ k_sup_beta(SupRowsArgs<T> a)
                 part = warp_sum(part);
                 if (lane == 0) h.sigma[A * Nb + B] += part;
             }
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// The same in double (k_sup_rows): the strings of S are few (450 of 12,870 in
+// 200,000 determinants), so the beta strings present are numbered and everything
+// is restricted to them first:
+//   k_sup_number, one CTA: blist, the beta strings of S in order, and their
+//     numbers (-1: none);
+//   k_sup_tables, a warp per beta string j: its excitations and its M_beta row
+//     that stay among them (j-minor, so that neighbouring rows read neighbouring
+//     words), and D[pq][j] = sum_{r in B_j} V[pq][rr];
+//   k_sup_rows, one CTA per alpha string A: a thread per row (A, B), psi's rows A
+//     and A_e of the numbered strings in shared memory, the next one on its way
+//     (cp.async) while one is used; A's M_alpha row, filtered once, reads psi down
+//     column B.
+// k_sup_alpha stages all Nb amplitudes of a row for each A_e and multiplies all 64
+// excitations, k_sup_beta a column of Na.  Bound by FP64 (a multiply-add per
+// coupling inside S), then by the runs' lengths.  Measured, 200,000 determinants of
+// 8 + 8 electrons in 16 orbitals: 1,330 -> 332 us (k_sup_rows 285); the sums are in
+// another order, so float, whose results are kept, stays with the two above.
+// ---------------------------------------------------------------------------
+constexpr int kSupRowMax = 896;        // entries of an M_alpha row: 849 at most
+
+__global__ void __launch_bounds__(1024)
+k_sup_number(const uint8_t *__restrict__ flagB, int Nb, int32_t *__restrict__ number,
+             int32_t *__restrict__ blist, unsigned long long *__restrict__ ctr)
+{
+    __shared__ int wt[32];
+    const int per = (Nb + 1023) / 1024, b0 = int(threadIdx.x) * per, b1 = min(Nb, b0 + per);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int c = 0;
+    for (int b = b0; b < b1; ++b) c += flagB[b];
+    int x = c;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wt[w] = x;
+    __syncthreads();
+    int pos = x - c;
+    for (int i = 0; i < w; ++i) pos += wt[i];
+    for (int b = b0; b < b1; ++b) {
+        const bool in = flagB[b] != 0;
+        number[b] = in ? pos : -1;
+        if (in) blist[pos++] = b;
+    }
+    if (threadIdx.x == 1023) ctr[1] = (unsigned long long)pos;
+}
+
+__global__ void __launch_bounds__(256)
+k_sup_tables(SupRowsArgs<double> a)
+{
+    const SparseArgs<double> &h = a.s;
+    const int n = h.n, nn = n * n, nb = int(a.ctr[1]), lane = threadIdx.x & 31;
+    const uint32_t below = (1u << lane) - 1u;
+    for (int j = int(blockIdx.x) * 8 + int(threadIdx.x >> 5); j < nb; j += int(gridDim.x) * 8) {
+        const int64_t B = a.blist[j];
+        if (blockIdx.y) {                         // the diagonal sums: a half of the blocks
+            const uint32_t bm = h.bstr[B];
+            for (int q = lane; q < nn; q += 32)
+                a.dbeta[size_t(q) * nb + j] = sum_mask(h.V + size_t(q) * nn, n + 1, bm);
+            continue;
+        }
+        int c = 0;
+        for (int f0 = 0; f0 < h.nexb; f0 += 32) {
+            const int f = f0 + lane;
+            const uint32_t w = f < h.nexb ? h.bex[B * h.nexb + f] : 0u;
+            const int o = f < h.nexb ? a.number[w & 0xFFFFu] : -1;
+            const unsigned in = __ballot_sync(0xffffffffu, o >= 0);
+            if (o >= 0)
+                a.fex[size_t(c + __popc(in & below)) * nb + j] =
+                    uint32_t(o) | (((w >> 20) & 15u) * n + ((w >> 16) & 15u)) << 16 | (w & 0x80000000u);
+            c += __popc(in);
+        }
+        if (lane == 0) a.nfex[j] = c;
+        c = 0;
+        const int k1 = h.Mb_ptr[B + 1];
+#pragma unroll 4
+        for (int k0 = h.Mb_ptr[B]; k0 < k1; k0 += 32) {
+            const int k = k0 + lane;
+            const int o = k < k1 ? a.number[h.Mb_col[k]] : -1;
+            const unsigned in = __ballot_sync(0xffffffffu, o >= 0);
+            if (o >= 0) {
+                const size_t at = size_t(c + __popc(in & below)) * nb + j;
+                a.mcol[at] = uint16_t(o);
+                a.mval[at] = h.Mb_val[k];
+            }
+            c += __popc(in);
+        }
+        if (lane == 0) a.nm[j] = c;
+    }
+}
+
+__device__ __forceinline__ void cp_async8(double *dst, const double *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;"
+                 ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))), "l"(src)
+                 : "memory");
+}
+
+size_t sup_rows_smem(int64_t Nb, int nn)
+{
+    return (2 * (size_t(Nb) + size_t(nn)) + size_t(nn) + kSupRowMax) * sizeof(double) +
+           kSupRowMax * sizeof(int32_t);
+}
+
+__global__ void __launch_bounds__(kSupThreads, 1)
+k_sup_rows(SupRowsArgs<double> a)
+{
+    extern __shared__ __align__(16) unsigned char sup_sm[];
+    const SparseArgs<double> &h = a.s;
+    const int n = h.n, nn = n * n, nexa = h.nexa;
+    const int64_t Nb = h.Nb;
+    const int nb = int(a.ctr[1]);
+    double *row0 = reinterpret_cast<double *>(sup_sm);    // two rows of psi
+    double *vrow0 = row0 + 2 * Nb;                        // V[pq_e][.] of each
+    double *dA = vrow0 + 2 * nn;                          // sum_{p in A} V[pp][.]
+    double *mav = dA + nn;                                // A's M_alpha row inside S
+    int32_t *mac = reinterpret_cast<int32_t *>(mav + kSupRowMax);
+    __shared__ uint32_t aexs[64];
+    __shared__ int64_t sh_r;
+    __shared__ int sh_cnt[kSupThreads / 32], sh_ne, sh_nm;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    auto stage = [&](int buf, int64_t R, int pq) {
+        double *row = row0 + buf * Nb;
+        for (int j = tid; j < nb; j += kSupThreads) cp_async8(row + j, h.psi + R * Nb + a.blist[j]);
+        if (pq >= 0)
+            for (int q = tid; q < nn; q += kSupThreads)
+                cp_async8(vrow0 + buf * nn + q, h.V + size_t(pq) * nn + q);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    auto pq_of = [&](uint32_t u) { return int((u >> 20) & 15) * n + int((u >> 16) & 15); };
+    for (;;) {
+        __syncthreads();                          // the previous run's rows are read
+        if (tid == 0) sh_r = int64_t(atomicAdd(a.ctr + 2, 1ull));
+        __syncthreads();
+        const int64_t r = sh_r;
+        if (r >= int64_t(a.ctr[0])) break;
+        const int64_t t0 = a.runs[r], A = a.ralpha[r];
+        // the run's length: A's row of the bitmap (bits A Nb .. A Nb + Nb - 1)
+        {
+            const int64_t b0 = A * Nb, b1 = b0 + Nb, w0 = b0 >> 5, w1 = (b1 - 1) >> 5;
+            int c = 0;
+            for (int64_t w = w0 + tid; w <= w1; w += kSupThreads) {
+                uint32_t x = a.bits[w];
+                if (w == w0) x &= ~0u << (b0 & 31);
+                if (w == w1 && (b1 & 31)) x &= (1u << (b1 & 31)) - 1u;
+                c += __popc(x);
+            }
+            c = warp_sum(c);
+            if (lane == 0) sh_cnt[warp] = c;
+        }
+        const uint32_t am = h.astr[A];
+        for (int i = tid; i < nn; i += kSupThreads) dA[i] = sum_diag<double>(h.V, n, nn, am, i);
+        if (warp < 2) {
+            // A's excitations (warp 0) and M_alpha row (warp 1) to strings of S
+            int c = 0;
+            const int k1 = warp ? h.Ma_ptr[A + 1] : nexa;
+            for (int k0 = warp ? h.Ma_ptr[A] : 0; k0 < k1; k0 += 32) {
+                const int k = k0 + lane;
+                uint32_t u = 0u;
+                if (k < k1) u = warp ? uint32_t(h.Ma_col[k]) : h.aex[A * nexa + k];
+                const bool in = k < k1 && a.flagA[u & 0xFFFFu];
+                const unsigned bal = __ballot_sync(0xffffffffu, in);
+                const int pos = c + __popc(bal & ((1u << lane) - 1u));
+                if (in && warp == 0) aexs[pos] = u;
+                if (in && warp == 1) {
+                    mac[pos] = int32_t(u);
+                    mav[pos] = h.Ma_val[k];
+                }
+                c += __popc(bal);
+            }
+            if (lane == 0) *(warp ? &sh_nm : &sh_ne) = c;
+        }
+        __syncthreads();
+        int64_t mA = 0;
+        for (int w = 0; w < kSupThreads / 32; ++w) mA += sh_cnt[w];
+        if (t0 + mA > a.cap) mA = a.cap - t0;    // an overflowed (invalid) support
+        const int ne = sh_ne, nma = sh_nm;
+        const int64_t *Brun = a.list + t0;
+        for (int64_t c0 = 0; c0 < mA; c0 += kSupThreads) {
+            // row A in buffer 0, then the rows A_e in turn
+            stage(0, A, -1);
+            if (ne) stage(1, aexs[0] & 0xFFFFu, pq_of(aexs[0]));
+            const int64_t i = c0 + tid;
+            const bool act = i < mA;
+            const int64_t B = act ? Brun[i] - A * Nb : 0;
+            const int j = act ? a.number[B] : 0, nf = act ? a.nfex[j] : 0, nm = act ? a.nm[j] : 0;
+            const uint32_t bm = act ? h.bstr[B] : 0u;
+            double s = 0.0;
+            if (act) {
+                const double *col = h.psi + B;
+#pragma unroll 4
+                for (int k = 0; k < nma; ++k) s = fma(mav[k], __ldg(col + int64_t(mac[k]) * Nb), s);
+            }
+            if (ne) asm volatile("cp.async.wait_group 1;" ::: "memory");
+            else asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncthreads();
+            const uint32_t *ex = a.fex + j;
+            {
+                const double *row = row0;
+#pragma unroll 4
+                for (int k = 0; k < nm; ++k)
+                    s = fma(a.mval[size_t(k) * nb + j], row[a.mcol[size_t(k) * nb + j]], s);
+                for (int f = 0; f < nf; ++f) {
+                    const uint32_t w = ex[size_t(f) * nb];
+                    const double c = dA[(w >> 16) & 255u];
+                    s = fma((w >> 31) ? -c : c, row[w & 0xFFFFu], s);
+                }
+                if (act) {
+                    double d = 0.0;
+                    for (uint32_t mm = bm; mm; mm &= mm - 1) d += dA[(__ffs(mm) - 1) * (n + 1)];
+                    s = fma(d, row[j], s);
+                }
+            }
+            for (int e = 0; e < ne; ++e) {
+                const int buf = (e + 1) & 1;
+                const uint32_t u = aexs[e];
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+                __syncthreads();                  // this row is there, the last one read
+                if (e + 1 < ne) stage(buf ^ 1, aexs[e + 1] & 0xFFFFu, pq_of(aexs[e + 1]));
+                if (!act) continue;
+                const double *row = row0 + buf * Nb, *vrow = vrow0 + buf * nn;
+                double t = __ldg(a.dbeta + size_t(pq_of(u)) * nb + j) * row[j];
+#pragma unroll 4
+                for (int f = 0; f < nf; ++f) {
+                    const uint32_t w = ex[size_t(f) * nb];
+                    const double c = vrow[(w >> 16) & 255u];
+                    t = fma((w >> 31) ? -c : c, row[w & 0xFFFFu], t);
+                }
+                s = (u >> 31) ? s - t : s + t;
+            }
+            if (act) h.sigma[Brun[i]] = s;
+            __syncthreads();                      // both buffers are free
         }
     }
 }
@@ -2087,6 +2322,19 @@ cudaError_t hpsi_support(const SupRowsArgs<T> &a, int num_sms, cudaStream_t st)
     k_sup_runs<<<unsigned(g), 256, 0, st>>>(a.list, a.cnt, a.cap, h.Nb, a.runs, a.ralpha,
                                              a.flagA, a.flagB, a.ctr);
     hy::count_launch();
+    if constexpr (sizeof(T) == 8) {
+        k_sup_number<<<1, 1024, 0, st>>>(a.flagB, int(h.Nb), a.number, a.blist, a.ctr);
+        hy::count_launch();
+        k_sup_tables<<<dim3(unsigned(num_sms) * 2, 2), 256, 0, st>>>(a);
+        hy::count_launch();
+        const size_t sr = sup_rows_smem(h.Nb, h.n * h.n);
+        e = cudaFuncSetAttribute(k_sup_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sr));
+        if (e != cudaSuccess) return e;
+        // 512 threads of at most 128 registers: one CTA an SM, whatever it stages
+        k_sup_rows<<<unsigned(num_sms), kSupThreads, sr, st>>>(a);
+        hy::count_launch();
+        return cudaGetLastError();
+    } else {
     k_sup_blist<<<unsigned(num_sms), 256, 0, st>>>(a.flagB, h.Nb, a.blist, a.ctr);
     hy::count_launch();
     const size_t sa = sup_alpha_smem<T>(h.Nb, h.n * h.n), sb = size_t(h.Na) * sizeof(T);
@@ -2094,12 +2342,12 @@ cudaError_t hpsi_support(const SupRowsArgs<T> &a, int num_sms, cudaStream_t st)
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_sup_beta<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sb));
     if (e != cudaSuccess) return e;
-    const unsigned per_sm = sizeof(T) == 8 ? 1u : 2u;
-    k_sup_alpha<T><<<unsigned(num_sms) * per_sm, kSupThreads, sa, st>>>(a);
+    k_sup_alpha<T><<<unsigned(num_sms) * 2u, kSupThreads, sa, st>>>(a);
     hy::count_launch();
-    k_sup_beta<T><<<unsigned(num_sms) * per_sm, kSupThreads, sb, st>>>(a);
+    k_sup_beta<T><<<unsigned(num_sms) * 2u, kSupThreads, sb, st>>>(a);
     hy::count_launch();
     return cudaGetLastError();
+    }
 }
 
 template <typename T>
