@@ -580,7 +580,10 @@ hy_status gradient(hy_adapt *a, const std::vector<double> &th, hy_dtype dt,
         HY_TRY(cu(cudaMemcpyAsync(lam, sigma, size_t(a->N) * es, cudaMemcpyDeviceToDevice, st),
                   "copy"));
     }
-    for (size_t l = j; l-- > 0;) {
+    if (lam_closed)
+        HY_TRY(hy::sstate_reverse_closed(F, L, a->p, a->ops.data(), a->d_ops, th.data(), int64_t(j),
+                                         a->sparse_m, a->d_ga, st));
+    for (size_t l = lam_closed ? 0 : j; l-- > 0;) {
         HY_TRY(hy::sstate_gradients(F, lam, a->p, a->d_ops + l, 1, a->sparse_m, a->d_ga + l, st));
         if (l == 0) break;
         // phi_{l-1} = U_l^T phi_l lies inside S_{l-1}, within psi's support S:
@@ -588,7 +591,7 @@ hy_status gradient(hy_adapt *a, const std::vector<double> &th, hy_dtype dt,
         // rotations keep S's list (closed) instead of listing such partners
         HY_TRY(hy::sstate_excite(F, a->p, a->ops[l], -th[l], st, true));
         if (lam_sparse)
-            HY_TRY(hy::sstate_excite(L, a->p, a->ops[l], -th[l], st, lam_closed));
+            HY_TRY(hy::sstate_excite(L, a->p, a->ops[l], -th[l], st, false));
         else
             HY_TRY(hy_apply_excitation(a->h, a->p, a->ops[l], -th[l], lam, dt, 0, st));
     }

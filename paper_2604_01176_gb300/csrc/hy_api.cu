@@ -2777,21 +2777,28 @@ hy_status sstate_copy(SparseState *dst, const SparseState *src, void *stream)
 
 void sstate_set_hint(SparseState *s, int64_t n) { s->hint = n; }
 
+namespace {
+hy::k::SvOpArgs sv_op_args(const hy_ham *h, const hy_pool *p)
+{
+    hy::k::SvOpArgs o;
+    o.desc = p->d_desc;
+    o.astr = h->d_astr;
+    o.bstr = h->d_bstr;
+    o.rank16 = h->d_rank16;
+    o.n = h->n;
+    o.Nb = h->Nb;
+    o.qubit = p->qubit;
+    return o;
+}
+}  // namespace
+
 hy_status sstate_excite(SparseState *s, const hy_pool *p, int64_t k, double theta, void *stream,
                         bool closed)
 {
     const hy_ham *h = s->h;
     if (!p || p->h != h || k < 0 || k >= int64_t(p->ops.size()))
         return fail(HY_ERR_ARG, "bad operator");
-    hy::k::SvOpArgs o;
-    o.desc = p->d_desc;
-    o.astr = h->d_astr;
-    o.bstr = h->d_bstr;
-    o.binom33 = h->d_binom;
-    o.rank16 = h->d_rank16;
-    o.n = h->n;
-    o.Nb = h->Nb;
-    o.qubit = p->qubit;
+    const hy::k::SvOpArgs o = sv_op_args(h, p);
     const int nc = p->ops[k].desc[0];
     cudaStream_t st = as_stream(stream);
     // bytes estimated from the support the host last read back (the count
@@ -2817,15 +2824,7 @@ hy_status sstate_prepare(SparseState *s, const hy_pool *p, const int32_t *ops, c
     const hy_ham *h = s->h;
     if (!p || p->h != h || (L > 0 && (!ops || !cs)) || L < 0 || L > (1 << 20))
         return fail(HY_ERR_ARG, "bad arguments");
-    hy::k::SvOpArgs o;
-    o.desc = p->d_desc;
-    o.astr = h->d_astr;
-    o.bstr = h->d_bstr;
-    o.binom33 = h->d_binom;
-    o.rank16 = h->d_rank16;
-    o.n = h->n;
-    o.Nb = h->Nb;
-    o.qubit = p->qubit;
+    const hy::k::SvOpArgs o = sv_op_args(h, p);
     cudaStream_t st = as_stream(stream);
     hy::ProfScope prof(HY_PROF_SPARSE_EXCITE, stream, 0.0);
     if (s->dt == HY_F64)
@@ -2938,22 +2937,6 @@ int64_t prog_steps(const hy_pool *p, const int32_t *ops_host, int64_t L)
     for (int64_t l = 0; l < L; ++l) s += p->ops[size_t(ops_host[l])].desc[0];
     return s;
 }
-
-namespace {
-hy::k::SvOpArgs sv_op_args(const hy_ham *h, const hy_pool *p)
-{
-    hy::k::SvOpArgs o;
-    o.desc = p->d_desc;
-    o.astr = h->d_astr;
-    o.bstr = h->d_bstr;
-    o.binom33 = h->d_binom;
-    o.rank16 = h->d_rank16;
-    o.n = h->n;
-    o.Nb = h->Nb;
-    o.qubit = p->qubit;
-    return o;
-}
-}  // namespace
 
 hy_status prog_compile(SupportProgram *g, const SparseState *s, int64_t m, const hy_pool *p,
                        const int32_t *ops, int64_t L, int64_t steps, void *stream)
@@ -3186,15 +3169,7 @@ hy_status sstate_grad_forward(SparseState *f, SparseState *w, const hy_pool *p, 
     if (!p || p->h != h || w->h != h || w->dt != f->dt || !sigma || !g || L < 1 ||
         L > (1 << 20) || !ops || !cs)
         return fail(HY_ERR_ARG, "bad arguments");
-    hy::k::SvOpArgs o;
-    o.desc = p->d_desc;
-    o.astr = h->d_astr;
-    o.bstr = h->d_bstr;
-    o.binom33 = h->d_binom;
-    o.rank16 = h->d_rank16;
-    o.n = h->n;
-    o.Nb = h->Nb;
-    o.qubit = p->qubit;
+    const hy::k::SvOpArgs o = sv_op_args(h, p);
     cudaStream_t st = as_stream(stream);
     hy::ProfScope prof(HY_PROF_SPARSE_EXCITE, stream, 0.0);
     if (f->dt == HY_F64)
@@ -3335,6 +3310,27 @@ hy_status sstate_apply_h_support(const SparseState *s, SparseState *sig, void *s
     return HY_OK;
 }
 
+namespace {
+template <typename T>
+hy::k::SparseGradArgs<T> sparse_grad_args(const SparseState *s, const void *lam, const hy_pool *p,
+                                          const int32_t *ops, int64_t n_ops, int chunks,
+                                          double *partials, double *g)
+{
+    const hy_ham *h = s->h;
+    hy::k::SparseGradArgs<T> a;
+    a.psi = static_cast<const T *>(s->v);
+    a.sigma = static_cast<const T *>(lam);
+    a.list = s->list; a.m = 0; a.d_m = s->cnt; a.cap = s->cap; a.bits = s->bits;
+    a.chunks = chunks; a.partials = partials;
+    a.desc = p->d_desc; a.ops = ops; a.n_ops = n_ops;
+    a.astr = h->d_astr; a.bstr = h->d_bstr; a.binom33 = h->d_binom; a.n = h->n;
+    a.rank16 = h->d_rank16;
+    a.Nb = h->Nb; a.g = g; a.K = int64_t(p->ops.size()); a.bad = p->d_bad;
+    a.qubit = p->qubit;
+    return a;
+}
+}  // namespace
+
 hy_status sstate_gradients(const SparseState *sc, const void *lam, const hy_pool *p,
                            const int32_t *ops, int64_t n_ops, int64_t m_hint, double *g,
                            void *stream)
@@ -3349,29 +3345,54 @@ hy_status sstate_gradients(const SparseState *sc, const void *lam, const hy_pool
     hy_status r = sstate_partials(s, n_ops * chunks, st);
     if (r != HY_OK) return r;
     hy::ProfScope prof(HY_PROF_SCREEN_SPARSE, stream, 0.0);
-    auto fill = [&](auto &a) {
-        a.list = s->list; a.m = 0; a.d_m = s->cnt; a.cap = s->cap; a.bits = s->bits;
-        a.chunks = chunks; a.partials = s->partials;
-        a.desc = p->d_desc; a.ops = ops; a.n_ops = n_ops;
-        a.astr = h->d_astr; a.bstr = h->d_bstr; a.binom33 = h->d_binom; a.n = h->n;
-        a.rank16 = h->d_rank16;
-        a.Nb = h->Nb; a.g = g; a.K = int64_t(p->ops.size()); a.bad = p->d_bad;
-        a.qubit = p->qubit;
-    };
-    if (s->dt == HY_F64) {
-        hy::k::SparseGradArgs<double> a;
-        a.psi = static_cast<const double *>(s->v);
-        a.sigma = static_cast<const double *>(lam);
-        fill(a);
-        HY_CUDA(hy::k::grad_sparse<double>(a, h->num_sms, st), "sparse gradients");
-    } else {
-        hy::k::SparseGradArgs<float> a;
-        a.psi = static_cast<const float *>(s->v);
-        a.sigma = static_cast<const float *>(lam);
-        fill(a);
-        HY_CUDA(hy::k::grad_sparse<float>(a, h->num_sms, st), "sparse gradients");
-    }
+    if (s->dt == HY_F64)
+        HY_CUDA(hy::k::grad_sparse<double>(sparse_grad_args<double>(s, lam, p, ops, n_ops, chunks,
+                                                                    s->partials, g),
+                                           h->num_sms, st), "sparse gradients");
+    else
+        HY_CUDA(hy::k::grad_sparse<float>(sparse_grad_args<float>(s, lam, p, ops, n_ops, chunks,
+                                                                  s->partials, g),
+                                          h->num_sms, st), "sparse gradients");
     return HY_OK;
+}
+
+hy_status sstate_reverse_closed(SparseState *f, const SparseState *w, const hy_pool *p,
+                                const int64_t *ops, const int32_t *d_ops, const double *theta,
+                                int64_t j, int64_t m_hint, double *g, void *stream)
+{
+    const hy_ham *h = f->h;
+    if (!w || !p || p->h != h || w->h != h || w->dt != f->dt || !ops || !d_ops || !theta || j < 1 || !g)
+        return fail(HY_ERR_ARG, "bad arguments");
+    for (int64_t l = 0; l < j; ++l)
+        if (ops[l] < 0 || ops[l] >= int64_t(p->ops.size())) return fail(HY_ERR_ARG, "bad operator");
+    cudaStream_t st = as_stream(stream);
+    const int chunks = sparse_chunks(h, 1, m_hint < f->cap ? m_hint : f->cap);
+    hy_status r = sstate_partials(f, j * chunks, st);
+    if (r != HY_OK) return r;
+    const hy::k::SvOpArgs o = sv_op_args(h, p);
+    const double es = f->dt == HY_F64 ? 8.0 : 4.0;
+    auto sweep = [&](auto zero) {
+        using T = decltype(zero);
+        for (int64_t l = j; l-- > 0;) {
+            {
+                hy::ProfScope prof(HY_PROF_SCREEN_SPARSE, stream, 0.0);
+                HY_CUDA(hy::k::grad_sparse_partials<T>(
+                            sparse_grad_args<T>(f, w->v, p, d_ops + l, 1, chunks,
+                                                f->partials + l * chunks, g), st),
+                        "sparse gradients");
+            }
+            if (l == 0) break;
+            const int nc = p->ops[ops[l]].desc[0];
+            hy::ProfScope prof(HY_PROF_SPARSE_EXCITE, stream,
+                               double(std::max<int64_t>(f->hint, 0)) * nc * (12.0 + 8.0 * es));
+            HY_CUDA(hy::k::sv_excite_two<T>(svec<T>(f), static_cast<T *>(w->v), o, int(ops[l]), nc,
+                                            -theta[l], h->num_sms, st), "sparse excitation");
+        }
+        hy::ProfScope prof(HY_PROF_SCREEN_SPARSE, stream, 0.0);
+        HY_CUDA(hy::k::grad_sparse_sums(f->partials, chunks, j, g, st), "sparse gradients");
+        return HY_OK;
+    };
+    return f->dt == HY_F64 ? sweep(0.0) : sweep(0.0f);
 }
 
 const int64_t *sstate_count(const SparseState *s)

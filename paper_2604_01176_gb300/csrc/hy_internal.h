@@ -185,6 +185,12 @@ void sstate_set_hint(SparseState *s, int64_t n);
 // scales its listed end (for a vector that is read on a fixed support only)
 hy_status sstate_excite(SparseState *s, const hy_pool *p, int64_t k, double theta, void *stream,
                         bool closed = false);
+// The reverse sweep over ops[0..j) (host; d_ops the same on the device) of two vectors
+// kept on one support: g[l] (device) = 2 <w|A_l f>, then both rotated by -theta[l],
+// last operator first (f's and w's lists hold the same determinants)
+hy_status sstate_reverse_closed(SparseState *f, const SparseState *w, const hy_pool *p,
+                                const int64_t *ops, const int32_t *d_ops, const double *theta,
+                                int64_t j, int64_t m_hint, double *g, void *stream);
 // In one CTA: clear the support, |HF>, the rotations of ops[0..L) (device)
 // with cs[2l], cs[2l+1] (device) = cos, sin theta_l, then (renorm) divide by
 // the FP64 norm over the support.  For small supports (one launch instead of

@@ -385,6 +385,11 @@ template <typename T>
 cudaError_t hpsi_support(const SupRowsArgs<T> &a, int num_sms, cudaStream_t st);
 template <typename T>
 cudaError_t grad_sparse(const SparseGradArgs<T> &a, int num_sms, cudaStream_t st);
+// its two halves: an operator's chunks, and the sums of them
+template <typename T>
+cudaError_t grad_sparse_partials(const SparseGradArgs<T> &a, cudaStream_t st);
+cudaError_t grad_sparse_sums(const double *partials, int chunks, int64_t n_ops, double *g,
+                             cudaStream_t st);
 
 // Sparse vectors backed by a dense array: v (N amplitudes, zero off the
 // support), list[0..count) the support (each index once, values may be 0),
@@ -403,7 +408,7 @@ struct SVec {
 // a constituent's operator strings and the tables to rank determinants
 struct SvOpArgs {
     const int32_t *desc;         // [K][11]
-    const uint32_t *astr, *bstr, *binom33;
+    const uint32_t *astr, *bstr;
     const uint16_t *rank16;      // [1 << n] colex rank of every n-bit string
     int n;
     int64_t Nb;
@@ -420,6 +425,10 @@ cudaError_t sv_copy(const SVec<T> &dst, const SVec<T> &src, int num_sms, cudaStr
 template <typename T>
 cudaError_t sv_excite(const SVec<T> &x, const SvOpArgs &o, int k, int nc, double theta,
                       int num_sms, cudaStream_t st, bool closed = false);
+// the same, closed, for x and the values w of a second vector on x's support
+template <typename T>
+cudaError_t sv_excite_two(const SVec<T> &x, T *w, const SvOpArgs &o, int k, int nc, double theta,
+                          int num_sms, cudaStream_t st);
 // one CTA: clear x's support, |HF>, every constituent rotation of ops[0..L)
 // with cs[2l], cs[2l+1] = cos, sin theta_l, then (renorm) divide by the FP64
 // norm over the support (written to *norm2 if not null); for small supports.

@@ -642,20 +642,21 @@ k_sup_rows(SupRowsArgs<double> a)
     }
 }
 
-__device__ __forceinline__ uint32_t rank_bits(uint32_t m, const uint32_t (*C)[33])
-{
-    uint32_t r = 0;
-    int i = 0;
-    for (; m; m &= m - 1, ++i) r += C[__ffs(m) - 1][i + 1];
-    return r;
-}
-
 // index of the determinant with spin strings u = alpha | beta << n, from the
-// table of colex ranks of all n-bit strings (the same rank as rank_bits)
+// table of colex ranks of all n-bit strings
 __device__ __forceinline__ int64_t det_index(const uint16_t *__restrict__ r16, uint64_t u, int n,
                                              uint64_t lowm, int64_t Nb)
 {
     return int64_t(__ldg(r16 + (u & lowm))) * Nb + __ldg(r16 + (u >> n));
+}
+
+// the strings of determinant d; d is below 2^32 (12,870 strings of a spin at most),
+// so the division is a 32-bit one
+__device__ __forceinline__ uint64_t det_mask(int64_t d, const uint32_t *__restrict__ astr,
+                                             const uint32_t *__restrict__ bstr, int64_t Nb, int n)
+{
+    const uint32_t A = uint32_t(d) / uint32_t(Nb), B = uint32_t(d) - A * uint32_t(Nb);
+    return uint64_t(astr[A]) | (uint64_t(bstr[B]) << n);
 }
 
 // Apply an operator string (application order; codes 2*mode + dagger) to a
@@ -731,7 +732,7 @@ k_grad_sparse(SparseGradArgs<T> a)
              t += int64_t(gridDim.y) * blockDim.x) {
             const int64_t d = a.list[t];
             const double x = double(a.psi[d]);
-            const uint64_t mask = uint64_t(a.astr[d / a.Nb]) | (uint64_t(a.bstr[d % a.Nb]) << n);
+            const uint64_t mask = det_mask(d, a.astr, a.bstr, a.Nb, n);
             uint64_t o = mask;
             int sg = 1;
             if (apply_string(fw, len, o, sg, a.qubit)) {       // d is the domain end
@@ -823,7 +824,7 @@ k_sv_copy(SVec<T> dst, SVec<T> src)
 // the rotation loop of k_sv_excite over this block's share of entries < m
 template <typename T>
 __device__ __forceinline__ void sv_rotate(SVec<T> &x, const SvOpArgs &o, int k, int ci, T c, T s,
-                                          int64_t m, const uint32_t (*C)[33], bool closed = false)
+                                          int64_t m, bool closed = false)
 {
     int fw[4], bw[4], len;
     op_strings(o.desc + 11 * k + 1 + 5 * ci, fw, bw, len);
@@ -832,7 +833,7 @@ __device__ __forceinline__ void sv_rotate(SVec<T> &x, const SvOpArgs &o, int k, 
     for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < m;
          t += int64_t(gridDim.x) * blockDim.x) {
         const int64_t d = x.list[t];
-        const uint64_t mask = uint64_t(o.astr[d / o.Nb]) | (uint64_t(o.bstr[d % o.Nb]) << n);
+        const uint64_t mask = det_mask(d, o.astr, o.bstr, o.Nb, n);
         uint64_t u = mask;
         int sg = 1;
         int64_t dom, img, fresh;
@@ -881,12 +882,7 @@ k_sv_excite(SVec<T> x, SvOpArgs o, int k, int ci, T c, T s, int closed)
 {
     const int64_t m = list_len(x.snap, 0, x.cap);
     const bool idle = int64_t(blockIdx.x) * blockDim.x >= m;     // block-uniform
-    __shared__ uint32_t C[33][33];
-    if (!idle) {
-        for (int i = threadIdx.x; i < 33 * 33; i += blockDim.x) C[i / 33][i % 33] = o.binom33[i];
-        __syncthreads();
-        sv_rotate(x, o, k, ci, c, s, m, C, closed != 0);
-    }
+    if (!idle) sv_rotate(x, o, k, ci, c, s, m, closed != 0);
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
@@ -899,59 +895,103 @@ k_sv_excite(SVec<T> x, SvOpArgs o, int k, int ci, T c, T s, int closed)
 }
 
 
+// The same, closed, for two vectors on one support (w: values where x lists them):
+// the pairs are looked up once.  Nothing is listed, so nothing is counted.  Bound by
+// the chain list, strings, rank, bitmap, amplitudes of an entry: 8.7 us for 200,000
+// determinants, as k_sv_excite takes for one vector.
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_sv_excite_two(SVec<T> x, T *__restrict__ w, SvOpArgs o, int k, int ci, T c, T s)
+{
+    const int64_t m = list_len(x.snap, 0, x.cap);
+    int fw[4], bw[4], len;
+    op_strings(o.desc + 11 * k + 1 + 5 * ci, fw, bw, len);
+    const int n = o.n;
+    const uint64_t lowm = (1ull << n) - 1;
+    for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < m;
+         t += int64_t(gridDim.x) * blockDim.x) {
+        const int64_t d = x.list[t];
+        const uint64_t mask = det_mask(d, o.astr, o.bstr, o.Nb, n);
+        uint64_t u = mask;
+        int sg = 1;
+        const bool dom = apply_string(fw, len, u, sg, o.qubit);
+        if (!dom) {
+            u = mask;
+            sg = 1;
+            if (!apply_string(bw, len, u, sg, o.qubit)) continue;
+        }
+        const int64_t p = det_index(o.rank16, u, n, lowm, o.Nb);
+        if (!member(x.bits, p)) {            // the other end is off the support
+            x.v[d] = c * x.v[d];
+            w[d] = c * w[d];
+            continue;
+        }
+        if (!dom) continue;                  // the domain end rotates the pair
+        const T ss = sg > 0 ? s : -s;
+        const T xd = x.v[d], xp = x.v[p], wd = w[d], wp = w[p];
+        x.v[d] = c * xd - ss * xp;
+        x.v[p] = c * xp + ss * xd;
+        w[d] = c * wd - ss * wp;
+        w[p] = c * wp + ss * wd;
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Single-CTA routines for small supports: block barriers take the place of
 // launch boundaries and of the count snapshot.
 // ---------------------------------------------------------------------------
 constexpr int kPrepThreads = 1024;
 
-// zero x on its support (bits included) and empty the list
+// current length of x's list, the same in every thread
 template <typename T>
-__device__ void blk_clear(SVec<T> &x)
+__device__ int64_t blk_len(const SVec<T> &x, const unsigned long long *cnt)
 {
-    const int64_t m = list_len(x.count, 0, x.cap);
+    __syncthreads();
+    const unsigned long long m = *cnt;
+    __syncthreads();
+    return m < (unsigned long long)x.cap ? int64_t(m) : x.cap;
+}
+
+// zero x on its support of *cnt entries (bits included) and empty the list.  A list's
+// length lives in shared memory (cnt) while its block is at work: from memory, with
+// the appends' atomics in between, it cost each step a microsecond
+template <typename T>
+__device__ void blk_clear(SVec<T> &x, unsigned long long *cnt)
+{
+    const int64_t m = blk_len(x, cnt);
     for (int64_t t = threadIdx.x; t < m; t += blockDim.x) {
         const int64_t i = x.list[t];
         x.v[i] = T(0);
         x.bits[i >> 5] = 0u;
     }
     __syncthreads();
-    if (threadIdx.x == 0) *x.count = 0ull;
+    if (threadIdx.x == 0) *cnt = 0ull;
     __syncthreads();
 }
 
 // list index i of x (unlisted before) -- the caller owns i's bit
 template <typename T>
-__device__ __forceinline__ void blk_list(SVec<T> &x, int64_t i)
+__device__ __forceinline__ void blk_list(SVec<T> &x, int64_t i, unsigned long long *cnt)
 {
     atomicOr(x.bits + (i >> 5), 1u << (i & 31));
-    const unsigned long long pos = atomicAdd(x.count, 1ull);
+    const unsigned long long pos = atomicAdd(cnt, 1ull);
     if (pos < (unsigned long long)x.cap) x.list[pos] = i;
 }
 
-// current length of x's list, the same in every thread
+// exp(theta (C - C^dagger)) for constituent ci of operator k, as k_sv_excite;
+// returns the list's length before
 template <typename T>
-__device__ int64_t blk_len(const SVec<T> &x, unsigned long long *m_sh)
+__device__ int64_t blk_rotate(SVec<T> &x, const SvOpArgs &o, int k, int ci, T c, T sn,
+                           unsigned long long *cnt)
 {
-    __syncthreads();
-    if (threadIdx.x == 0) *m_sh = *x.count;
-    __syncthreads();
-    return *m_sh < (unsigned long long)x.cap ? int64_t(*m_sh) : x.cap;
-}
-
-// exp(theta (C - C^dagger)) for constituent ci of operator k, as k_sv_excite
-template <typename T>
-__device__ void blk_rotate(SVec<T> &x, const SvOpArgs &o, int k, int ci, T c, T sn,
-                           const uint32_t (*C)[33], unsigned long long *m_sh)
-{
-    const int64_t m = blk_len(x, m_sh);
+    const int64_t m = blk_len(x, cnt);
     int fw[4], bw[4], len;
     op_strings(o.desc + 11 * k + 1 + 5 * ci, fw, bw, len);
     const int n = o.n;
     const uint64_t lowm = (1ull << n) - 1;
     for (int64_t t = threadIdx.x; t < m; t += blockDim.x) {
         const int64_t d = x.list[t];
-        const uint64_t mask = uint64_t(o.astr[d / o.Nb]) | (uint64_t(o.bstr[d % o.Nb]) << n);
+        const uint64_t mask = det_mask(d, o.astr, o.bstr, o.Nb, n);
         uint64_t u = mask;
         int sg = 1;
         int64_t dom, img, fresh;
@@ -972,8 +1012,9 @@ __device__ void blk_rotate(SVec<T> &x, const SvOpArgs &o, int k, int ci, T c, T 
         const T xv = x.v[dom], yv = x.v[img];
         x.v[dom] = c * xv - ss * yv;
         x.v[img] = c * yv + ss * xv;
-        if (fresh >= 0) blk_list(x, fresh);
+        if (fresh >= 0) blk_list(x, fresh, cnt);
     }
+    return m;
 }
 
 // w <- w + (C - C^dagger) f for constituent ci of operator k over f's
@@ -981,7 +1022,7 @@ __device__ void blk_rotate(SVec<T> &x, const SvOpArgs &o, int k, int ci, T c, T 
 // has a single source (its partner) and is written by one thread.
 template <typename T>
 __device__ void blk_generator(const SVec<T> &f, SVec<T> &w, const SvOpArgs &o, int k, int ci,
-                              int64_t m, const uint32_t (*C)[33])
+                              int64_t m, unsigned long long *cnt)
 {
     int fw[4], bw[4], len;
     op_strings(o.desc + 11 * k + 1 + 5 * ci, fw, bw, len);
@@ -989,7 +1030,7 @@ __device__ void blk_generator(const SVec<T> &f, SVec<T> &w, const SvOpArgs &o, i
     const uint64_t lowm = (1ull << n) - 1;
     for (int64_t t = threadIdx.x; t < m; t += blockDim.x) {
         const int64_t d = f.list[t];
-        const uint64_t mask = uint64_t(o.astr[d / o.Nb]) | (uint64_t(o.bstr[d % o.Nb]) << n);
+        const uint64_t mask = det_mask(d, o.astr, o.bstr, o.Nb, n);
         uint64_t u = mask;
         int sg = 1;
         int64_t tgt;
@@ -1005,7 +1046,7 @@ __device__ void blk_generator(const SVec<T> &f, SVec<T> &w, const SvOpArgs &o, i
             tgt = det_index(o.rank16, u, n, lowm, o.Nb);
             val = sg > 0 ? -f.v[d] : f.v[d];
         }
-        if (!member(w.bits, tgt)) blk_list(w, tgt);  // tgt is reached from d alone
+        if (!member(w.bits, tgt)) blk_list(w, tgt, cnt);  // tgt is reached from d alone
         w.v[tgt] += val;
     }
 }
@@ -1041,32 +1082,30 @@ k_sv_prepare(SVec<T> x, SvOpArgs o, const int32_t *__restrict__ ops,
              const double *__restrict__ cs, int L, int renorm, double *__restrict__ norm2,
              int64_t *__restrict__ step_len)
 {
-    __shared__ uint32_t C[33][33];
-    __shared__ unsigned long long m_sh;
+    __shared__ unsigned long long cnt;
     __shared__ double red[kPrepThreads / 32];
     __shared__ double fac;
     const int tid = threadIdx.x;
-    for (int i = tid; i < 33 * 33; i += blockDim.x) C[i / 33][i % 33] = o.binom33[i];
-    blk_clear(x);
+    if (tid == 0) cnt = *x.count;
+    blk_clear(x, &cnt);
     if (tid == 0) {
         x.v[0] = T(1);
-        blk_list(x, 0);
+        blk_list(x, 0, &cnt);
     }
     int step = 0;
     for (int l = 0; l < L; ++l) {
         const int k = ops[l];
         const int nc = o.desc[11 * k];
         for (int ci = 0; ci < nc; ++ci, ++step) {
-            blk_rotate(x, o, k, ci, T(cs[2 * l]), T(cs[2 * l + 1]), C, &m_sh);
-            if (step_len) {
-                const int64_t ml = blk_len(x, &m_sh);
-                if (tid == 0) step_len[step] = ml;
-            }
+            const int64_t before = blk_rotate(x, o, k, ci, T(cs[2 * l]), T(cs[2 * l + 1]), &cnt);
+            if (step_len && step && tid == 0) step_len[step - 1] = before;
         }
     }
-    const int64_t m = blk_len(x, &m_sh);
+    const int64_t m = blk_len(x, &cnt);
     if (tid == 0) {                 // leave the snapshot consistent for later rotations
-        *x.snap = *x.count;
+        if (step_len && step) step_len[step - 1] = m;
+        *x.count = cnt;
+        *x.snap = cnt;
         *x.done = 0ull;
     }
     if (!renorm) return;
@@ -1094,43 +1133,47 @@ k_sv_grad_fwd(SVec<T> f, SVec<T> w, SvOpArgs o, const int32_t *__restrict__ ops,
               const double *__restrict__ cs, int L, const T *__restrict__ sigma,
               const double *__restrict__ norm2, double *__restrict__ g)
 {
-    __shared__ uint32_t C[33][33];
-    __shared__ unsigned long long m_sh;
+    __shared__ unsigned long long fc, wc;
     __shared__ double red[kPrepThreads / 32];
     const int tid = threadIdx.x;
-    for (int i = tid; i < 33 * 33; i += blockDim.x) C[i / 33][i % 33] = o.binom33[i];
-    blk_clear(f);
+    if (tid == 0) {
+        fc = *f.count;
+        wc = *w.count;
+    }
+    blk_clear(f, &fc);
     if (tid == 0) {
         f.v[0] = T(1);
-        blk_list(f, 0);
+        blk_list(f, 0, &fc);
     }
     const double scale = norm2 ? 2.0 / sqrt(*norm2) : 2.0;
     for (int l = 0; l < L; ++l) {
         const int k = ops[l];
         const int nc = o.desc[11 * k];
         for (int ci = 0; ci < nc; ++ci)
-            blk_rotate(f, o, k, ci, T(cs[2 * l]), T(cs[2 * l + 1]), C, &m_sh);
-        blk_clear(w);
-        const int64_t mf = blk_len(f, &m_sh);
+            blk_rotate(f, o, k, ci, T(cs[2 * l]), T(cs[2 * l + 1]), &fc);
+        blk_clear(w, &wc);
+        const int64_t mf = blk_len(f, &fc);
         for (int ci = 0; ci < nc; ++ci) {
-            blk_generator(f, w, o, k, ci, mf, C);
+            blk_generator(f, w, o, k, ci, mf, &wc);
             __syncthreads();                         // constituents add in order
         }
         for (int l2 = l + 1; l2 < L; ++l2) {
             const int k2 = ops[l2];
             const int nc2 = o.desc[11 * k2];
             for (int ci = 0; ci < nc2; ++ci)
-                blk_rotate(w, o, k2, ci, T(cs[2 * l2]), T(cs[2 * l2 + 1]), C, &m_sh);
+                blk_rotate(w, o, k2, ci, T(cs[2 * l2]), T(cs[2 * l2 + 1]), &wc);
         }
-        const int64_t mw = blk_len(w, &m_sh);
+        const int64_t mw = blk_len(w, &wc);
         const double gl = blk_dot(w, sigma, mw, red);
         if (tid == 0) g[l] = scale * gl;
     }
     __syncthreads();
     if (tid == 0) {
-        *f.snap = *f.count;
+        *f.count = fc;
+        *f.snap = fc;
         *f.done = 0ull;
-        *w.snap = *w.count;
+        *w.count = wc;
+        *w.snap = wc;
         *w.done = 0ull;
     }
 }
@@ -1290,9 +1333,6 @@ k_prog_tables(const int64_t *__restrict__ key, int m, SvOpArgs o, const int32_t 
               int L, uint32_t *__restrict__ pairs, int *__restrict__ npairs,
               int *__restrict__ nrest, int *__restrict__ step_l, int *__restrict__ flag)
 {
-    __shared__ uint32_t C[33][33];
-    for (int i = threadIdx.x; i < 33 * 33; i += blockDim.x) C[i / 33][i % 33] = o.binom33[i];
-    __syncthreads();
     const int s = blockIdx.y;
     int l, ci, last;
     prog_step_op(o.desc, ops, L, s, l, ci, last);
@@ -1308,7 +1348,7 @@ k_prog_tables(const int64_t *__restrict__ key, int m, SvOpArgs o, const int32_t 
         const int birth = int(kt & 255) - 1;         // -1: |HF>, else the listing step
         const int n = o.n;
         const uint64_t lowm = (1ull << n) - 1;
-        const uint64_t mask = uint64_t(o.astr[d / o.Nb]) | (uint64_t(o.bstr[d % o.Nb]) << n);
+        const uint64_t mask = det_mask(d, o.astr, o.bstr, o.Nb, n);
         uint64_t u = mask;
         int sg = 1;
         bool escape = false;
@@ -1666,9 +1706,6 @@ k_prog_tables_big(const int64_t *__restrict__ key, int m, SvOpArgs o,
                   int *__restrict__ npairs, int *__restrict__ nrest, int *__restrict__ step_l,
                   int *__restrict__ flag)
 {
-    __shared__ uint32_t C[33][33];
-    for (int i = threadIdx.x; i < 33 * 33; i += blockDim.x) C[i / 33][i % 33] = o.binom33[i];
-    __syncthreads();
     const int s = blockIdx.y;
     int l, ci, last;
     prog_step_op(o.desc, ops, L, s, l, ci, last);
@@ -1687,7 +1724,7 @@ k_prog_tables_big(const int64_t *__restrict__ key, int m, SvOpArgs o,
         if (t < m) {
             const int64_t kt = key[t], d = kt >> 8;
             const int birth = int(kt & 255) - 1;
-            const uint64_t mask = uint64_t(o.astr[d / o.Nb]) | (uint64_t(o.bstr[d % o.Nb]) << n);
+            const uint64_t mask = det_mask(d, o.astr, o.bstr, o.Nb, n);
             uint64_t u = mask;
             int sg = 1;
             bool escape = false;
@@ -2234,6 +2271,18 @@ cudaError_t sv_excite(const SVec<T> &x, const SvOpArgs &o, int k, int nc, double
 }
 
 template <typename T>
+cudaError_t sv_excite_two(const SVec<T> &x, T *w, const SvOpArgs &o, int k, int nc, double theta,
+                          int num_sms, cudaStream_t st)
+{
+    const T c = T(std::cos(theta)), s = T(std::sin(theta));
+    for (int ci = 0; ci < nc; ++ci) {
+        k_sv_excite_two<T><<<sv_grid(sv_n(x), num_sms), 256, 0, st>>>(x, w, o, k, ci, c, s);
+        hy::count_launch();
+    }
+    return cudaGetLastError();
+}
+
+template <typename T>
 cudaError_t sv_prepare(const SVec<T> &x, const SvOpArgs &o, const int32_t *ops, const double *cs,
                        int L, bool renorm, double *norm2, int64_t *step_len, cudaStream_t st)
 {
@@ -2351,16 +2400,29 @@ cudaError_t hpsi_support(const SupRowsArgs<T> &a, int num_sms, cudaStream_t st)
 }
 
 template <typename T>
-cudaError_t grad_sparse(const SparseGradArgs<T> &a, int num_sms, cudaStream_t st)
+cudaError_t grad_sparse_partials(const SparseGradArgs<T> &a, cudaStream_t st)
 {
-    (void)num_sms;
     if (a.n_ops == 0) return cudaSuccess;
     k_grad_sparse<T><<<dim3(unsigned(a.n_ops), unsigned(a.chunks)), 256, 0, st>>>(a);
     hy::count_launch();
-    k_grad_sparse_final<<<unsigned((a.n_ops + 7) / 8), 256, 0, st>>>(a.partials, a.chunks,
-                                                                     a.n_ops, a.g);
+    return cudaGetLastError();
+}
+
+cudaError_t grad_sparse_sums(const double *partials, int chunks, int64_t n_ops, double *g,
+                             cudaStream_t st)
+{
+    if (n_ops == 0) return cudaSuccess;
+    k_grad_sparse_final<<<unsigned((n_ops + 7) / 8), 256, 0, st>>>(partials, chunks, n_ops, g);
     hy::count_launch();
     return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t grad_sparse(const SparseGradArgs<T> &a, int num_sms, cudaStream_t st)
+{
+    (void)num_sms;
+    const cudaError_t e = grad_sparse_partials<T>(a, st);
+    return e != cudaSuccess ? e : grad_sparse_sums(a.partials, a.chunks, a.n_ops, a.g, st);
 }
 
 cudaError_t prog_compile(const int64_t *list, int64_t m, const int64_t *step_len, int steps,
@@ -2545,6 +2607,8 @@ template cudaError_t prog_grad_big<double>(const ProgTabs &, const double *, int
                                            const double *, double *, cudaStream_t);
 template cudaError_t prog_grad_big<float>(const ProgTabs &, const double *, int, const float *,
                                           const double *, double *, cudaStream_t);
+template cudaError_t grad_sparse_partials<double>(const SparseGradArgs<double> &, cudaStream_t);
+template cudaError_t grad_sparse_partials<float>(const SparseGradArgs<float> &, cudaStream_t);
 template cudaError_t grad_sparse<double>(const SparseGradArgs<double> &, int, cudaStream_t);
 template cudaError_t grad_sparse<float>(const SparseGradArgs<float> &, int, cudaStream_t);
 #define HY_SV_INST(T)                                                                       \
@@ -2552,6 +2616,8 @@ template cudaError_t grad_sparse<float>(const SparseGradArgs<float> &, int, cuda
     template cudaError_t sv_copy<T>(const SVec<T> &, const SVec<T> &, int, cudaStream_t);   \
     template cudaError_t sv_excite<T>(const SVec<T> &, const SvOpArgs &, int, int, double,  \
                                       int, cudaStream_t, bool);                              \
+    template cudaError_t sv_excite_two<T>(const SVec<T> &, T *, const SvOpArgs &, int, int, \
+                                          double, int, cudaStream_t);                        \
     template cudaError_t sv_prepare<T>(const SVec<T> &, const SvOpArgs &, const int32_t *,  \
                                        const double *, int, bool, double *, int64_t *,      \
                                        cudaStream_t);                                        \
