@@ -119,7 +119,7 @@ struct hy_ham {
     // off-diagonal same-spin tables as tensor-core operands (hy_same.cu; pack
     // null: the CSR kernel runs), by spin, and the CTA pairs that run at once
     hy::k::SameArgs same[2] = {};
-    int same_pairs = 0;
+    int same_pairs = -1;            // not tried yet: made by the first float sweep
     double *d_V64 = nullptr;
     float *d_V32 = nullptr;
     double *d_h1 = nullptr, *d_eri = nullptr;   // integrals (ranker features)
@@ -408,6 +408,73 @@ hy::k::Rows64Mol rows64_mol(const hy_ham *h, int cols)
     return r;
 }
 
+// the float same-spin table of one spin as tensor-core operands; without the
+// memory for it the CSR kernel stays in use
+hy_status pack_same_spin(hy_ham *h, int spin)
+{
+    const int64_t N = spin == 0 ? h->Na : h->Nb;
+    const DevCsr<float> &M = spin == 0 ? h->Ma32 : h->Mb32;
+    const int nrb = hy::k::same_row_blocks(N), nch = hy::k::same_chunks(N);
+    DevArena tmp, ar;
+    uint32_t *place = nullptr;
+    int32_t *count = nullptr;
+    std::vector<int32_t> cnt(size_t(nrb), 0);
+    cudaError_t e = tmp.alloc(&place, size_t(nrb) * nch, true);
+    if (e == cudaSuccess) e = tmp.alloc(&count, size_t(nrb));
+    if (e == cudaSuccess) e = hy::k::same_used(M.ptr, M.col, N, place, count, nullptr);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(cnt.data(), count, cnt.size() * sizeof(int32_t), cudaMemcpyDeviceToHost);
+    std::vector<int64_t> base(size_t(nrb) + 1, 0);
+    for (int i = 0; i < nrb; ++i) base[i + 1] = base[i] + cnt[i];
+    int64_t *d_base = nullptr;
+    uint16_t *list = nullptr;
+    unsigned char *pack = nullptr;
+    float *diag = nullptr;
+    if (e == cudaSuccess) e = ar.upload(&d_base, base.data(), base.size());
+    if (e == cudaSuccess) e = ar.alloc(&list, size_t(base[nrb]));
+    if (e == cudaSuccess) e = ar.alloc(&diag, size_t(N), true);
+    if (e == cudaSuccess) e = ar.alloc(&pack, size_t(base[nrb]) * hy::k::same_block_bytes(), true);
+    if (e == cudaSuccess && pack)
+        e = hy::k::same_fill(M.ptr, M.col, M.val, N, place, d_base, list, pack, diag, nullptr);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    tmp.release();
+    if (e != cudaSuccess || !pack) {
+        ar.release();
+        if (e != cudaSuccess && e != cudaErrorMemoryAllocation) return cuda_fail(e, "same-spin operands");
+        cudaGetLastError();
+        return HY_OK;
+    }
+    h->arena.ptrs.insert(h->arena.ptrs.end(), ar.ptrs.begin(), ar.ptrs.end());
+    h->arena.uploaded += ar.uploaded;
+    hy::k::SameArgs &a = h->same[spin];
+    a.N = N;
+    a.pack = pack;
+    a.base = d_base;
+    a.list = list;
+    a.diag = diag;
+    return HY_OK;
+}
+
+// both spins' operands, where the rule of hy_kernels.cuh asks for them: with a
+// Hamiltonian's first float sweep (double users never pay for them, 2 ms and 2 GB at
+// 12,870 strings); not while a stream is being captured
+hy_status pack_same(hy_ham *h, cudaStream_t st)
+{
+    if (std::min(h->Na, h->Nb) < hy::k::kSameStrings || !h->d_status) {
+        h->same_pairs = 0;
+        return HY_OK;
+    }
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return HY_OK;
+    }
+    h->same_pairs = hy::k::same_pairs();
+    hy_status s = HY_OK;
+    for (int spin = 0; spin < 2 && s == HY_OK && h->same_pairs > 0; ++spin) s = pack_same_spin(h, spin);
+    return s;
+}
+
 // sigma rows [r0, r1) (alpha strings) of H psi; sigma holds those rows only.
 // Every output element is formed by the same arithmetic in the same order
 // whatever the range, so shards concatenate to the full sigma bit for bit.
@@ -444,6 +511,10 @@ hy_status apply_h_t(hy_ham *h, const T *psi, T *sigma, cudaStream_t st, int64_t 
         ? size_t(h->Na) * size_t(h->A.nex + 1) * size_t(Nbp) * sizeof(float) : 0;
     // the tensor-core same-spin part takes the same place before it
     size_t xbytes = 0;
+    if (sizeof(T) == sizeof(float) && h->same_pairs < 0 && h->cpl_impl != 1) {
+        hy_status s = pack_same(h, st);
+        if (s != HY_OK) return s;
+    }
     if (sizeof(T) == sizeof(float) && h->same[0].pack && h->same[1].pack && h->cpl_impl != 1 && h->d_status)
         xbytes = std::max(hy::k::same_x_bytes(h->Na, h->Nb), hy::k::same_x_bytes(h->Nb, nr));
     bool dense = false, same = false;
@@ -1016,53 +1087,6 @@ hy_status fold_same_spin(hy_ham *h)
     return HY_OK;
 }
 
-// the float same-spin table of one spin as tensor-core operands; without the
-// memory for it the CSR kernel stays in use
-hy_status pack_same_spin(hy_ham *h, int spin)
-{
-    const int64_t N = spin == 0 ? h->Na : h->Nb;
-    const DevCsr<float> &M = spin == 0 ? h->Ma32 : h->Mb32;
-    const int nrb = hy::k::same_row_blocks(N), nch = hy::k::same_chunks(N);
-    DevArena tmp, ar;
-    uint32_t *place = nullptr;
-    int32_t *count = nullptr;
-    std::vector<int32_t> cnt(size_t(nrb), 0);
-    cudaError_t e = tmp.alloc(&place, size_t(nrb) * nch, true);
-    if (e == cudaSuccess) e = tmp.alloc(&count, size_t(nrb));
-    if (e == cudaSuccess) e = hy::k::same_used(M.ptr, M.col, N, place, count, nullptr);
-    if (e == cudaSuccess)
-        e = cudaMemcpy(cnt.data(), count, cnt.size() * sizeof(int32_t), cudaMemcpyDeviceToHost);
-    std::vector<int64_t> base(size_t(nrb) + 1, 0);
-    for (int i = 0; i < nrb; ++i) base[i + 1] = base[i] + cnt[i];
-    int64_t *d_base = nullptr;
-    uint16_t *list = nullptr;
-    unsigned char *pack = nullptr;
-    float *diag = nullptr;
-    if (e == cudaSuccess) e = ar.upload(&d_base, base.data(), base.size());
-    if (e == cudaSuccess) e = ar.alloc(&list, size_t(base[nrb]));
-    if (e == cudaSuccess) e = ar.alloc(&diag, size_t(N), true);
-    if (e == cudaSuccess) e = ar.alloc(&pack, size_t(base[nrb]) * hy::k::same_block_bytes(), true);
-    if (e == cudaSuccess && pack)
-        e = hy::k::same_fill(M.ptr, M.col, M.val, N, place, d_base, list, pack, diag, nullptr);
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    tmp.release();
-    if (e != cudaSuccess || !pack) {
-        ar.release();
-        if (e != cudaSuccess && e != cudaErrorMemoryAllocation) return cuda_fail(e, "same-spin operands");
-        cudaGetLastError();
-        return HY_OK;
-    }
-    h->arena.ptrs.insert(h->arena.ptrs.end(), ar.ptrs.begin(), ar.ptrs.end());
-    h->arena.uploaded += ar.uploaded;
-    hy::k::SameArgs &a = h->same[spin];
-    a.N = N;
-    a.pack = pack;
-    a.base = d_base;
-    a.list = list;
-    a.diag = diag;
-    return HY_OK;
-}
-
 // host copies of the same-spin tables, for host consumers (the explicit-H
 // builder); copied once from the device
 hy_status ensure_host_csr(hy_ham *h)
@@ -1169,10 +1193,6 @@ hy_status finish_ham(hy_ham *h, hy_ham **out)
                                   h->num_sms, nullptr), "coupling tables");
     }
     if (s == HY_OK) s = fold_same_spin(h);
-    if (s == HY_OK && std::min(h->Na, h->Nb) >= hy::k::kSameStrings) {
-        h->same_pairs = hy::k::same_pairs();
-        for (int spin = 0; spin < 2 && s == HY_OK && h->same_pairs > 0; ++spin) s = pack_same_spin(h, spin);
-    }
     if (s != HY_OK) {
         std::string msg = g_err;
         hy_ham_destroy(h);

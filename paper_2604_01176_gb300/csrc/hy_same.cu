@@ -12,7 +12,7 @@
 // still ends sooner.
 //
 // Both factors lie in memory as MMA operands, hi and lo: M's off-diagonal part once
-// per Hamiltonian (same_used, same_fill: 256 rows by 32 columns that hold anything),
+// per Hamiltonian, with its first float sweep (same_used, same_fill: 256 rows by 32 columns that hold anything),
 // X per call (k_same_x, from either layout of psi, so the beta side needs no
 // transposed copy).  A pair of CTAs (cta_group::2) multiplies 256 columns of X (its
 // M side, so that a lane of tensor memory is a column and rows of Y are written

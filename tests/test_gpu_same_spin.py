@@ -58,3 +58,21 @@ def test_waits_run_out_and_are_reported():
         ham.apply_h(psi)
     assert ei.value.status == 4 and "timed out" in str(ei.value)
     assert torch.equal(ham.apply_h(psi), good)
+
+
+def test_captured_sweep_replays():
+    """A sweep captured after a Hamiltonian's first float one (which makes the
+    operands) replays to the same bits on new amplitudes."""
+    hy, ham, psi = _ham((12, 6, 5))
+    out = torch.empty_like(psi)
+    ham.apply_h(psi, out=out)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        ham.apply_h(psi, out=out)
+    new = torch.from_numpy(synth.random_state(ham.n_det, 10)).cuda().float()
+    ref = ham.apply_h(new)
+    psi.copy_(new)
+    out.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, ref)
