@@ -3300,26 +3300,32 @@ hy_status sstate_apply_h_support(const SparseState *s, SparseState *sig, void *s
         a.flagB = sig->flags + h->Na;
         a.blist = sig->blist;
         a.ctr = sig->ctr;
+        a.first = nullptr;
     };
     if (s->dt == HY_F64) {
         hy::k::SupRowsArgs<double> a;
         a.s = sparse_args<double>(h, s->v, sigma, sig->list, 0);
         run(a);
         // the tables lie one behind the other, the widest first
-        const size_t nb = size_t(h->Nb), nn = size_t(h->n) * h->n;
+        const size_t nb = size_t(h->Nb), na = size_t(h->Na), nn = size_t(h->n) * h->n;
         const size_t nnz = nb * size_t(hy::k::fold_candidates(h->n, h->nb));
+        const size_t tasks = size_t(hy::k::sup_tasks(sig->cap, h->Na));
         if (!sig->sup_tables) {
             const cudaError_t e =
-                cudaMalloc(&sig->sup_tables, (nnz + nn * nb) * 8 + (64 + 3) * nb * 4 + nnz * 2);
+                cudaMalloc(&sig->sup_tables, tasks * sizeof(int4) + (nnz + nn * nb) * 8 +
+                                                 ((64 + 3) * nb + 2 * na) * 4 + nnz * 2);
             if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(support rows)");
         }
-        a.mval = static_cast<double *>(sig->sup_tables);
+        a.tasks = static_cast<int4 *>(sig->sup_tables);
+        a.mval = reinterpret_cast<double *>(a.tasks + tasks);
         a.dbeta = a.mval + nnz;
         a.fex = reinterpret_cast<uint32_t *>(a.dbeta + nn * nb);
         a.number = reinterpret_cast<int32_t *>(a.fex + 64 * nb);
         a.nfex = a.number + nb;
         a.nm = a.nfex + nb;
-        a.mcol = reinterpret_cast<uint16_t *>(a.nm + nb);
+        a.first = a.nm + nb;
+        a.alist = a.first + na;
+        a.mcol = reinterpret_cast<uint16_t *>(a.alist + na);
         HY_CUDA(hy::k::hpsi_support<double>(a, h->num_sms, st), "support H psi");
     } else {
         hy::k::SupRowsArgs<float> a;

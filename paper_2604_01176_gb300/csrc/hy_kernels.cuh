@@ -354,6 +354,8 @@ cudaError_t hpsi_scatter(const SparseArgs<T> &a, int num_sms, cudaStream_t st);
 // the set bits of a membership bitmap of `words` words as a list in
 // increasing order (at most cap written; cnt[0] = cnt[1] = the number of set
 // bits, cnt[2] = 0); blk: scratch of bits_compact_blocks(words) int64
+// tasks of k_sup_rows for a list of at most cap rows
+inline int64_t sup_tasks(int64_t cap, int64_t Na) { return cap / 256 + Na; }
 inline int64_t bits_compact_blocks(int64_t words) { return (words + 2047) / 2048; }
 cudaError_t bits_compact(const uint32_t *bits, int64_t words, int64_t *list, int64_t cap,
                          unsigned long long *cnt, int64_t *blk, cudaStream_t st);
@@ -374,8 +376,12 @@ struct SupRowsArgs {
     uint8_t *flagA, *flagB;
     int32_t *blist;
     unsigned long long *ctr;
-    // double only: by beta string or its number in S (number: Nb, nfex, nm: Nb;
-    // fex: 64 Nb; mcol, mval: Nb times M_beta's longest row; dbeta: n^2 Nb)
+    // double only (else null): by beta string or its number in S (number: Nb, nfex, nm:
+    // Nb; fex: 64 Nb; mcol, mval: Nb times M_beta's longest row; dbeta: n^2 Nb), by
+    // alpha string (first, alist: Na), and the tasks (cap / 256 + Na: first row,
+    // alpha string, rows)
+    int32_t *first, *alist;
+    int4 *tasks;
     int32_t *number, *nfex, *nm;
     uint32_t *fex;
     uint16_t *mcol;

@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(256)
 k_sup_runs(const int64_t *__restrict__ list, const unsigned long long *__restrict__ cnt,
            int64_t cap, int64_t Nb, int64_t *__restrict__ runs, int32_t *__restrict__ ralpha,
            uint8_t *__restrict__ flagA, uint8_t *__restrict__ flagB,
-           unsigned long long *__restrict__ ctr)
+           unsigned long long *__restrict__ ctr, int32_t *__restrict__ first)
 {
     const int64_t m = list_len(cnt, 0, cap);
     for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < m;
@@ -201,6 +201,7 @@ k_sup_runs(const int64_t *__restrict__ list, const unsigned long long *__restric
             runs[pos] = t;
             ralpha[pos] = int32_t(A);
             flagA[A] = 1;
+            if (first) first[A] = int32_t(t);
         }
     }
 }
@@ -410,47 +411,87 @@ k_sup_beta(SupRowsArgs<T> a)
 // The same in double (k_sup_rows): the strings of S are few (450 of 12,870 in
 // 200,000 determinants), so the beta strings present are numbered and everything
 // is restricted to them first:
-//   k_sup_number, one CTA: blist, the beta strings of S in order, and their
-//     numbers (-1: none);
+//   k_sup_number, one CTA a spin: blist, the beta strings of S in order, and their
+//     numbers (-1: none); the runs of S by alpha string, cut into tasks of at most
+//     256 rows;
 //   k_sup_tables, a warp per beta string j: its excitations and its M_beta row
 //     that stay among them (j-minor, so that neighbouring rows read neighbouring
 //     words), and D[pq][j] = sum_{r in B_j} V[pq][rr];
-//   k_sup_rows, one CTA per alpha string A: a thread per row (A, B), psi's rows A
-//     and A_e of the numbered strings in shared memory, the next one on its way
-//     (cp.async) while one is used; A's M_alpha row, filtered once, reads psi down
-//     column B.
+//   k_sup_rows, a CTA per task: a thread per row (A, B); psi's row A and rows A_e of
+//     the numbered strings in shared memory (cp.async), as many together as fit half
+//     of it, the next ones on their way; A's M_alpha row, filtered once, reads psi
+//     down column B.
 // k_sup_alpha stages all Nb amplitudes of a row for each A_e and multiplies all 64
 // excitations, k_sup_beta a column of Na.  Bound by FP64 (a multiply-add per
-// coupling inside S), then by the runs' lengths.  Measured, 200,000 determinants of
-// 8 + 8 electrons in 16 orbitals: 1,330 -> 332 us (k_sup_rows 285); the sums are in
-// another order, so float, whose results are kept, stays with the two above.
+// coupling inside S; a third of its rate reached), then by the chains of loads that
+// feed it.  Measured, 200,000 determinants of 8 + 8 electrons in 16 orbitals, all of it:
+// 1,330 -> 290 us; k_sup_rows 242 (a CTA of 512 threads an SM, whole runs, a row at
+// a time: 285).  The sums are in another order, so float, whose results are kept,
+// stays with the two above.
 // ---------------------------------------------------------------------------
 constexpr int kSupRowMax = 896;        // entries of an M_alpha row: 849 at most
 
-__global__ void __launch_bounds__(1024)
-k_sup_number(const uint8_t *__restrict__ flagB, int Nb, int32_t *__restrict__ number,
-             int32_t *__restrict__ blist, unsigned long long *__restrict__ ctr)
+constexpr int kSupTask = 256;          // rows of a task, threads of its CTA
+
+// exclusive prefix of c over a block of 1,024 threads and the total
+__device__ __forceinline__ int scan_1024(int c, int *wt, int &total)
 {
-    __shared__ int wt[32];
-    const int per = (Nb + 1023) / 1024, b0 = int(threadIdx.x) * per, b1 = min(Nb, b0 + per);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int c = 0;
-    for (int b = b0; b < b1; ++b) c += flagB[b];
     int x = c;
     for (int o = 1; o < 32; o <<= 1) {
         const int y = __shfl_up_sync(0xffffffffu, x, o);
         if (lane >= o) x += y;
     }
+    __syncthreads();
     if (lane == 31) wt[w] = x;
     __syncthreads();
-    int pos = x - c;
-    for (int i = 0; i < w; ++i) pos += wt[i];
-    for (int b = b0; b < b1; ++b) {
-        const bool in = flagB[b] != 0;
-        number[b] = in ? pos : -1;
-        if (in) blist[pos++] = b;
+    int before = 0;
+    total = 0;
+    for (int i = 0; i < 32; ++i) {
+        if (i < w) before += wt[i];
+        total += wt[i];
     }
-    if (threadIdx.x == 1023) ctr[1] = (unsigned long long)pos;
+    return before + x - c;
+}
+
+__global__ void __launch_bounds__(1024)
+k_sup_number(SupRowsArgs<double> a)
+{
+    __shared__ int wt[32];
+    const bool beta = blockIdx.x == 0;
+    const int N = int(beta ? a.s.Nb : a.s.Na), per = (N + 1023) / 1024;
+    const int s0 = min(N, int(threadIdx.x) * per), s1 = min(N, s0 + per);
+    const uint8_t *flag = beta ? a.flagB : a.flagA;
+    int32_t *list = beta ? a.blist : a.alist;
+    int c = 0, n;
+    for (int s = s0; s < s1; ++s) c += flag[s];
+    int pos = scan_1024(c, wt, n);
+    for (int s = s0; s < s1; ++s) {
+        const bool in = flag[s] != 0;
+        if (beta) a.number[s] = in ? pos : -1;
+        if (in) list[pos++] = s;
+    }
+    if (beta) {
+        if (threadIdx.x == 0) a.ctr[1] = (unsigned long long)n;
+        return;
+    }
+    __syncthreads();                              // the list is written
+    const int m = int(list_len(a.cnt, 0, a.cap));
+    int base = 0;
+    for (int i0 = 0; i0 < n; i0 += 1024) {
+        const int i = i0 + int(threadIdx.x);
+        int A = 0, t = 0, rows = 0, total;
+        if (i < n) {
+            A = list[i];
+            t = a.first[A];
+            rows = (i + 1 < n ? a.first[list[i + 1]] : m) - t;
+        }
+        int at = base + scan_1024((rows + kSupTask - 1) / kSupTask, wt, total);
+        for (int r = 0; r < rows; r += kSupTask)
+            a.tasks[at++] = make_int4(t + r, A, min(kSupTask, rows - r), 0);
+        base += total;
+    }
+    if (threadIdx.x == 0) a.ctr[3] = (unsigned long long)base;
 }
 
 __global__ void __launch_bounds__(256)
@@ -504,141 +545,114 @@ __device__ __forceinline__ void cp_async8(double *dst, const double *src)
                  : "memory");
 }
 
+// a slot: a row of psi and V[pq_e][.]; at least one whole one, two CTAs an SM
 size_t sup_rows_smem(int64_t Nb, int nn)
 {
-    return (2 * (size_t(Nb) + size_t(nn)) + size_t(nn) + kSupRowMax) * sizeof(double) +
-           kSupRowMax * sizeof(int32_t);
+    return (size_t(Nb) + 2 * size_t(nn)) * sizeof(double) + kSupRowMax * sizeof(uint32_t);
 }
 
-__global__ void __launch_bounds__(kSupThreads, 1)
+__global__ void __launch_bounds__(kSupTask, 2)
 k_sup_rows(SupRowsArgs<double> a)
 {
     extern __shared__ __align__(16) unsigned char sup_sm[];
     const SparseArgs<double> &h = a.s;
     const int n = h.n, nn = n * n, nexa = h.nexa;
     const int64_t Nb = h.Nb;
-    const int nb = int(a.ctr[1]);
-    double *row0 = reinterpret_cast<double *>(sup_sm);    // two rows of psi
-    double *vrow0 = row0 + 2 * Nb;                        // V[pq_e][.] of each
-    double *dA = vrow0 + 2 * nn;                          // sum_{p in A} V[pp][.]
-    double *mav = dA + nn;                                // A's M_alpha row inside S
-    int32_t *mac = reinterpret_cast<int32_t *>(mav + kSupRowMax);
-    __shared__ uint32_t aexs[64];
-    __shared__ int64_t sh_r;
-    __shared__ int sh_cnt[kSupThreads / 32], sh_ne, sh_nm;
+    const int nb = int(a.ctr[1]), width = nb + nn;
+    double *slots = reinterpret_cast<double *>(sup_sm);
+    double *dA = slots + Nb + nn;                         // sum_{p in A} V[pp][.]
+    uint32_t *mac = reinterpret_cast<uint32_t *>(dA + nn);    // A's M_alpha row inside S
+    __shared__ uint32_t aexs[65];                         // [0]: row A itself
+    __shared__ int sh_task, sh_ne, sh_nm;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    auto stage = [&](int buf, int64_t R, int pq) {
-        double *row = row0 + buf * Nb;
-        for (int j = tid; j < nb; j += kSupThreads) cp_async8(row + j, h.psi + R * Nb + a.blist[j]);
-        if (pq >= 0)
-            for (int q = tid; q < nn; q += kSupThreads)
-                cp_async8(vrow0 + buf * nn + q, h.V + size_t(pq) * nn + q);
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
+    const int fit = int((Nb + nn) / width);               // slots; in two halves, or one
+    const int group = fit > 1 ? min(fit / 2, 65) : 1, ring = fit > 1 ? 2 * group : 1;
     auto pq_of = [&](uint32_t u) { return int((u >> 20) & 15) * n + int((u >> 16) & 15); };
     for (;;) {
-        __syncthreads();                          // the previous run's rows are read
-        if (tid == 0) sh_r = int64_t(atomicAdd(a.ctr + 2, 1ull));
+        __syncthreads();                          // the previous task's rows are read
+        if (tid == 0) sh_task = int(atomicAdd(a.ctr + 2, 1ull));
         __syncthreads();
-        const int64_t r = sh_r;
-        if (r >= int64_t(a.ctr[0])) break;
-        const int64_t t0 = a.runs[r], A = a.ralpha[r];
-        // the run's length: A's row of the bitmap (bits A Nb .. A Nb + Nb - 1)
-        {
-            const int64_t b0 = A * Nb, b1 = b0 + Nb, w0 = b0 >> 5, w1 = (b1 - 1) >> 5;
-            int c = 0;
-            for (int64_t w = w0 + tid; w <= w1; w += kSupThreads) {
-                uint32_t x = a.bits[w];
-                if (w == w0) x &= ~0u << (b0 & 31);
-                if (w == w1 && (b1 & 31)) x &= (1u << (b1 & 31)) - 1u;
-                c += __popc(x);
-            }
-            c = warp_sum(c);
-            if (lane == 0) sh_cnt[warp] = c;
-        }
+        if (sh_task >= int(a.ctr[3])) break;
+        const int4 task = a.tasks[sh_task];
+        const int64_t A = task.y;
         const uint32_t am = h.astr[A];
-        for (int i = tid; i < nn; i += kSupThreads) dA[i] = sum_diag<double>(h.V, n, nn, am, i);
+        for (int i = tid; i < nn; i += kSupTask) dA[i] = sum_diag<double>(h.V, n, nn, am, i);
         if (warp < 2) {
-            // A's excitations (warp 0) and M_alpha row (warp 1) to strings of S
-            int c = 0;
-            const int k1 = warp ? h.Ma_ptr[A + 1] : nexa;
-            for (int k0 = warp ? h.Ma_ptr[A] : 0; k0 < k1; k0 += 32) {
+            // A's excitations (warp 0) and M_alpha row (warp 1: the column and the
+            // entry's place) to strings of S
+            int c = warp ? 0 : 1;
+            const int kb = warp ? h.Ma_ptr[A] : 0, k1 = warp ? h.Ma_ptr[A + 1] : nexa;
+            for (int k0 = kb; k0 < k1; k0 += 32) {
                 const int k = k0 + lane;
                 uint32_t u = 0u;
                 if (k < k1) u = warp ? uint32_t(h.Ma_col[k]) : h.aex[A * nexa + k];
                 const bool in = k < k1 && a.flagA[u & 0xFFFFu];
                 const unsigned bal = __ballot_sync(0xffffffffu, in);
                 const int pos = c + __popc(bal & ((1u << lane) - 1u));
-                if (in && warp == 0) aexs[pos] = u;
-                if (in && warp == 1) {
-                    mac[pos] = int32_t(u);
-                    mav[pos] = h.Ma_val[k];
-                }
+                if (in) (warp ? mac : aexs)[pos] = warp ? u | uint32_t(k - kb) << 16 : u;
                 c += __popc(bal);
             }
             if (lane == 0) *(warp ? &sh_nm : &sh_ne) = c;
+            if (tid == 0) aexs[0] = uint32_t(A);
         }
         __syncthreads();
-        int64_t mA = 0;
-        for (int w = 0; w < kSupThreads / 32; ++w) mA += sh_cnt[w];
-        if (t0 + mA > a.cap) mA = a.cap - t0;    // an overflowed (invalid) support
-        const int ne = sh_ne, nma = sh_nm;
-        const int64_t *Brun = a.list + t0;
-        for (int64_t c0 = 0; c0 < mA; c0 += kSupThreads) {
-            // row A in buffer 0, then the rows A_e in turn
-            stage(0, A, -1);
-            if (ne) stage(1, aexs[0] & 0xFFFFu, pq_of(aexs[0]));
-            const int64_t i = c0 + tid;
-            const bool act = i < mA;
-            const int64_t B = act ? Brun[i] - A * Nb : 0;
-            const int j = act ? a.number[B] : 0, nf = act ? a.nfex[j] : 0, nm = act ? a.nm[j] : 0;
-            const uint32_t bm = act ? h.bstr[B] : 0u;
-            double s = 0.0;
-            if (act) {
-                const double *col = h.psi + B;
-#pragma unroll 4
-                for (int k = 0; k < nma; ++k) s = fma(mav[k], __ldg(col + int64_t(mac[k]) * Nb), s);
+        const int items = sh_ne, nma = sh_nm;     // row A and the rows A_e
+        auto stage = [&](int first) {
+            for (int q = first; q < min(items, first + group); ++q) {
+                const uint32_t u = aexs[q];
+                double *slot = slots + size_t(q % ring) * width;
+                const double *src = h.psi + int64_t(u & 0xFFFFu) * Nb, *v = h.V + size_t(pq_of(u)) * nn;
+                for (int j = tid; j < nb; j += kSupTask) cp_async8(slot + j, src + a.blist[j]);
+                if (q)
+                    for (int i = tid; i < nn; i += kSupTask) cp_async8(slot + nb + i, v + i);
             }
-            if (ne) asm volatile("cp.async.wait_group 1;" ::: "memory");
-            else asm volatile("cp.async.wait_group 0;" ::: "memory");
-            __syncthreads();
-            const uint32_t *ex = a.fex + j;
-            {
-                const double *row = row0;
-#pragma unroll 4
-                for (int k = 0; k < nm; ++k)
-                    s = fma(a.mval[size_t(k) * nb + j], row[a.mcol[size_t(k) * nb + j]], s);
-                for (int f = 0; f < nf; ++f) {
-                    const uint32_t w = ex[size_t(f) * nb];
-                    const double c = dA[(w >> 16) & 255u];
-                    s = fma((w >> 31) ? -c : c, row[w & 0xFFFFu], s);
-                }
-                if (act) {
-                    double d = 0.0;
-                    for (uint32_t mm = bm; mm; mm &= mm - 1) d += dA[(__ffs(mm) - 1) * (n + 1)];
-                    s = fma(d, row[j], s);
-                }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        stage(0);
+        const bool act = tid < task.z;
+        const int64_t d = act ? a.list[task.x + tid] : 0, B = act ? d - A * Nb : 0;
+        const int j = act ? a.number[B] : 0, nf = act ? a.nfex[j] : 0, nm = act ? a.nm[j] : 0;
+        const uint32_t *ex = a.fex + j;
+        double s = 0.0;
+        if (act) {
+            const double *col = h.psi + B, *val = h.Ma_val + h.Ma_ptr[A];
+#pragma unroll 8
+            for (int k = 0; k < nma; ++k) {
+                const uint32_t u = mac[k];
+                s = fma(__ldg(val + (u >> 16)), __ldg(col + int64_t(u & 0xFFFFu) * Nb), s);
             }
-            for (int e = 0; e < ne; ++e) {
-                const int buf = (e + 1) & 1;
-                const uint32_t u = aexs[e];
-                asm volatile("cp.async.wait_group 0;" ::: "memory");
-                __syncthreads();                  // this row is there, the last one read
-                if (e + 1 < ne) stage(buf ^ 1, aexs[e + 1] & 0xFFFFu, pq_of(aexs[e + 1]));
-                if (!act) continue;
-                const double *row = row0 + buf * Nb, *vrow = vrow0 + buf * nn;
-                double t = __ldg(a.dbeta + size_t(pq_of(u)) * nb + j) * row[j];
-#pragma unroll 4
-                for (int f = 0; f < nf; ++f) {
-                    const uint32_t w = ex[size_t(f) * nb];
-                    const double c = vrow[(w >> 16) & 255u];
-                    t = fma((w >> 31) ? -c : c, row[w & 0xFFFFu], t);
-                }
-                s = (u >> 31) ? s - t : s + t;
-            }
-            if (act) h.sigma[Brun[i]] = s;
-            __syncthreads();                      // both buffers are free
         }
+        for (int first = 0; first < items; first += group) {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncthreads();                      // these rows are there, the last ones read
+            if (ring > 1 && first + group < items) stage(first + group);
+            for (int q = first; act && q < min(items, first + group); ++q) {
+                const double *row = slots + size_t(q % ring) * width;
+                if (q == 0) {
+#pragma unroll 8
+                    for (int k = 0; k < nm; ++k)
+                        s = fma(a.mval[size_t(k) * nb + j], row[a.mcol[size_t(k) * nb + j]], s);
+                    double t = 0.0;
+                    for (uint32_t mm = h.bstr[B]; mm; mm &= mm - 1) t += dA[(__ffs(mm) - 1) * (n + 1)];
+                    s = fma(t, row[j], s);
+                }
+                const double *c = q ? row + nb : dA;
+                const uint32_t u = aexs[q];
+                double t = q ? __ldg(a.dbeta + size_t(pq_of(u)) * nb + j) * row[j] : 0.0;
+#pragma unroll 8
+                for (int f = 0; f < nf; ++f) {
+                    const uint32_t w = ex[size_t(f) * nb];
+                    const double v = c[(w >> 16) & 255u];
+                    t = fma((w >> 31) ? -v : v, row[w & 0xFFFFu], t);
+                }
+                s = q && (u >> 31) ? s - t : s + t;
+            }
+            if (ring == 1 && first + group < items) {
+                __syncthreads();
+                stage(first + group);
+            }
+        }
+        if (act) h.sigma[d] = s;
     }
 }
 
@@ -2430,18 +2444,17 @@ cudaError_t hpsi_support(const SupRowsArgs<T> &a, int num_sms, cudaStream_t st)
     if (g > int64_t(num_sms) * 8) g = int64_t(num_sms) * 8;
     if (g < 1) g = 1;
     k_sup_runs<<<unsigned(g), 256, 0, st>>>(a.list, a.cnt, a.cap, h.Nb, a.runs, a.ralpha,
-                                             a.flagA, a.flagB, a.ctr);
+                                             a.flagA, a.flagB, a.ctr, a.first);
     hy::count_launch();
     if constexpr (sizeof(T) == 8) {
-        k_sup_number<<<1, 1024, 0, st>>>(a.flagB, int(h.Nb), a.number, a.blist, a.ctr);
+        k_sup_number<<<2, 1024, 0, st>>>(a);
         hy::count_launch();
         k_sup_tables<<<dim3(unsigned(num_sms) * 2, 2), 256, 0, st>>>(a);
         hy::count_launch();
         const size_t sr = sup_rows_smem(h.Nb, h.n * h.n);
         e = cudaFuncSetAttribute(k_sup_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sr));
         if (e != cudaSuccess) return e;
-        // 512 threads of at most 128 registers: one CTA an SM, whatever it stages
-        k_sup_rows<<<unsigned(num_sms), kSupThreads, sr, st>>>(a);
+        k_sup_rows<<<unsigned(num_sms) * 2, kSupTask, sr, st>>>(a);
         hy::count_launch();
         return cudaGetLastError();
     } else {
