@@ -848,14 +848,15 @@ def run_ours(args, rank, world):
 
 # kernels behind each class of the library's event profiler
 CLASS_KERNELS = {
-    "hpsi": "k_spmm + k_transpose + k_add_transposed + coupling (dense H|psi>)",
+    "hpsi": "k_rows64 (double, up to 1,716 beta strings), k_same or k_spmm with their transposes, "
+            "coupling (dense H|psi>)",
     "hpsi_sparse": "sparse H|psi>: k_hpsi_scatter (all of sigma, after a memset), "
-                   "k_hss_apply (the stored support Hamiltonian), k_sup_alpha + k_sup_beta "
+                   "k_hss_apply (the stored support Hamiltonian), k_sup_rows (float: k_sup_alpha + k_sup_beta) "
                    "(rows of the support)",
     "excite": "k_excite / k_excite_n (dense pair rotations: 4 s bytes per pair)",
     "sparse_excite": "k_sv_excite, k_sv_prepare, support programs k_prog_prepare[_big] + "
                      "k_prog_grad[_big] and their compilation, H_SS build",
-    "screen": "k_grad_partial + k_grad_final (dense pool gradients)",
+    "screen": "k_screen, k_screen32 or k_grad_partial with their sums (dense pool gradients)",
     "screen_sparse": "k_grad_sparse + k_grad_sparse_final (support-restricted pool "
                      "gradients)",
     "reduce": "dots, norms, renormalisation",
@@ -864,10 +865,10 @@ CLASS_KERNELS = {
 }
 # the source files whose kernels each class launches (for the traffic record)
 CLASS_SOURCES = {
-    "hpsi": ["hy_sigma.cu", "hy_cpl_tc.cu"],
+    "hpsi": ["hy_sigma.cu", "hy_cpl_tc.cu", "hy_same.cu", "hy_rows64.cu"],
     "hpsi_sparse": ["hy_sparse.cu", "hy_api.cu", "hy_adapt.cpp"],
     "excite": ["hy_sweeps.cu"], "sparse_excite": ["hy_sparse.cu"],
-    "screen": ["hy_sweeps.cu"], "screen_sparse": ["hy_sparse.cu"],
+    "screen": ["hy_sweeps.cu", "hy_screen.cu", "hy_screen32.cu"], "screen_sparse": ["hy_sparse.cu"],
     "reduce": ["hy_sweeps.cu"], "features": ["hy_ranker.cu"], "hmat": ["hy_hmat.cu"],
 }
 

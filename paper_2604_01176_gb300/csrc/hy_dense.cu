@@ -8,7 +8,7 @@
 // CTAs walks the whole chain, the cluster barrier (hardware, well below a
 // microsecond) in the place of the launch boundary.  The vectors are spread
 // over the CTAs' shared memories (up to kDenseMaxN determinants: psi, or phi
-// and lambda, 8,192 amplitudes of each per CTA), partners read and written
+// and lambda, 4,096 amplitudes of each per CTA), partners read and written
 // through distributed shared memory.
 //
 // Bound: the latency of a pass (pair, amplitudes, store, barrier).  Four

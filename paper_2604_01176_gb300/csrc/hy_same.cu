@@ -31,7 +31,7 @@
 // is added to it once.
 // Waits are bounded as in hy_cpl_tc.cu.
 // Measured: 12,870 strings squared 33.0 -> 12.3 ms a side (71 % of the MMA rate,
-// the rest between stages: 96 KB of L2 reads a pair and 1,536 clocks), 1,716 360 ->
+// the rest between stages: 128 KB of L2 reads a pair and 1,536 clocks), 1,716 360 ->
 // 73 us; whole float H|psi>, 16 orbitals, 8+8, 142.9 -> 101.2 ms; 12 orbitals, 6+6,
 // 541 -> 492 us.
 #include "hy_kernels.cuh"
