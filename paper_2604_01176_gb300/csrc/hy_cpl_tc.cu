@@ -350,13 +350,17 @@ k_cpl_tc(CplDenseArgs a, int *status, long long spin_limit, int issue)
 // memory for all column tiles of J, already split (n x 8 KB), an operand stage
 // is the 16 types of one r, and the roles run apart, joined by mbarriers only:
 //   * two groups of eight warps build alternate stages.  A thread owns a column
-//     and eight s; its eight partners' indices and signs are one 16-byte load
+//     and eight s; its eight partners' places and signs are one 16-byte load
 //     from a table made when the Hamiltonian is (cpl_entries: 16 bits each,
 //     absent pairs point at a zero behind psi's row), so a stage is eight
 //     gathers, splits and four 16-byte stores;
 //   * one warp issues the MMAs of a stage (six) and commits it;
 //   * four warps read finished accumulators (two in tensor memory, used in turn)
 //     while the next tile is multiplied.
+// The diagonal slot is one more row of W_J where 64 rows have room for it (all but 8
+// electrons in 16 orbitals: DIAG, summed in FP32 by the builders).  W_J is rounded
+// when it is split and the small products go first (hy_same.cu): the error of the
+// float H|psi> against double, 13 orbitals, 7+6: 2.9e-7 -> 2.3e-7.
 // r that no column of a tile holds is skipped.  k_cpl_tc's block-wide barrier
 // per chunk left it at 3,600 clocks per 32 types, 768 of them tensor time.
 // Bound by the hand-over of stages (build, fence, arrive, issue, commit): with
@@ -364,8 +368,9 @@ k_cpl_tc(CplDenseArgs a, int *status, long long spin_limit, int issue)
 // half.  Stages of 8 types (twice the hand-overs) cost 30 %, four groups of four
 // warps, a column's 16 types to a thread, 6-20 %.  Measured, whole float H|psi>:
 // 16 orbitals, 8+8 (66 of 129 ms left of the coupling's) 205 -> 143 ms; 13
-// orbitals, 7+6: 2,989 -> 1,713 us; 11 orbitals, 6+5: 285 -> 183 us; also with few
-// strings: 12 orbitals, 2+2: 62.6 -> 55.9 us.
+// orbitals, 7+6: 2,989 -> 1,713 us; 11 orbitals, 6+5: 285 -> 174 us; also with few
+// strings: 12 orbitals, 2+2: 62.6 -> 55.9 us.  The diagonal's sums by their own loop,
+// all loads at once, gave 11 orbitals 5 % and 13 orbitals 2 % of that.
 // ---------------------------------------------------------------------------
 namespace {
 
@@ -442,6 +447,7 @@ size_t cpl_tcw_smem(int64_t Nb, int n, int stages)
            size_t((Nb + 1 + 3) / 4 * 16);
 }
 
+template <bool DIAG>
 __global__ void __launch_bounds__(kTwThreads, 1)
 k_cpl_tcw(CplDenseArgs a, int nst, int *status, long long spin_limit, int issue)
 {
@@ -487,8 +493,9 @@ k_cpl_tcw(CplDenseArgs a, int nst, int *status, long long spin_limit, int issue)
         // two groups of eight warps take the r in turn; r number i goes to stage
         // i % nst, a thread fills half of a column's types
         const int par = warp >> 3, half = (warp >> 2) & 1, col = tid & (kTcN - 1);
-        const uint32_t none = uint32_t(Nb) | (uint32_t(Nb) << 16);
+        const uint32_t none = uint32_t(Nb * 4) | (uint32_t(Nb * 4) << 16);
         const uint32_t off = kmaj(col, half * 8, kTwSbo);
+        const unsigned char *row = reinterpret_cast<const unsigned char *>(prow);
         uint32_t it = 0;            // r of all tiles so far
         int slot = par, use = 0;    // where this group's next r goes, how often used
         uint32_t tile_no = 0;
@@ -527,35 +534,52 @@ k_cpl_tcw(CplDenseArgs a, int nst, int *status, long long spin_limit, int issue)
             for (int i = tid; i < Nb; i += kTwBuilders) prow[i] = __ldg(src + i);
             if (tid == 0) prow[Nb] = 0.0f;
             const uint32_t jm = a.astr[J];
+            auto diag_coef = [&](int r, int s) {         // sum_{p in J} V[pp][rs]
+                float v = 0.0f;
+                if (r < n && s < n) {
+                    const float *V = a.V + r * n + s;        // the loads go out together
+#pragma unroll
+                    for (int p = 0; p < 16; ++p)
+                        if ((jm >> p) & 1u) v += __ldg(V + size_t(p * n + p) * nn);
+                }
+                return v;
+            };
+            // a thread's m and k4 are the same for all its r
+            const uint32_t u = (tid & 63) < nexa ? __ldg(a.aex + J * nexa + (tid & 63)) : 0u;
+#pragma unroll 4
             for (int i = tid; i < n * kTcM * 4; i += kTwBuilders) {
                 const int m = i & 63, k4 = (i >> 6) & 3, r = i >> 8;
                 float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
                 if (m < nexa) {
-                    const uint32_t u = a.aex[J * nexa + m];
                     const int pj = (u >> 16) & 15, qj = (u >> 20) & 15;
                     const float *V = a.V + size_t(qj * n + pj) * nn + r * n;
 #pragma unroll
                     for (int q = 0; q < 4; ++q)
                         if (4 * k4 + q < n) v[q] = (u >> 31) ? -__ldg(V + 4 * k4 + q) : __ldg(V + 4 * k4 + q);
+                } else if (!DIAG && m == nexa) {
+                    continue;
                 }
                 float4 h, l;
-                split(v[0], h.x, l.x);
-                split(v[1], h.y, l.y);
-                split(v[2], h.z, l.z);
-                split(v[3], h.w, l.w);
+                split_rn(v[0], h.x, l.x);
+                split_rn(v[1], h.y, l.y);
+                split_rn(v[2], h.z, l.z);
+                split_rn(v[3], h.w, l.w);
                 unsigned char *dst = Wa + size_t(r) * 2 * kTwA + kmaj(m, 4 * k4, kTwSbo);
                 *reinterpret_cast<float4 *>(dst) = h;
                 *reinterpret_cast<float4 *>(dst + kTwA) = l;
             }
-            for (int i = tid; i < 256; i += kTwBuilders) {
-                const int r = i >> 4, s = i & 15;
-                float v = 0.0f;
-                if (r < n && s < n)
-                    for (uint32_t mm = jm; mm; mm &= mm - 1) {
-                        const int p = __ffs(mm) - 1;
-                        v += a.V[size_t(p * n + p) * nn + r * n + s];
-                    }
-                Wd[i] = v;
+            for (int i = tid; i < n * 16; i += kTwBuilders) {
+                const int r = i >> 4, sp = i & 15;
+                const float v = diag_coef(r, sp);
+                if (DIAG) {
+                    Wd[i] = v;
+                } else {                     // one more row of W_J
+                    float h, l;
+                    split_rn(v, h, l);
+                    unsigned char *dst = Wa + size_t(r) * 2 * kTwA + kmaj(nexa, sp, kTwSbo);
+                    *reinterpret_cast<float *>(dst) = h;
+                    *reinterpret_cast<float *>(dst + kTwA) = l;
+                }
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             builders_and(true);
@@ -579,16 +603,20 @@ k_cpl_tcw(CplDenseArgs a, int nst, int *status, long long spin_limit, int issue)
                     }
                     const uint32_t w[4] = {e.x, e.y, e.z, e.w};
                     float h[8], l[8];
-                    const float4 c0 = *reinterpret_cast<const float4 *>(Wd + r * 16 + half * 8);
-                    const float4 c1 = *reinterpret_cast<const float4 *>(Wd + r * 16 + half * 8 + 4);
-                    const float c[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        const uint32_t x = q & 1 ? w[q >> 1] >> 16 : w[q >> 1] & 0xFFFFu;
-                        const float v = __uint_as_float(__float_as_uint(prow[x & 0x7FFFu]) ^
-                                                        ((x & 0x8000u) << 16));
-                        dsum = fmaf(c[q], v, dsum);
-                        split(v, h[q], l[q]);
+                    for (int q = 0; q < 4; ++q) {
+                        // four times the place in the row, and the sign
+                        const float x = *reinterpret_cast<const float *>(row + (w[q] & 0xFFFCu));
+                        const float y = *reinterpret_cast<const float *>(row + ((w[q] >> 16) & 0xFFFCu));
+                        const float xs = __uint_as_float(__float_as_uint(x) ^ (w[q] << 31));
+                        const float ys = __uint_as_float(__float_as_uint(y) ^ ((w[q] << 15) & 0x80000000u));
+                        if (DIAG) {
+                            const float2 c = *reinterpret_cast<const float2 *>(Wd + r * 16 + half * 8 + 2 * q);
+                            dsum = fmaf(c.x, xs, dsum);
+                            dsum = fmaf(c.y, ys, dsum);
+                        }
+                        split(xs, h[2 * q], l[2 * q]);
+                        split(ys, h[2 * q + 1], l[2 * q + 1]);
                     }
                     // the MMAs that read this stage last
                     if (use)
@@ -599,7 +627,7 @@ k_cpl_tcw(CplDenseArgs a, int nst, int *status, long long spin_limit, int issue)
                     *reinterpret_cast<float4 *>(Bh + off + 128) = make_float4(h[4], h[5], h[6], h[7]);
                     *reinterpret_cast<float4 *>(Bl + off) = make_float4(l[0], l[1], l[2], l[3]);
                     *reinterpret_cast<float4 *>(Bl + off + 128) = make_float4(l[4], l[5], l[6], l[7]);
-                    if (!left) {
+                    if (DIAG && !left) {
                         // the tile's last stage of this group: its part of the
                         // diagonal slot, once that tile's place has been read
                         const uint32_t buf = tile_no & 1u, used = tile_no >> 1;
@@ -648,14 +676,15 @@ k_cpl_tcw(CplDenseArgs a, int nst, int *status, long long spin_limit, int issue)
                         const uint32_t bh = sa + uint32_t(slot) * uint32_t(2 * kTwB);
                         if (elect_one()) {
 #pragma unroll
-                            for (int ks = 0; ks < 2; ++ks) {
+                            for (int ks = 0; ks < 2; ++ks) {      // the small products first
                                 const uint64_t da = sdesc(ah + ks * 256u, kTwSbo);
                                 const uint64_t db = sdesc(bh + ks * 256u, kTwSbo);
-                                mma(d, da, db, acc);
-                                mma(d, da, db + (kTwB >> 4), 1u);
+                                mma(d, da, db + (kTwB >> 4), ks ? 1u : acc);
                                 mma(d, da + (kTwA >> 4), db, 1u);
-                                acc = 1u;
                             }
+#pragma unroll
+                            for (int ks = 0; ks < 2; ++ks)
+                                mma(d, sdesc(ah + ks * 256u, kTwSbo), sdesc(bh + ks * 256u, kTwSbo), 1u);
                             commit(&ctl->empty[slot]);
                         }
                         acc = 1u;
@@ -679,6 +708,7 @@ k_cpl_tcw(CplDenseArgs a, int nst, int *status, long long spin_limit, int issue)
     } else {
         // ---- epilogue --------------------------------------------------------
         const int ew = warp - kTwBuilders / 32;        // sub-partition: warp % 4
+        const int rows = DIAG ? nexa : slots;
         uint32_t it = 0, tile_no = 0;
         bool ok = true;
         for (int64_t jj = blockIdx.x; jj < a.nJ && ok; jj += gridDim.x) {
@@ -697,7 +727,7 @@ k_cpl_tcw(CplDenseArgs a, int nst, int *status, long long spin_limit, int issue)
                 for (int cb = 0; cb < kTcN / 32; ++cb) {
                     float v[32];
                     tmem_ld32(rowaddr + uint32_t(cb * 32), v);
-                    if (lane < 16 && m < nexa) {
+                    if (lane < 16 && m < rows) {
 #pragma unroll
                         for (int i = 0; i < 32; i += 4)
                             if (b0 + cb * 32 + i < int(a.Nbp))      // Nbp: Nb rounded up to 64
@@ -708,7 +738,7 @@ k_cpl_tcw(CplDenseArgs a, int nst, int *status, long long spin_limit, int issue)
                 // the diagonal slot: 32 columns a warp; a group without a stage in
                 // this tile (one r only) has left nothing
                 const int c = ew * 32 + lane;
-                if (b0 + c < Nb) {
+                if (DIAG && b0 + c < Nb) {
                     const float *d = dpart + buf * 4 * kTcN + c;
                     const float s = stages >= 2 ? (d[0] + d[kTcN]) + (d[2 * kTcN] + d[3 * kTcN])
                                                 : d[g1 * kTcN] + d[(g1 + 1) * kTcN];
@@ -730,7 +760,7 @@ k_cpl_tcw(CplDenseArgs a, int nst, int *status, long long spin_limit, int issue)
 // entries and the r each tile holds (k_cpl_tcw), from the packed beta
 // excitations: entry (tile, i, column, s) belongs to the i-th occupied orbital r
 // of the column's string: its partner with r -> s (s empty), itself (s = r), or
-// the zero behind psi's row; bit 15: sign
+// the zero behind psi's row; four times the place in the row, plus the sign
 __global__ void __launch_bounds__(256)
 k_cpl_entries(const uint32_t *__restrict__ bstr, const uint32_t *__restrict__ bexT, int Nb, int n,
               int nocc, int tiles, uint16_t *__restrict__ entries, uint32_t *__restrict__ tmask)
@@ -740,18 +770,18 @@ k_cpl_entries(const uint32_t *__restrict__ bstr, const uint32_t *__restrict__ be
          id += int64_t(gridDim.x) * blockDim.x) {
         const int s = int(id & 15), col = int(id >> 4) & (kTcN - 1);
         const int ti = int(id / (16 * kTcN)), i = ti % nocc, tile = ti / nocc, b = tile * kTcN + col;
-        uint32_t e = uint32_t(Nb);
+        uint32_t e = uint32_t(Nb) * 4;
         if (b < Nb) {
             const uint32_t m = bstr[b];
             uint32_t mm = m;
             for (int k = 0; k < i; ++k) mm &= mm - 1;
             const int r = __ffs(mm) - 1;
             if (s == r) {
-                e = uint32_t(b);
+                e = uint32_t(b) * 4;
             } else if (s < n && !((m >> s) & 1u)) {
                 const int f = i * (n - nocc) + s - __popc(m & ((1u << s) - 1u));
                 const uint32_t u = bexT[size_t(f) * Nb + b];
-                e = (u & 0x7FFFu) | ((u >> 31) << 15);
+                e = (u & 0x3FFFu) * 4 | (u >> 31);
             }
             if (s == 0 && i == 0) atomicOr(tmask + tile, m);
         }
@@ -784,14 +814,16 @@ cudaError_t coupling_tc(const CplDenseArgs &a, int *status, long long spin_limit
         int nst = kTwMaxStages;
         while (nst > 2 && cpl_tcw_smem(a.Nb, a.n, nst) > 227 * 1024) --nst;
         const size_t smem = cpl_tcw_smem(a.Nb, a.n, nst);
-        const cudaError_t e = cudaFuncSetAttribute(
-            k_cpl_tcw, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-        if (e != cudaSuccess) return e;
-        if (a.nJ == 0) return cudaSuccess;
-        k_cpl_tcw<<<unsigned(std::min<int64_t>(num_sms, a.nJ)), kTwThreads, smem, st>>>(
-            a, nst, status, spin_limit, issue);
-        hy::count_launch();
-        return cudaGetLastError();
+        auto run = [&](auto *kernel) {
+            const cudaError_t e = cudaFuncSetAttribute(
+                kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+            if (e != cudaSuccess || a.nJ == 0) return e;
+            kernel<<<unsigned(std::min<int64_t>(num_sms, a.nJ)), kTwThreads, smem, st>>>(
+                a, nst, status, spin_limit, issue);
+            hy::count_launch();
+            return cudaGetLastError();
+        };
+        return a.nexa < kTcM ? run(k_cpl_tcw<false>) : run(k_cpl_tcw<true>);
     }
     const size_t smem = cpl_tc_smem(a.Nb);
     cudaError_t err = cudaFuncSetAttribute(k_cpl_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
