@@ -657,7 +657,8 @@ k_cpl_tcw(CplDenseArgs a, int nst, int *status, long long spin_limit, int issue)
     } else if (warp == kTwIssueWarp) {
         // ---- MMA issue -----------------------------------------------------
         // the whole warp walks the stages (uniform registers hold the operand
-        // descriptors), one elected lane issues
+        // descriptors), one elected lane issues.  One lane's wait decides for all: a
+        // limit that runs out between two lanes' polls must not part them before elect
         uint32_t tile_no = 0;
         int slot = 0, use = 0;
         bool ok = true;
@@ -665,11 +666,12 @@ k_cpl_tcw(CplDenseArgs a, int nst, int *status, long long spin_limit, int issue)
         for (int64_t jj = blockIdx.x; jj < a.nJ && ok; jj += gridDim.x)
             for (int tile = 0; tile < tiles && ok; ++tile, ++tile_no) {
                 const uint32_t buf = tile_no & 1u, used = tile_no >> 1;
-                if (used) ok = tw_wait(ctl, &ctl->acc_empty[buf], (used - 1) & 1u, spin_limit, status);
+                if (used)
+                    ok = tw_wait_warp(ctl, &ctl->acc_empty[buf], (used - 1) & 1u, spin_limit, status);
                 const uint32_t d = tmem + buf * kTmemCols;
                 uint32_t acc = 0;
                 for (uint32_t left = __ldg(a.tmask + tile); left && ok; left &= left - 1) {
-                    ok = tw_wait(ctl, &ctl->full[slot], use & 1u, spin_limit, status);
+                    ok = tw_wait_warp(ctl, &ctl->full[slot], use & 1u, spin_limit, status);
                     if (ok && issue) {
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         const uint32_t ah = wa + uint32_t(__ffs(left) - 1) * uint32_t(2 * kTwA);
