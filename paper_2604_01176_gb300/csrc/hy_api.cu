@@ -7,10 +7,12 @@
 #include <algorithm>
 #include <atomic>
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <new>
 #include <string>
 #include <type_traits>
+#include <utility>
 #include <vector>
 
 #include "hy_internal.h"
@@ -90,6 +92,23 @@ std::atomic<long long> g_launches{0};
 namespace hy {
 void set_last_error(const std::string &msg) { g_err = msg; }
 void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
+
+namespace k {
+cudaError_t allow_smem(const void *kernel, size_t bytes)
+{
+    static std::mutex mu;
+    static std::map<std::pair<int, const void *>, size_t> limits;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    size_t &limit = limits[{dev, kernel}];
+    const size_t want = std::max(limit, bytes);     // set each time: a reset context has forgotten it
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(want));
+    if (e == cudaSuccess) limit = want;
+    return e;
+}
+}  // namespace k
 }  // namespace hy
 
 struct hy_ham {

@@ -330,8 +330,7 @@ cudaError_t batch_rows(const BatchArgs<T> &a, int grid, cudaStream_t st)
 {
     const int groups = a.threads / a.gsize;
     const size_t smem = a.group_smem * groups;
-    cudaError_t e = cudaFuncSetAttribute(k_batch_rows<T>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t e = allow_smem(k_batch_rows<T>, smem);
     if (e != cudaSuccess) return e;
     k_batch_rows<T><<<grid, a.threads, smem, st>>>(a); hy::count_launch();
     return cudaGetLastError();
@@ -342,8 +341,7 @@ cudaError_t batch_occupancy(const BatchArgs<T> &a, int *per_sm)
 {
     const int groups = a.threads / a.gsize;
     const size_t smem = a.group_smem * groups;
-    cudaError_t e = cudaFuncSetAttribute(k_batch_rows<T>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t e = allow_smem(k_batch_rows<T>, smem);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_batch_rows<T>, a.threads, smem);
 }

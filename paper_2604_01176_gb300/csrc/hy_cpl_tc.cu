@@ -817,8 +817,7 @@ cudaError_t coupling_tc(const CplDenseArgs &a, int *status, long long spin_limit
         while (nst > 2 && cpl_tcw_smem(a.Nb, a.n, nst) > 227 * 1024) --nst;
         const size_t smem = cpl_tcw_smem(a.Nb, a.n, nst);
         auto run = [&](auto *kernel) {
-            const cudaError_t e = cudaFuncSetAttribute(
-                kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+            const cudaError_t e = allow_smem(kernel, smem);
             if (e != cudaSuccess || a.nJ == 0) return e;
             kernel<<<unsigned(std::min<int64_t>(num_sms, a.nJ)), kTwThreads, smem, st>>>(
                 a, nst, status, spin_limit, issue);
@@ -828,8 +827,7 @@ cudaError_t coupling_tc(const CplDenseArgs &a, int *status, long long spin_limit
         return a.nexa < kTcM ? run(k_cpl_tcw<false>) : run(k_cpl_tcw<true>);
     }
     const size_t smem = cpl_tc_smem(a.Nb);
-    cudaError_t err = cudaFuncSetAttribute(k_cpl_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           int(smem));
+    cudaError_t err = allow_smem(k_cpl_tc, smem);
     if (err != cudaSuccess) return err;
     if (a.nJ == 0) return cudaSuccess;
     int64_t grid = num_sms;

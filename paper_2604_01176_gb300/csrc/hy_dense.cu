@@ -335,7 +335,7 @@ namespace {
 template <typename... P, typename... A>
 cudaError_t launch_cluster(void (*kernel)(P...), size_t smem, cudaStream_t st, A... args)
 {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t e = allow_smem(kernel, smem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;

@@ -314,8 +314,7 @@ template <typename T, int MAXG>
 cudaError_t launch_spmv(const SpmvArgs<T> &a, int threads, int num_sms, cudaStream_t st)
 {
     const size_t smem = 2 * size_t(a.Nb) * sizeof(T);
-    cudaError_t e = cudaFuncSetAttribute(k_hmat_spmv<T, MAXG>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t e = allow_smem(k_hmat_spmv<T, MAXG>, smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hmat_spmv<T, MAXG>, threads, smem);

@@ -9,6 +9,16 @@ namespace hy {
 void count_launch();
 namespace k {
 
+// Raises a kernel's limit of dynamic shared memory on the current device to `bytes`,
+// and never lowers it: the limit belongs to the function, and another thread may be
+// about to launch the same kernel with more.
+cudaError_t allow_smem(const void *kernel, size_t bytes);
+template <typename... P>
+cudaError_t allow_smem(void (*kernel)(P...), size_t bytes)
+{
+    return allow_smem(reinterpret_cast<const void *>(kernel), bytes);
+}
+
 // Pool metadata on the device.  A constituent C = eps * Ca * Cb with Ca / Cb
 // a pattern id into the alpha / beta pattern lists (-1 = identity).
 struct ConsDev {

@@ -1200,8 +1200,7 @@ hy_status hy_ranker_predict(hy_ranker *r, const float *feat, int64_t m, float *s
         p.F = r->F;
         p.H = r->H;
         const size_t smem = hy::k::mlp_smem(r->H);
-        RTRY(rcu(cudaFuncSetAttribute(hy::k::k_mlp, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      int(smem)), "mlp predict"));
+        RTRY(rcu(hy::k::allow_smem(hy::k::k_mlp, smem), "mlp predict"));
         hy::k::k_mlp<<<unsigned((m + hy::k::kMlpRows - 1) / hy::k::kMlpRows), 256, smem, st>>>(
             p, feat, m, score);
         hy::count_launch();

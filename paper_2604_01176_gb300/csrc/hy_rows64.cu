@@ -245,8 +245,7 @@ cudaError_t rows64(const Rows64Args &a, int64_t n_tasks, int slices, int cols, s
 {
     if (n_tasks <= 0) return cudaSuccess;
     auto run = [&](auto *kernel) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             int(smem));
+        cudaError_t e = allow_smem(kernel, smem);
         if (e != cudaSuccess) return e;
         kernel<<<unsigned(n_tasks), unsigned(slices * cols), smem, st>>>(a);
         hy::count_launch();

@@ -472,7 +472,7 @@ int same_pairs()
     cfg.blockDim = dim3(kSmThreads);
     cfg.dynamicSmemBytes = kSmSmem;
     int n = 0;
-    if (cudaFuncSetAttribute(k_same, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmSmem)) != cudaSuccess ||
+    if (allow_smem(k_same, kSmSmem) != cudaSuccess ||
         cudaOccupancyMaxActiveClusters(&n, k_same, &cfg) != cudaSuccess) {
         cudaGetLastError();
         return 0;
@@ -493,8 +493,7 @@ cudaError_t same(const SameArgs &a, const float *src, int64_t stride, bool trans
         k_same_x<false><<<grid, 256, 0, st>>>(src, stride, int(a.N), a.ncols, nch, a.xpack);
     }
     hy::count_launch();
-    const cudaError_t e =
-        cudaFuncSetAttribute(k_same, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmSmem));
+    const cudaError_t e = allow_smem(k_same, kSmSmem);
     if (e != cudaSuccess) return e;
     const int64_t tiles = ((a.row1 - 1) / kSmRows + 1 - a.row0 / kSmRows) * ncb;
     k_same<<<unsigned(2 * std::min<int64_t>(pairs, tiles)), kSmThreads, kSmSmem, st>>>(a, status, spin_limit);

@@ -283,8 +283,7 @@ k_screen_final(const ScreenMol *__restrict__ mols, int count, const double *__re
 template <int CFG>
 cudaError_t screen_cfg(const ScreenArgs &a, int n_tasks, size_t smem, cudaStream_t st)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_screen<CFG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         int(smem));
+    cudaError_t e = allow_smem(k_screen<CFG>, smem);
     if (e != cudaSuccess) return e;
     k_screen<CFG><<<unsigned(n_tasks), kScThreads, smem, st>>>(a);
     hy::count_launch();

@@ -255,8 +255,7 @@ cudaError_t run32(Screen32Args &a, cudaStream_t st)
     const int64_t others = (int64_t(a.npA + a.npB) * a.CH + G - 1) / G;
     const size_t smem = size_t(DB ? 4 : 2) * (size_t(a.Nb) + 1) * sizeof(float2);
     auto *kern = k_screen32<NK, PB, G, DB>;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               int(smem));
+    const cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<unsigned(a.n_ab + others), 256 * G, smem, st>>>(a);
     hy::count_launch();

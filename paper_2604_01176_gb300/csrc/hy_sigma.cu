@@ -322,8 +322,7 @@ cudaError_t coupling(const CouplingArgs<T> &a, int num_sms, cudaStream_t st)
     const int cpt = int((a.Nb + threads - 1) / threads);
     if (cpt > kCouplingMaxCpt) return cudaErrorInvalidValue;
     const size_t smem = coupling_smem<T>(a.Nb, a.n);
-    cudaError_t err = cudaFuncSetAttribute(
-        k_coupling<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t err = allow_smem(k_coupling<T>, smem);
     if (err != cudaSuccess) return err;
     int per_sm = 0;
     err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_coupling<T>, threads, smem);
@@ -545,8 +544,7 @@ cudaError_t coupling_dense(const CplDenseArgs &a, int num_sms, cudaStream_t st)
     if (a.Na == 0 || a.Nb == 0) return cudaSuccess;
     if (a.nexa + 1 > kGM) return cudaErrorInvalidValue;
     const size_t smem = cpl_dense_smem(a.Nb, a.n);
-    cudaError_t err = cudaFuncSetAttribute(k_cpl_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           int(smem));
+    cudaError_t err = allow_smem(k_cpl_gemm, smem);
     if (err != cudaSuccess) return err;
     int per_sm = 0;
     err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cpl_gemm, kGThreads, smem);

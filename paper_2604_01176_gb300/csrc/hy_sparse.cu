@@ -2452,7 +2452,7 @@ cudaError_t hpsi_support(const SupRowsArgs<T> &a, int num_sms, cudaStream_t st)
         k_sup_tables<<<dim3(unsigned(num_sms) * 2, 2), 256, 0, st>>>(a);
         hy::count_launch();
         const size_t sr = sup_rows_smem(h.Nb, h.n * h.n);
-        e = cudaFuncSetAttribute(k_sup_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sr));
+        e = allow_smem(k_sup_rows, sr);
         if (e != cudaSuccess) return e;
         k_sup_rows<<<unsigned(num_sms) * 2, kSupTask, sr, st>>>(a);
         hy::count_launch();
@@ -2461,9 +2461,9 @@ cudaError_t hpsi_support(const SupRowsArgs<T> &a, int num_sms, cudaStream_t st)
     k_sup_blist<<<unsigned(num_sms), 256, 0, st>>>(a.flagB, h.Nb, a.blist, a.ctr);
     hy::count_launch();
     const size_t sa = sup_alpha_smem<T>(h.Nb, h.n * h.n), sb = size_t(h.Na) * sizeof(T);
-    e = cudaFuncSetAttribute(k_sup_alpha<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sa));
+    e = allow_smem(k_sup_alpha<T>, sa);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_sup_beta<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sb));
+        e = allow_smem(k_sup_beta<T>, sb);
     if (e != cudaSuccess) return e;
     k_sup_alpha<T><<<unsigned(num_sms) * 2u, kSupThreads, sa, st>>>(a);
     hy::count_launch();
