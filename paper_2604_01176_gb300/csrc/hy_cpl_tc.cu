@@ -156,8 +156,9 @@ k_cpl_tc(CplDenseArgs a, int *status, long long spin_limit, int issue)
     auto drain = [&](uint64_t *b, uint32_t &waited, uint32_t issued) {
         while (ok && waited < issued) {
             if (!wait_bar(b, waited & 1u, spin_limit)) {
-                ok = false;
+                ok = false;             // this commit is still out: waited for at the end
                 atomicExch(status, 1);
+                break;
             }
             ++waited;
         }
@@ -333,10 +334,12 @@ k_cpl_tc(CplDenseArgs a, int *status, long long spin_limit, int issue)
             __syncthreads();
         }
     }
-    // on a timeout, give the MMAs still in flight a bounded chance to finish
-    if (!ok) {
-        while (waited0 < issued0) wait_bar(&bar[0], (waited0++) & 1u, spin_limit);
-        while (waited1 < issued1) wait_bar(&bar[1], (waited1++) & 1u, spin_limit);
+    // on a timeout, give the MMAs still in flight a bounded chance to finish, whatever
+    // the limit of the other waits (test mode: nothing was issued, nothing will come)
+    if (!ok && issue) {
+        const long long drain_limit = spin_limit > (1ll << 24) ? spin_limit : 1ll << 24;
+        while (waited0 < issued0) wait_bar(&bar[0], (waited0++) & 1u, drain_limit);
+        while (waited1 < issued1) wait_bar(&bar[1], (waited1++) & 1u, drain_limit);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();

@@ -39,3 +39,10 @@ def _run(cfg, limit):
                          ids=lambda c: "n%da%db%d" % c)
 def test_wide_coupling(cfg, limit):
     _run(cfg, limit)
+
+
+# the kernel of up to 10 orbitals: MMAs in flight at a timeout end before the block does
+@pytest.mark.parametrize("limit", [1, 2, 5, 20, 100])
+@pytest.mark.parametrize("cfg", [(6, 3, 3), (10, 5, 5), (10, 2, 7)], ids=lambda c: "n%da%db%d" % c)
+def test_coupling(cfg, limit):
+    _run(cfg, limit)
