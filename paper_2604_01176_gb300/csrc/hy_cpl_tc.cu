@@ -660,8 +660,11 @@ k_cpl_tcw(CplDenseArgs a, int nst, int *status, long long spin_limit, int issue)
     } else if (warp == kTwIssueWarp) {
         // ---- MMA issue -----------------------------------------------------
         // the whole warp walks the stages (uniform registers hold the operand
-        // descriptors), one elected lane issues.  One lane's wait decides for all: a
-        // limit that runs out between two lanes' polls must not part them before elect
+        // descriptors), one lane, elected once, issues.  Nothing in the loops needs the
+        // lanes together: a limit that runs out between two lanes' polls parts them.
+        // One lane polling for all costs 5 % (16 orbitals) to 12 % of the sweep, electing
+        // and meeting again at each stage 3 to 10 %
+        const bool lead = elect_one();
         uint32_t tile_no = 0;
         int slot = 0, use = 0;
         bool ok = true;
@@ -670,16 +673,16 @@ k_cpl_tcw(CplDenseArgs a, int nst, int *status, long long spin_limit, int issue)
             for (int tile = 0; tile < tiles && ok; ++tile, ++tile_no) {
                 const uint32_t buf = tile_no & 1u, used = tile_no >> 1;
                 if (used)
-                    ok = tw_wait_warp(ctl, &ctl->acc_empty[buf], (used - 1) & 1u, spin_limit, status);
+                    ok = tw_wait(ctl, &ctl->acc_empty[buf], (used - 1) & 1u, spin_limit, status);
                 const uint32_t d = tmem + buf * kTmemCols;
                 uint32_t acc = 0;
                 for (uint32_t left = __ldg(a.tmask + tile); left && ok; left &= left - 1) {
-                    ok = tw_wait_warp(ctl, &ctl->full[slot], use & 1u, spin_limit, status);
+                    ok = tw_wait(ctl, &ctl->full[slot], use & 1u, spin_limit, status);
                     if (ok && issue) {
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         const uint32_t ah = wa + uint32_t(__ffs(left) - 1) * uint32_t(2 * kTwA);
                         const uint32_t bh = sa + uint32_t(slot) * uint32_t(2 * kTwB);
-                        if (elect_one()) {
+                        if (lead) {
 #pragma unroll
                             for (int ks = 0; ks < 2; ++ks) {      // the small products first
                                 const uint64_t da = sdesc(ah + ks * 256u, kTwSbo);
@@ -693,19 +696,17 @@ k_cpl_tcw(CplDenseArgs a, int nst, int *status, long long spin_limit, int issue)
                             commit(&ctl->empty[slot]);
                         }
                         acc = 1u;
-                        __syncwarp();
                     }
                     if (++slot == nst) {
                         slot = 0;
                         ++use;
                     }
                 }
-                if (ok && issue && elect_one()) commit(&ctl->acc_full[buf]);
-                __syncwarp();
+                if (ok && issue && lead) commit(&ctl->acc_full[buf]);
             }
         // every MMA issued is done before the tensor memory goes back
         if (issue) {
-            if (elect_one()) commit(&ctl->fin);
+            if (lead) commit(&ctl->fin);
             __syncwarp();
             wait_bar(&ctl->fin, 0, spin_limit > (1ll << 24) ? spin_limit : 1ll << 24);
         }
