@@ -165,7 +165,8 @@ struct hy_ham {
     // tensor-core kernel with its MMAs withheld (a test of the bounded waits)
     int cpl_impl = 0;
     long long tc_spin_limit = 1ll << 26;   // polls of a stage barrier before giving up
-    int *d_status = nullptr;        // device: a bounded wait of k_cpl_tc ran out
+    // device: [0] a bounded wait of a tensor-core kernel ran out, [1], [2] same_rows'
+    int *d_status = nullptr;
     int *h_status = nullptr;        // pinned host mirror, copied after each launch
     // alpha strings whose coupling rows a row range needs (hy_apply_h_rows)
     int32_t *d_jlist = nullptr;
@@ -577,14 +578,21 @@ hy_status apply_h_t(hy_ham *h, const T *psi, T *sigma, cudaStream_t st, int64_t 
             a.ncols = h->Nb;
             a.row0 = r0;
             a.row1 = r1;
-            HY_CUDA(hy::k::same(a, psi, h->Nb, false, h->same_pairs, h->d_status, h->tc_spin_limit, st),
-                    "alpha part");
+            // psi is looked over whole, whatever the rows: ranges give the full sweep's sums
+            HY_CUDA(hy::k::same(a, psi, h->Nb, false, h->same_pairs, h->d_status, h->d_status + 1,
+                                h->tc_spin_limit, st), "alpha part");
             b.Y = tau;
             b.ncols = nr;
             b.row0 = 0;
             b.row1 = h->Nb;
-            HY_CUDA(hy::k::same(b, psi + r0 * h->Nb, h->Nb, true, h->same_pairs, h->d_status,
+            HY_CUDA(hy::k::same(b, psi + r0 * h->Nb, h->Nb, true, h->same_pairs, h->d_status, nullptr,
                                 h->tc_spin_limit, st), "beta part");
+            hy::k::SameRows rows{};
+            rows.aptr = Ma->ptr; rows.acol = Ma->col; rows.aval = Ma->val;
+            rows.bptr = Mb->ptr; rows.bcol = Mb->col; rows.bval = Mb->val;
+            rows.psi = psi; rows.sigma = sigma; rows.tau = tau;
+            rows.Nb = h->Nb; rows.row0 = r0; rows.row1 = r1;
+            HY_CUDA(hy::k::same_rows(rows, h->d_status + 1, h->num_sms, st), "same-spin parts by rows");
             tc = true;
         }
     }
@@ -1145,8 +1153,8 @@ hy_status finish_ham(hy_ham *h, hy_ham **out)
         return cuda_fail(e, "device query");
     }
     h->dot_blocks = 8 * h->num_sms;
-    e = cudaMalloc(&h->d_status, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(h->d_status, 0, sizeof(int));
+    e = cudaMalloc(&h->d_status, 3 * sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(h->d_status, 0, 3 * sizeof(int));
     if (e == cudaSuccess) e = cudaMallocHost(&h->h_status, sizeof(int));
     if (e != cudaSuccess) {
         cudaFree(h->d_status);

@@ -147,9 +147,20 @@ cudaError_t same_fill(const int32_t *ptr, const int32_t *col, const float *val, 
                       unsigned char *pack, float *diag, cudaStream_t st);
 int same_pairs();
 size_t same_x_bytes(int64_t N, int64_t ncols);
-// element (J, c) of X: src[c * stride + J] if trans, else src[J * stride + c]
+// element (J, c) of X: src[c * stride + J] if trans, else src[J * stride + c].  bad (or
+// null): two ints, zero before; bad[0] is set if X has an element the product may not
+// be trusted with (hy_same.cu)
 cudaError_t same(const SameArgs &a, const float *src, int64_t stride, bool trans, int pairs, int *status,
-                 long long spin_limit, cudaStream_t st);
+                 int *bad, long long spin_limit, cudaStream_t st);
+// sigma (alpha rows [row0, row1)) and tau (beta rows, one column per alpha row) by CSR
+// rows if bad[0] is set, which it clears
+struct SameRows {
+    const int32_t *aptr, *acol, *bptr, *bcol;
+    const float *aval, *bval, *psi;
+    float *sigma, *tau;
+    int64_t Nb, row0, row1;
+};
+cudaError_t same_rows(const SameRows &a, int *bad, int num_sms, cudaStream_t st);
 
 template <typename T>
 cudaError_t spmm(const int32_t *ptr, const int32_t *col, const T *val,

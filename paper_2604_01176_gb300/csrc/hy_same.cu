@@ -30,6 +30,10 @@
 // The diagonal is large and needs no sum: Y starts as diag * X in FP32, and the sum
 // is added to it once.
 // Waits are bounded as in hy_cpl_tc.cu.
+// A dense product multiplies amplitudes by zeros too: one that is not finite, or so
+// large that its rounded half is not, would spoil rows that M does not couple to it.
+// Packing X looks for such a one, and k_same_rows then does both sides over, row by
+// row; else it ends at once (6 of 969 us at 13 orbitals, 7+5, with the looking).
 // Measured: 12,870 strings squared 33.0 -> 12.3 ms a side (71 % of the MMA rate,
 // the rest between stages: 128 KB of L2 reads a pair and 1,536 clocks), 1,716 360 ->
 // 73 us; whole float H|psi>, 16 orbitals, 8+8, 142.9 -> 101.2 ms; 12 orbitals, 6+6,
@@ -355,12 +359,14 @@ k_same(SameArgs a, int *status, long long spin_limit)
 // X as operands: block [128 columns][32 J], hi then lo, zero outside.  Bound by
 // memory (4 bytes read, 8 written an element).
 //   TRANS: element (J, c) is src[c * stride + J], else src[J * stride + c]
+//   bad (or null): set to 1 if an element has no finite halves
 // ---------------------------------------------------------------------------
 template <bool TRANS>
 __global__ void __launch_bounds__(256)
 k_same_x(const float *__restrict__ src, int64_t stride, int N, int64_t ncols, int64_t nch,
-         unsigned char *__restrict__ out)
+         unsigned char *__restrict__ out, int *__restrict__ bad)
 {
+    bool odd = false;
     // lanes along the direction that is contiguous in src
     const int t = threadIdx.x;
     const int64_t ch = TRANS ? blockIdx.x : blockIdx.y, cb = TRANS ? blockIdx.y : blockIdx.x;
@@ -384,6 +390,39 @@ k_same_x(const float *__restrict__ src, int64_t stride, int N, int64_t ncols, in
         const uint32_t off = kmaj(xcol, 4 * k4, kSmSbo);
         *reinterpret_cast<float4 *>(blk + off) = h;
         *reinterpret_cast<float4 *>(blk + kSmOp + off) = l;
+        // x, or hi alone, infinite or NaN: lo is then too
+        auto none = [](float x) { return (__float_as_uint(x) & 0x7F800000u) == 0x7F800000u; };
+        odd = odd || none(l.x) || none(l.y) || none(l.z) || none(l.w);
+    }
+    if (bad && odd) *bad = 1;
+}
+
+// Both sides by rows, as k_spmm sums them, if bad[0]; the last block clears it
+// (bad[1]: blocks done)
+__global__ void __launch_bounds__(256)
+k_same_rows(SameRows a, int *bad)
+{
+    if (*reinterpret_cast<volatile int *>(bad) == 0) return;
+    const int64_t nr = a.row1 - a.row0, ca = (a.Nb + 255) / 256, cb = (nr + 255) / 256;
+    const int64_t na = nr * ca, items = na + a.Nb * cb;
+    for (int64_t i = blockIdx.x; i < items; i += gridDim.x) {
+        const bool al = i < na;
+        const int64_t j = al ? i : i - na, r = al ? a.row0 + j / ca : j / cb;
+        const int64_t c = (al ? j % ca : j % cb) * 256 + threadIdx.x;
+        if (c >= (al ? a.Nb : nr)) continue;
+        const int32_t *ptr = al ? a.aptr : a.bptr, *col = al ? a.acol : a.bcol;
+        const float *val = al ? a.aval : a.bval;
+        const float *x = al ? a.psi + c : a.psi + (a.row0 + c) * a.Nb;
+        const int64_t step = al ? a.Nb : 1;
+        float s[2] = {0.0f, 0.0f};
+        const int k0 = ptr[r], k1 = ptr[r + 1];
+        for (int k = k0; k < k1; ++k) s[(k - k0) & 1] = fmaf(val[k], x[col[k] * step], s[(k - k0) & 1]);
+        (al ? a.sigma + (r - a.row0) * a.Nb : a.tau + r * nr)[c] = s[0] + s[1];
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(bad + 1, 1) == int(gridDim.x) - 1) bad[0] = bad[1] = 0;
     }
 }
 
@@ -480,17 +519,24 @@ int same_pairs()
     return n;
 }
 
+cudaError_t same_rows(const SameRows &a, int *bad, int num_sms, cudaStream_t st)
+{
+    k_same_rows<<<unsigned(2 * num_sms), 256, 0, st>>>(a, bad);
+    hy::count_launch();
+    return cudaGetLastError();
+}
+
 cudaError_t same(const SameArgs &a, const float *src, int64_t stride, bool trans, int pairs, int *status,
-                 long long spin_limit, cudaStream_t st)
+                 int *bad, long long spin_limit, cudaStream_t st)
 {
     if (a.row1 <= a.row0 || a.ncols == 0) return cudaSuccess;
     const int64_t nch = same_chunks(a.N), ncb = (a.ncols + kSmCols - 1) / kSmCols;
     if (trans) {
         const dim3 grid(unsigned(nch), unsigned(2 * ncb));
-        k_same_x<true><<<grid, 256, 0, st>>>(src, stride, int(a.N), a.ncols, nch, a.xpack);
+        k_same_x<true><<<grid, 256, 0, st>>>(src, stride, int(a.N), a.ncols, nch, a.xpack, bad);
     } else {
         const dim3 grid(unsigned(2 * ncb), unsigned(nch));
-        k_same_x<false><<<grid, 256, 0, st>>>(src, stride, int(a.N), a.ncols, nch, a.xpack);
+        k_same_x<false><<<grid, 256, 0, st>>>(src, stride, int(a.N), a.ncols, nch, a.xpack, bad);
     }
     hy::count_launch();
     const cudaError_t e = allow_smem(k_same, kSmSmem);
