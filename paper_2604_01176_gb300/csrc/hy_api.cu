@@ -428,14 +428,13 @@ hy::k::Rows64Mol rows64_mol(const hy_ham *h, int cols)
     return r;
 }
 
-// the float same-spin table of one spin as tensor-core operands; without the
-// memory for it the CSR kernel stays in use
-hy_status pack_same_spin(hy_ham *h, int spin)
+// the float same-spin table of one spin as tensor-core operands, its memory ar's
+cudaError_t pack_same_spin(const hy_ham *h, int spin, DevArena &ar, hy::k::SameArgs &a)
 {
     const int64_t N = spin == 0 ? h->Na : h->Nb;
     const DevCsr<float> &M = spin == 0 ? h->Ma32 : h->Mb32;
     const int nrb = hy::k::same_row_blocks(N), nch = hy::k::same_chunks(N);
-    DevArena tmp, ar;
+    DevArena tmp;
     uint32_t *place = nullptr;
     int32_t *count = nullptr;
     std::vector<int32_t> cnt(size_t(nrb), 0);
@@ -458,7 +457,32 @@ hy_status pack_same_spin(hy_ham *h, int spin)
         e = hy::k::same_fill(M.ptr, M.col, M.val, N, place, d_base, list, pack, diag, nullptr);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     tmp.release();
-    if (e != cudaSuccess || !pack) {
+    a.N = N;
+    a.pack = pack;
+    a.base = d_base;
+    a.list = list;
+    a.diag = diag;
+    return e;
+}
+
+// both spins' operands, where the rule of hy_kernels.cuh asks for them: with a
+// Hamiltonian's first float sweep (double users never pay for them, 2 ms and 2 GB at
+// 12,870 strings); not while a stream is being captured.  Without the memory for both,
+// none is kept and the CSR kernel stays in use
+hy_status pack_same(hy_ham *h, cudaStream_t st)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return HY_OK;
+    }
+    h->same_pairs = hy::k::same_pairs();
+    if (h->same_pairs <= 0) return HY_OK;
+    DevArena ar;
+    hy::k::SameArgs a[2] = {};
+    cudaError_t e = pack_same_spin(h, 0, ar, a[0]);
+    if (e == cudaSuccess && a[0].pack) e = pack_same_spin(h, 1, ar, a[1]);
+    if (e != cudaSuccess || !a[0].pack || !a[1].pack) {
         ar.release();
         if (e != cudaSuccess && e != cudaErrorMemoryAllocation) return cuda_fail(e, "same-spin operands");
         cudaGetLastError();
@@ -466,33 +490,9 @@ hy_status pack_same_spin(hy_ham *h, int spin)
     }
     h->arena.ptrs.insert(h->arena.ptrs.end(), ar.ptrs.begin(), ar.ptrs.end());
     h->arena.uploaded += ar.uploaded;
-    hy::k::SameArgs &a = h->same[spin];
-    a.N = N;
-    a.pack = pack;
-    a.base = d_base;
-    a.list = list;
-    a.diag = diag;
+    h->same[0] = a[0];
+    h->same[1] = a[1];
     return HY_OK;
-}
-
-// both spins' operands, where the rule of hy_kernels.cuh asks for them: with a
-// Hamiltonian's first float sweep (double users never pay for them, 2 ms and 2 GB at
-// 12,870 strings); not while a stream is being captured
-hy_status pack_same(hy_ham *h, cudaStream_t st)
-{
-    if (std::min(h->Na, h->Nb) < hy::k::kSameStrings || !h->d_status) {
-        h->same_pairs = 0;
-        return HY_OK;
-    }
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
-        return HY_OK;
-    }
-    h->same_pairs = hy::k::same_pairs();
-    hy_status s = HY_OK;
-    for (int spin = 0; spin < 2 && s == HY_OK && h->same_pairs > 0; ++spin) s = pack_same_spin(h, spin);
-    return s;
 }
 
 // sigma rows [r0, r1) (alpha strings) of H psi; sigma holds those rows only.
@@ -529,19 +529,21 @@ hy_status apply_h_t(hy_ham *h, const T *psi, T *sigma, cudaStream_t st, int64_t 
     const int64_t Nbp = (h->Nb + 63) / 64 * 64;
     const size_t tbytes = sizeof(T) == sizeof(float)
         ? size_t(h->Na) * size_t(h->A.nex + 1) * size_t(Nbp) * sizeof(float) : 0;
-    // the tensor-core same-spin part takes the same place before it
+    // the tensor-core same-spin parts take the same place before it (as much for any
+    // range of rows: which kernels run must not depend on it), and only with it: memory
+    // for T comes before memory for their operands
     size_t xbytes = 0;
-    if (sizeof(T) == sizeof(float) && h->same_pairs < 0 && h->cpl_impl != 1) {
-        hy_status s = pack_same(h, st);
-        if (s != HY_OK) return s;
-    }
-    if (sizeof(T) == sizeof(float) && h->same[0].pack && h->same[1].pack && h->cpl_impl != 1 && h->d_status)
-        xbytes = std::max(hy::k::same_x_bytes(h->Na, h->Nb), hy::k::same_x_bytes(h->Nb, nr));
+    if (sizeof(T) == sizeof(float) && h->cpl_impl != 1 && h->d_status &&
+        std::min(h->Na, h->Nb) >= hy::k::kSameStrings)
+        xbytes = std::max(hy::k::same_x_bytes(h->Na, h->Nb), hy::k::same_x_bytes(h->Nb, h->Na));
     bool dense = false, same = false;
-    if (xbytes && ensure_ws(h, L.total + std::max(tbytes, xbytes)) == HY_OK) {
-        dense = same = true;
-    } else if (tbytes && (cudaGetLastError(), ensure_ws(h, L.total + tbytes) == HY_OK)) {
+    if (tbytes && ensure_ws(h, L.total + std::max(tbytes, xbytes)) == HY_OK) {
         dense = true;
+        if (xbytes && h->same_pairs < 0) {
+            hy_status s = pack_same(h, st);
+            if (s != HY_OK) return s;
+        }
+        same = xbytes && h->same[0].pack && h->same[1].pack;
     } else {
         cudaGetLastError();   // clear a failed allocation
         hy_status s = ensure_ws(h, L.total);
