@@ -189,9 +189,11 @@ hy_status hy_ham_profile(hy_ham *h, int enable);
  * product T_J = W_J G_J) on the tensor cores (impl = 0, the default:
  * tcgen05 TF32 MMAs with split hi/lo operands, FP32 accuracy) or on the FP32
  * SIMT pipes (impl = 1).  Both feed the same phase B.  The same-spin parts
- * follow the choice where both spins have 512 strings or more and one is not
- * built without the memory for its operands (1 GB a spin for 12,870 strings);
- * else they run on the FP32 pipes.  A bounded wait of a tensor-core kernel
+ * follow the choice where both spins have 512 strings or more: the first float
+ * hy_apply_h or hy_apply_h_rows with impl 0 or 2 (captured or not) makes their
+ * operands, 1 GB a spin for 12,870 strings, and waits on the host for that once
+ * (2 ms).  If the memory for them is not there then, they run on the FP32 pipes
+ * from then on, as they do with fewer strings.  A bounded wait of a tensor-core kernel
  * that runs out is returned as HY_ERR_TIMEOUT by the next
  * hy_apply_h on this handle (the kernel itself gives up, releases its tensor
  * memory and returns; the context stays usable).  impl = 2 is a test of that
@@ -283,7 +285,9 @@ hy_status hy_unrank(const hy_ham *h, const int64_t *idx, uint64_t *dets,
 
 /* sigma = H psi on Omega_CIk (the paper's sparse H times sparse state).
  * psi, sigma: device arrays of n_det elements of the given dtype; they must
- * not alias.  The first call per dtype allocates the handle's workspace. */
+ * not alias.  The first call per dtype allocates the handle's workspace (and, in
+ * HY_F32, makes the operands that hy_ham_set_coupling tells of).  An amplitude
+ * that is not finite reaches the determinants within two excitations only. */
 hy_status hy_apply_h(const hy_ham *h, const void *psi, void *sigma,
                      hy_dtype dt, void *stream);
 
@@ -297,8 +301,11 @@ hy_status hy_apply_h(const hy_ham *h, const void *psi, void *sigma,
  * blocks (or an all-reduce of the scalars formed from them) completes the
  * operation.  Every element is computed by the same arithmetic in the same
  * order as in hy_apply_h, so blocks of any split concatenate to hy_apply_h's
- * sigma bit for bit.  The same-spin parts (on the tensor cores in blocks of
- * 256 rows) and the FP64 coupling cost the range's share of the full sweep;
+ * sigma bit for bit, as long as the same kernels run: not across a change of
+ * hy_ham_set_coupling, nor between calls of which only some had the memory for
+ * the float workspace.  The same-spin parts and the FP64 coupling cost the
+ * range's share of the full sweep, but on the tensor cores a range costs whole
+ * blocks of 256 rows and, once, 8 bytes written for every amplitude of psi;
  * the float tensor-core coupling forms its
  * per-string products for the range's strings and their single-excitation
  * partners (for a contiguous range of more than a few rows, nearly all).

@@ -429,7 +429,8 @@ hy::k::Rows64Mol rows64_mol(const hy_ham *h, int cols)
 }
 
 // the float same-spin table of one spin as tensor-core operands, its memory ar's
-cudaError_t pack_same_spin(const hy_ham *h, int spin, DevArena &ar, hy::k::SameArgs &a)
+cudaError_t pack_same_spin(const hy_ham *h, int spin, DevArena &ar, hy::k::SameArgs &a,
+                           cudaStream_t st)
 {
     const int64_t N = spin == 0 ? h->Na : h->Nb;
     const DevCsr<float> &M = spin == 0 ? h->Ma32 : h->Mb32;
@@ -438,24 +439,34 @@ cudaError_t pack_same_spin(const hy_ham *h, int spin, DevArena &ar, hy::k::SameA
     uint32_t *place = nullptr;
     int32_t *count = nullptr;
     std::vector<int32_t> cnt(size_t(nrb), 0);
-    cudaError_t e = tmp.alloc(&place, size_t(nrb) * nch, true);
+    auto zero = [&](void *p, size_t bytes) { return cudaMemsetAsync(p, 0, bytes, st); };
+    cudaError_t e = tmp.alloc(&place, size_t(nrb) * nch);
+    if (e == cudaSuccess) e = zero(place, size_t(nrb) * nch * sizeof(uint32_t));
     if (e == cudaSuccess) e = tmp.alloc(&count, size_t(nrb));
-    if (e == cudaSuccess) e = hy::k::same_used(M.ptr, M.col, N, place, count, nullptr);
+    if (e == cudaSuccess) e = hy::k::same_used(M.ptr, M.col, N, place, count, st);
     if (e == cudaSuccess)
-        e = cudaMemcpy(cnt.data(), count, cnt.size() * sizeof(int32_t), cudaMemcpyDeviceToHost);
+        e = cudaMemcpyAsync(cnt.data(), count, cnt.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     std::vector<int64_t> base(size_t(nrb) + 1, 0);
     for (int i = 0; i < nrb; ++i) base[i + 1] = base[i] + cnt[i];
     int64_t *d_base = nullptr;
     uint16_t *list = nullptr;
     unsigned char *pack = nullptr;
     float *diag = nullptr;
-    if (e == cudaSuccess) e = ar.upload(&d_base, base.data(), base.size());
+    if (e == cudaSuccess) e = ar.alloc(&d_base, base.size());
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(d_base, base.data(), base.size() * sizeof(int64_t), cudaMemcpyHostToDevice, st);
+    ar.uploaded += int64_t(base.size() * sizeof(int64_t));
     if (e == cudaSuccess) e = ar.alloc(&list, size_t(base[nrb]));
-    if (e == cudaSuccess) e = ar.alloc(&diag, size_t(N), true);
-    if (e == cudaSuccess) e = ar.alloc(&pack, size_t(base[nrb]) * hy::k::same_block_bytes(), true);
+    if (e == cudaSuccess) e = ar.alloc(&diag, size_t(N));
+    if (e == cudaSuccess) e = zero(diag, size_t(N) * sizeof(float));
+    const size_t bytes = size_t(base[nrb]) * hy::k::same_block_bytes();
+    if (e == cudaSuccess) e = ar.alloc(&pack, bytes);
+    if (e == cudaSuccess && pack) e = zero(pack, bytes);
     if (e == cudaSuccess && pack)
-        e = hy::k::same_fill(M.ptr, M.col, M.val, N, place, d_base, list, pack, diag, nullptr);
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+        e = hy::k::same_fill(M.ptr, M.col, M.val, N, place, d_base, list, pack, diag, st);
+    const cudaError_t done = cudaStreamSynchronize(st);     // the host's buffers are read, tmp is used
+    if (e == cudaSuccess) e = done;
     tmp.release();
     a.N = N;
     a.pack = pack;
@@ -467,23 +478,30 @@ cudaError_t pack_same_spin(const hy_ham *h, int spin, DevArena &ar, hy::k::SameA
 
 // both spins' operands, where the rule of hy_kernels.cuh asks for them: with a
 // Hamiltonian's first float sweep (double users never pay for them, 2 ms and 2 GB at
-// 12,870 strings); not while a stream is being captured.  Without the memory for both,
-// none is kept and the CSR kernel stays in use
-hy_status pack_same(hy_ham *h, cudaStream_t st)
+// 12,870 strings).  Made on a stream of their own that only this waits for, so that they
+// are also made when the sweep is being captured: a graph and the calls beside it have
+// to run the same kernels.  Without the memory for both, none is kept and the CSR kernel
+// stays in use
+hy_status pack_same(hy_ham *h)
 {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
-        return HY_OK;
-    }
     h->same_pairs = hy::k::same_pairs();
     if (h->same_pairs <= 0) return HY_OK;
+    // allocations and waits are allowed to this thread whatever is being captured
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    HY_CUDA(cudaThreadExchangeStreamCaptureMode(&mode), "capture mode");
     DevArena ar;
     hy::k::SameArgs a[2] = {};
-    cudaError_t e = pack_same_spin(h, 0, ar, a[0]);
-    if (e == cudaSuccess && a[0].pack) e = pack_same_spin(h, 1, ar, a[1]);
-    if (e != cudaSuccess || !a[0].pack || !a[1].pack) {
-        ar.release();
+    cudaStream_t st = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+    for (int spin = 0; spin < 2 && e == cudaSuccess; ++spin) {
+        e = pack_same_spin(h, spin, ar, a[spin], st);
+        if (!a[spin].pack) break;
+    }
+    if (st) cudaStreamDestroy(st);
+    const bool both = e == cudaSuccess && a[0].pack && a[1].pack;
+    if (!both) ar.release();
+    const cudaError_t back = cudaThreadExchangeStreamCaptureMode(&mode);
+    if (!both) {
         if (e != cudaSuccess && e != cudaErrorMemoryAllocation) return cuda_fail(e, "same-spin operands");
         cudaGetLastError();
         return HY_OK;
@@ -492,7 +510,7 @@ hy_status pack_same(hy_ham *h, cudaStream_t st)
     h->arena.uploaded += ar.uploaded;
     h->same[0] = a[0];
     h->same[1] = a[1];
-    return HY_OK;
+    return back == cudaSuccess ? HY_OK : cuda_fail(back, "capture mode");
 }
 
 // sigma rows [r0, r1) (alpha strings) of H psi; sigma holds those rows only.
@@ -540,7 +558,7 @@ hy_status apply_h_t(hy_ham *h, const T *psi, T *sigma, cudaStream_t st, int64_t 
     if (tbytes && ensure_ws(h, L.total + std::max(tbytes, xbytes)) == HY_OK) {
         dense = true;
         if (xbytes && h->same_pairs < 0) {
-            hy_status s = pack_same(h, st);
+            hy_status s = pack_same(h);
             if (s != HY_OK) return s;
         }
         same = xbytes && h->same[0].pack && h->same[1].pack;

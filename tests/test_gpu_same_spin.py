@@ -76,3 +76,24 @@ def test_captured_sweep_replays():
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(out, ref)
+
+
+def test_first_tensor_sweep_captured():
+    """The first sweep that asks for the tensor cores may be a captured one (the
+    workspace is there from a sweep on the FP32 pipes): the graph runs the kernels that
+    the calls beside it run, and gives their bits."""
+    hy, ham, psi = _ham((12, 6, 5))
+    out = torch.empty_like(psi)
+    ham.set_coupling("simt")
+    ham.apply_h(psi, out=out)
+    ham.set_coupling("tensor")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        ham.apply_h(psi, out=out)
+    out.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    ref = ham.apply_h(psi)
+    assert torch.equal(out, ref)
+    nb = ham.n_beta_str
+    assert torch.equal(ham.apply_h_rows(psi, 3, 300), out[3 * nb:300 * nb])
