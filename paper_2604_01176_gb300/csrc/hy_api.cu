@@ -2731,6 +2731,7 @@ struct hy::SparseState {
     uint8_t *flags = nullptr;
     unsigned long long *ctr = nullptr;
     void *sup_tables = nullptr;          // its tables in double (SupRowsArgs)
+    bool sup_bare = false;               // they did not fit: done without
 };
 
 namespace {
@@ -3357,22 +3358,30 @@ hy_status sstate_apply_h_support(const SparseState *s, SparseState *sig, void *s
         const size_t nb = size_t(h->Nb), na = size_t(h->Na), nn = size_t(h->n) * h->n;
         const size_t nnz = nb * size_t(hy::k::fold_candidates(h->n, h->nb));
         const size_t tasks = size_t(hy::k::sup_tasks(sig->cap, h->Na));
-        if (!sig->sup_tables) {
+        if (!sig->sup_tables && !sig->sup_bare) {
             const cudaError_t e =
                 cudaMalloc(&sig->sup_tables, tasks * sizeof(int4) + (nnz + nn * nb) * 8 +
                                                  ((64 + 3) * nb + 2 * na) * 4 + nnz * 2);
-            if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(support rows)");
+            if (e != cudaSuccess && e != cudaErrorMemoryAllocation)
+                return cuda_fail(e, "cudaMalloc(support rows)");
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                sig->sup_tables = nullptr;
+                sig->sup_bare = true;
+            }
         }
-        a.tasks = static_cast<int4 *>(sig->sup_tables);
-        a.mval = reinterpret_cast<double *>(a.tasks + tasks);
-        a.dbeta = a.mval + nnz;
-        a.fex = reinterpret_cast<uint32_t *>(a.dbeta + nn * nb);
-        a.number = reinterpret_cast<int32_t *>(a.fex + 64 * nb);
-        a.nfex = a.number + nb;
-        a.nm = a.nfex + nb;
-        a.first = a.nm + nb;
-        a.alist = a.first + na;
-        a.mcol = reinterpret_cast<uint16_t *>(a.alist + na);
+        if (sig->sup_tables) {
+            a.tasks = static_cast<int4 *>(sig->sup_tables);
+            a.mval = reinterpret_cast<double *>(a.tasks + tasks);
+            a.dbeta = a.mval + nnz;
+            a.fex = reinterpret_cast<uint32_t *>(a.dbeta + nn * nb);
+            a.number = reinterpret_cast<int32_t *>(a.fex + 64 * nb);
+            a.nfex = a.number + nb;
+            a.nm = a.nfex + nb;
+            a.first = a.nm + nb;
+            a.alist = a.first + na;
+            a.mcol = reinterpret_cast<uint16_t *>(a.alist + na);
+        }
         HY_CUDA(hy::k::hpsi_support<double>(a, h->num_sms, st), "support H psi");
     } else {
         hy::k::SupRowsArgs<float> a;

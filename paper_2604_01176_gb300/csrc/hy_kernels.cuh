@@ -397,7 +397,7 @@ struct SupRowsArgs {
     uint8_t *flagA, *flagB;
     int32_t *blist;
     unsigned long long *ctr;
-    // double only (else null): by beta string or its number in S (number: Nb, nfex, nm:
+    // double only (first null: without the tables of k_sup_rows): by beta string or its number in S (number: Nb, nfex, nm:
     // Nb; fex: 64 Nb; mcol, mval: Nb times M_beta's longest row; dbeta: n^2 Nb), by
     // alpha string (first, alist: Na), and the tasks (cap / 256 + Na: first row,
     // alpha string, rows)

@@ -427,7 +427,8 @@ k_sup_beta(SupRowsArgs<T> a)
 // feed it.  Measured, 200,000 determinants of 8 + 8 electrons in 16 orbitals, all of it:
 // 1,330 -> 290 us; k_sup_rows 242 (a CTA of 512 threads an SM, whole runs, a row at
 // a time: 285).  The sums are in another order, so float, whose results are kept,
-// stays with the two above.
+// stays with the two above, as does double where there is no memory for the tables
+// (140 MB at 16 orbitals).
 // ---------------------------------------------------------------------------
 constexpr int kSupRowMax = 896;        // entries of an M_alpha row: 849 at most
 
@@ -2447,30 +2448,31 @@ cudaError_t hpsi_support(const SupRowsArgs<T> &a, int num_sms, cudaStream_t st)
                                              a.flagA, a.flagB, a.ctr, a.first);
     hy::count_launch();
     if constexpr (sizeof(T) == 8) {
-        k_sup_number<<<2, 1024, 0, st>>>(a);
-        hy::count_launch();
-        k_sup_tables<<<dim3(unsigned(num_sms) * 2, 2), 256, 0, st>>>(a);
-        hy::count_launch();
-        const size_t sr = sup_rows_smem(h.Nb, h.n * h.n);
-        e = allow_smem(k_sup_rows, sr);
-        if (e != cudaSuccess) return e;
-        k_sup_rows<<<unsigned(num_sms) * 2, kSupTask, sr, st>>>(a);
-        hy::count_launch();
-        return cudaGetLastError();
-    } else {
+        if (a.first) {
+            k_sup_number<<<2, 1024, 0, st>>>(a);
+            hy::count_launch();
+            k_sup_tables<<<dim3(unsigned(num_sms) * 2, 2), 256, 0, st>>>(a);
+            hy::count_launch();
+            const size_t sr = sup_rows_smem(h.Nb, h.n * h.n);
+            e = allow_smem(k_sup_rows, sr);
+            if (e != cudaSuccess) return e;
+            k_sup_rows<<<unsigned(num_sms) * 2, kSupTask, sr, st>>>(a);
+            hy::count_launch();
+            return cudaGetLastError();
+        }
+    }
     k_sup_blist<<<unsigned(num_sms), 256, 0, st>>>(a.flagB, h.Nb, a.blist, a.ctr);
     hy::count_launch();
     const size_t sa = sup_alpha_smem<T>(h.Nb, h.n * h.n), sb = size_t(h.Na) * sizeof(T);
     e = allow_smem(k_sup_alpha<T>, sa);
-    if (e == cudaSuccess)
-        e = allow_smem(k_sup_beta<T>, sb);
+    if (e == cudaSuccess) e = allow_smem(k_sup_beta<T>, sb);
     if (e != cudaSuccess) return e;
-    k_sup_alpha<T><<<unsigned(num_sms) * 2u, kSupThreads, sa, st>>>(a);
+    const unsigned per_sm = sizeof(T) == 8 ? 1u : 2u;
+    k_sup_alpha<T><<<unsigned(num_sms) * per_sm, kSupThreads, sa, st>>>(a);
     hy::count_launch();
-    k_sup_beta<T><<<unsigned(num_sms) * 2u, kSupThreads, sb, st>>>(a);
+    k_sup_beta<T><<<unsigned(num_sms) * per_sm, kSupThreads, sb, st>>>(a);
     hy::count_launch();
     return cudaGetLastError();
-    }
 }
 
 template <typename T>

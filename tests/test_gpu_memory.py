@@ -1,6 +1,8 @@
 """Calls with little device memory left: scratch that does not fit is done without, and
 nothing is held that is not used.  The rest of the device is filled by one tensor.
 """
+import contextlib
+
 import numpy as np
 import pytest
 
@@ -17,10 +19,16 @@ def _free():
     return torch.cuda.mem_get_info()[0]
 
 
+@contextlib.contextmanager
 def _leave(nbytes):
-    """Fills the device up to about nbytes."""
+    """The device filled up to about nbytes."""
     torch.cuda.empty_cache()
-    return torch.empty(_free() - nbytes, dtype=torch.uint8, device="cuda")
+    filler = torch.empty(_free() - nbytes, dtype=torch.uint8, device="cuda")
+    try:
+        yield
+    finally:
+        del filler
+        torch.cuda.empty_cache()
 
 
 def test_same_spin_operands_of_one_spin():
@@ -38,12 +46,41 @@ def test_same_spin_operands_of_one_spin():
     other = hy.Hamiltonian(*synth.integrals(n, 714), n, na, nb)
     # T, 1,001 x 41 x 2,048 floats, and three states beside it
     ws = 1001 * 41 * 2048 * 4 + 3 * ham.n_det * 4
-    filler = _leave(ws + 45 * MB)
-    before = _free()
-    other.apply_h(x, out=out)
-    used = before - _free()
-    del filler
+    with _leave(ws + 45 * MB):
+        before = _free()
+        other.apply_h(x, out=out)
+        used = before - _free()
     tol = 2e-5 * ref.abs().max().item()
     assert (out.double() - ref).abs().max().item() <= tol
     assert ws - 2 * MB <= used <= ws + 12 * MB
     assert torch.equal(other.apply_h(x), out)
+
+
+def test_support_rows_without_tables():
+    """A double sparse evaluation beyond the support programs (16 orbitals, 1 + 8
+    electrons: 140 MB of tables) with 100 MB left.  Tolerances: energies 1e-10,
+    gradients 1e-9, as for the other sparse evaluations."""
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2604_01176_gb300 as hy
+    n, na, nb = 16, 1, 8
+    ham = hy.Hamiltonian(*synth.integrals(n, 900 + n), n, na, nb)
+    pool = hy.Pool(ham)
+    sp = hy.Adapt(ham, pool, "f64", max_iter=160, sparse=True, sparse_cap=ham.n_det)
+    de = hy.Adapt(ham, pool, "f64", max_iter=160)
+    rng = np.random.default_rng(17)
+    for length in range(20, 161, 20):
+        ops = [int(k) for k in rng.choice(len(pool), length)]
+        th = rng.uniform(0.1, 0.7, length)
+        de.set_ansatz(ops, th)
+        ref = de.evaluate(th, torch.float64)
+        if int((de.state(torch.float64) != 0).sum()) > 65536:
+            break
+    else:
+        pytest.fail("no support beyond the programs")
+    sp.set_ansatz(ops, th)
+    with _leave(100 * MB):
+        for _ in range(2):
+            e, g = sp.evaluate(th, torch.float64)
+            assert abs(e - ref[0]) < 1e-10
+            assert np.abs(np.asarray(g) - np.asarray(ref[1])).max() < 1e-9
