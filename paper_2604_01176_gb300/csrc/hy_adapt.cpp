@@ -151,6 +151,7 @@ hy_status set_err(hy_status s, const char *msg);
 hy_status cu(cudaError_t e, const char *what)
 {
     if (e == cudaSuccess) return HY_OK;
+    cudaGetLastError();         // reported: the check after the next launch is not to find it
     return set_err(e == cudaErrorMemoryAllocation ? HY_ERR_OOM : HY_ERR_CUDA, what);
 }
 

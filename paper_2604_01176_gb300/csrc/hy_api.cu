@@ -31,6 +31,7 @@ hy_status fail(hy_status s, const std::string &msg)
 hy_status cuda_fail(cudaError_t e, const char *what)
 {
     g_err = std::string(what) + ": " + cudaGetErrorString(e);
+    cudaGetLastError();         // reported: the check after the next launch is not to find it
     return e == cudaErrorMemoryAllocation ? HY_ERR_OOM : HY_ERR_CUDA;
 }
 
@@ -2189,11 +2190,10 @@ hy_status ensure_tw(hy_ham *h, int64_t cap)
     h->tw.w = nullptr;
     h->tw.cap = 0;
     cudaError_t e = cudaSuccess;
-    if (!h->tw.cnt) {
-        e = cudaMalloc(&h->tw.cnt, size_t(h->Na + 1) * sizeof(int32_t));
-        if (e == cudaSuccess) e = cudaMalloc(&h->tw.ptr, size_t(h->Na + 1) * sizeof(int32_t));
-        if (e == cudaSuccess) e = cudaMalloc(&h->tw.cur, size_t(h->Na) * sizeof(int32_t));
-    }
+    // each by itself: an earlier call may have got only some of them
+    if (!h->tw.cnt) e = cudaMalloc(&h->tw.cnt, size_t(h->Na + 1) * sizeof(int32_t));
+    if (e == cudaSuccess && !h->tw.ptr) e = cudaMalloc(&h->tw.ptr, size_t(h->Na + 1) * sizeof(int32_t));
+    if (e == cudaSuccess && !h->tw.cur) e = cudaMalloc(&h->tw.cur, size_t(h->Na) * sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMalloc(&h->tw.mask, size_t(cap) * sizeof(uint32_t));
     if (e == cudaSuccess) e = cudaMalloc(&h->tw.w, size_t(cap) * sizeof(float));
     if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(row groups)");
@@ -3329,14 +3329,14 @@ hy_status sstate_apply_h_support(const SparseState *s, SparseState *sig, void *s
                             cudaMemcpyDeviceToDevice, st), "copy bitmap");
     HY_CUDA(hy::k::bits_compact(sig->bits, sig->words, sig->list, sig->cap, sig->cnt, sig->blk, st),
             "support list");
-    if (!sig->runs) {
-        cudaError_t e = cudaMalloc(&sig->runs, size_t(h->Na) * sizeof(int64_t));
-        if (e == cudaSuccess) e = cudaMalloc(&sig->ralpha, size_t(h->Na) * sizeof(int32_t));
-        if (e == cudaSuccess) e = cudaMalloc(&sig->blist, size_t(h->Nb) * sizeof(int32_t));
-        if (e == cudaSuccess) e = cudaMalloc(&sig->flags, size_t(h->Na + h->Nb));
-        if (e == cudaSuccess) e = cudaMalloc(&sig->ctr, 4 * sizeof(unsigned long long));
-        if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(support rows)");
-    }
+    // each by itself: an earlier call may have got only some of them
+    cudaError_t e = cudaSuccess;
+    if (!sig->runs) e = cudaMalloc(&sig->runs, size_t(h->Na) * sizeof(int64_t));
+    if (e == cudaSuccess && !sig->ralpha) e = cudaMalloc(&sig->ralpha, size_t(h->Na) * sizeof(int32_t));
+    if (e == cudaSuccess && !sig->blist) e = cudaMalloc(&sig->blist, size_t(h->Nb) * sizeof(int32_t));
+    if (e == cudaSuccess && !sig->flags) e = cudaMalloc(&sig->flags, size_t(h->Na + h->Nb));
+    if (e == cudaSuccess && !sig->ctr) e = cudaMalloc(&sig->ctr, 4 * sizeof(unsigned long long));
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(support rows)");
     auto run = [&](auto &a) {
         a.list = sig->list;
         a.cnt = sig->cnt;
@@ -3359,8 +3359,7 @@ hy_status sstate_apply_h_support(const SparseState *s, SparseState *sig, void *s
         const size_t nnz = nb * size_t(hy::k::fold_candidates(h->n, h->nb));
         const size_t tasks = size_t(hy::k::sup_tasks(sig->cap, h->Na));
         if (!sig->sup_tables && !sig->sup_bare) {
-            const cudaError_t e =
-                cudaMalloc(&sig->sup_tables, tasks * sizeof(int4) + (nnz + nn * nb) * 8 +
+            e = cudaMalloc(&sig->sup_tables, tasks * sizeof(int4) + (nnz + nn * nb) * 8 +
                                                  ((64 + 3) * nb + 2 * na) * 4 + nnz * 2);
             if (e != cudaSuccess && e != cudaErrorMemoryAllocation)
                 return cuda_fail(e, "cudaMalloc(support rows)");

@@ -1038,6 +1038,7 @@ hy_status rerr(hy_status s, const std::string &m)
 hy_status rcu(cudaError_t e, const char *what)
 {
     if (e == cudaSuccess) return HY_OK;
+    cudaGetLastError();         // reported: the check after the next launch is not to find it
     return rerr(e == cudaErrorMemoryAllocation ? HY_ERR_OOM : HY_ERR_CUDA,
                 std::string(what) + ": " + cudaGetErrorString(e));
 }
@@ -1059,6 +1060,7 @@ hy_status ensure_act(hy_ranker *r, int64_t rows)
     }
     cudaFree(r->idx);
     r->idx = nullptr;
+    r->act_rows = 0;            // until all of them are there
     const size_t R = size_t(rows);
     RTRY(rcu(cudaMalloc(&r->xb, R * r->F * 4), "ranker buffers"));
     RTRY(rcu(cudaMalloc(&r->yb, R * 4), "ranker buffers"));

@@ -84,3 +84,20 @@ def test_support_rows_without_tables():
             e, g = sp.evaluate(th, torch.float64)
             assert abs(e - ref[0]) < 1e-10
             assert np.abs(np.asarray(g) - np.asarray(ref[1])).max() < 1e-9
+
+
+def test_ranker_buffers_half_allocated():
+    """A fit whose batch does not fit leaves the ranker able to predict."""
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2604_01176_gb300 as hy
+    r = hy.Ranker(hidden=600, seed=3)
+    x = torch.from_numpy(np.random.default_rng(1).standard_normal((4096, 16)).astype(np.float32)).cuda()
+    ref = r.predict(x)
+    r.add_samples(x, x[:, 0].double().contiguous())
+    with _leave(700 * MB):
+        with pytest.raises(hy.HyError) as ei:
+            r.fit(epochs=1, batch=1 << 17)
+        assert ei.value.status == 3
+        assert torch.equal(r.predict(x), ref)
+    assert torch.equal(r.predict(x), ref)
