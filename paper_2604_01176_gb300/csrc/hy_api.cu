@@ -140,6 +140,7 @@ struct hy_ham {
     // null: the CSR kernel runs), by spin, and the CTA pairs that run at once
     hy::k::SameArgs same[2] = {};
     int same_pairs = -1;            // not tried yet: made by the first float sweep
+    int8_t dense_fits[2] = {-1, -1};    // double, float: dense_fits of hy_dense.cu, -1 not asked yet
     double *d_V64 = nullptr;
     float *d_V32 = nullptr;
     double *d_h1 = nullptr, *d_eri = nullptr;   // integrals (ranker features)
@@ -1755,7 +1756,12 @@ bool dense_chain_ok(const hy_ham *h, hy_dtype dt, int64_t L)
     if (h->N > k::kDenseMaxN || L > k::kDenseMaxOps) return false;
     // float: one operator's screen deals its rows to 4 chunks per SM of 256
     // columns, so up to these counts no thread of it adds two pairs in float
-    return dt == HY_F64 || (h->Na <= int64_t(4) * h->num_sms && h->Nb <= 256);
+    if (dt == HY_F32 && (h->Na > int64_t(4) * h->num_sms || h->Nb > 256)) return false;
+    int8_t &fits = const_cast<hy_ham *>(h)->dense_fits[dt == HY_F32];
+    if (fits < 0)
+        fits = dt == HY_F64 ? k::dense_fits<double>(int(h->Na), int(h->Nb))
+                            : k::dense_fits<float>(int(h->Na), int(h->Nb));
+    return fits != 0;
 }
 
 namespace {

@@ -332,37 +332,79 @@ int dense_shift(const DensePool &p)
 
 namespace {
 // one cluster of kDenseCtas CTAs (beyond the portable eight: opted into)
-template <typename... P, typename... A>
-cudaError_t launch_cluster(void (*kernel)(P...), size_t smem, cudaStream_t st, A... args)
+template <typename... P>
+cudaError_t cluster_config(void (*kernel)(P...), size_t smem, cudaLaunchAttribute &at,
+                           cudaLaunchConfig_t &cfg)
 {
     cudaError_t e = allow_smem(kernel, smem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeClusterDimension;
     at.val.clusterDim.x = kDenseCtas;
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(kDenseCtas);
     cfg.blockDim = dim3(kDenseThreads);
     cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
+    return e;
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_cluster(void (*kernel)(P...), size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute at{};
+    cudaLaunchConfig_t cfg{};
+    cudaError_t e = cluster_config(kernel, smem, at, cfg);
+    if (e != cudaSuccess) return e;
+    cfg.stream = st;
     e = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
     hy::count_launch();
     return e;
 }
+
+template <typename... P>
+bool cluster_fits(void (*kernel)(P...), size_t smem)
+{
+    cudaLaunchAttribute at{};
+    cudaLaunchConfig_t cfg{};
+    int n = 0;
+    if (cluster_config(kernel, smem, at, cfg) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess)
+        return n > 0;
+    cudaGetLastError();
+    return false;
+}
+
+template <typename T>
+size_t prepare_smem(int L, int shift)
+{
+    return size_t(L) * 2 * sizeof(DenseStep<T>) + (size_t(1) << shift) * sizeof(T);
+}
+template <typename T>
+size_t gradient_smem(int L, int shift)
+{
+    return size_t(L) * (32 * sizeof(double) + 4 * sizeof(DenseStep<T>)) + (size_t(2) << shift) * sizeof(T);
+}
 }  // namespace
+
+template <typename T>
+bool dense_fits(int Na, int Nb)
+{
+    DensePool p{};
+    p.Na = Na;
+    p.Nb = Nb;
+    const int shift = dense_shift(p);
+    return cluster_fits(k_dense_prepare<T>, prepare_smem<T>(kDenseMaxOps, shift)) &&
+           cluster_fits(k_dense_gradient<T>, gradient_smem<T>(kDenseMaxOps, shift));
+}
 
 template <typename T>
 cudaError_t dense_prepare(const DensePool &p, const int32_t *ops, const double *cs, int L, T *psi,
                           double *norm2, cudaStream_t st)
 {
     const int shift = dense_shift(p);
-    const size_t smem = size_t(L) * 2 * sizeof(DenseStep<T>) + (size_t(1) << shift) * sizeof(T);
-    return launch_cluster(k_dense_prepare<T>, smem, st, p, ops, cs, L, psi, norm2, shift);
+    return launch_cluster(k_dense_prepare<T>, prepare_smem<T>(L, shift), st, p, ops, cs, L, psi, norm2, shift);
 }
 
 template <typename T>
@@ -370,11 +412,11 @@ cudaError_t dense_gradient(const DensePool &p, const int32_t *ops, const double 
                            const T *psi, const T *sigma, double *g, cudaStream_t st)
 {
     const int shift = dense_shift(p);
-    const size_t smem = size_t(L) * (32 * sizeof(double) + 4 * sizeof(DenseStep<T>)) +
-                        (size_t(2) << shift) * sizeof(T);
-    return launch_cluster(k_dense_gradient<T>, smem, st, p, ops, cs, L, psi, sigma, g, shift);
+    return launch_cluster(k_dense_gradient<T>, gradient_smem<T>(L, shift), st, p, ops, cs, L, psi, sigma, g, shift);
 }
 
+template bool dense_fits<double>(int, int);
+template bool dense_fits<float>(int, int);
 template cudaError_t dense_prepare<double>(const DensePool &, const int32_t *, const double *, int,
                                            double *, double *, cudaStream_t);
 template cudaError_t dense_prepare<float>(const DensePool &, const int32_t *, const double *, int,

@@ -147,8 +147,9 @@ class ProfScope {
 
 // The rotations of an ansatz on a small dense state, and its gradient, in one
 // launch each (hy_dense.cu); false where the per-rotation launches serve:
-// more than kDenseMaxN determinants, a longer ansatz, or float string counts
-// whose per-operator screens add several pairs in float
+// more than kDenseMaxN determinants, a longer ansatz, float string counts whose
+// per-operator screens add several pairs in float, or a device (an SM partition) that
+// cannot place a cluster of 16 CTAs
 bool dense_chain_ok(const hy_ham *h, hy_dtype dt, int64_t L);
 hy_status dense_chain_prepare(const hy_ham *h, const hy_pool *p, const int32_t *ops,
                               const double *cs, int64_t L, void *psi, hy_dtype dt, double *norm2,

@@ -274,6 +274,10 @@ struct DensePool {
     const int64_t *aoff, *acnt, *boff, *bcnt;
     int Na, Nb;
 };
+// whether the device at hand (or the part of it that the process has) can place a
+// cluster of either launch at its largest
+template <typename T>
+bool dense_fits(int Na, int Nb);
 template <typename T>
 cudaError_t dense_prepare(const DensePool &p, const int32_t *ops, const double *cs, int L, T *psi,
                           double *norm2, cudaStream_t st);

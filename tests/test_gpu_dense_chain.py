@@ -61,3 +61,31 @@ def test_chain_matches_single_calls(cfg, precision, kind):
         pool.apply_excitation(int(ops[l]), -float(th[l]), phi)
         pool.apply_excitation(int(ops[l]), -float(th[l]), lam)
     assert np.abs(g - ref).max(initial=0.0) <= tol * scale
+
+
+@pytest.mark.parametrize("precision", ["f64", "mixed"])
+@pytest.mark.parametrize("cfg", [(6, 3, 3), (8, 4, 4), (10, 5, 5)], ids=lambda c: "n%da%db%d" % c)
+def test_longest_ansatz_of_one_launch(cfg, precision):
+    """192 operators are walked in one launch each way (its largest shared memory), 193 by
+    the per-rotation launches; a last operator at angle 0 changes neither the energy
+    nor the other derivatives."""
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2604_01176_gb300 as hy
+    n, na, nb = cfg
+    ham = hy.Hamiltonian(*synth.integrals(n, 90 + n), n, na, nb)
+    pool = hy.Pool(ham)
+    rng = np.random.default_rng(n)
+    ops = rng.integers(0, len(pool), 193)
+    th = np.append(0.1 * rng.standard_normal(192), 0.0)
+    dt = torch.float64 if precision == "f64" else torch.float32
+    ad = hy.Adapt(ham, pool, precision, max_iter=193)
+    got = []
+    for length in (192, 193):
+        ad.set_ansatz(ops[:length], th[:length])
+        got.append(ad.evaluate(th[:length], dt))
+    (e1, g1), (e2, g2) = got
+    tol = 1e-12 if precision == "f64" else 1e-5
+    scale = max(1.0, abs(e1))
+    assert abs(e1 - e2) <= tol * scale
+    assert np.abs(g1 - g2[:192]).max() <= tol * scale
