@@ -785,10 +785,23 @@ hy_status build_screen_plan(ScreenPlan &sp, const hy_pool *const *pools, const i
         total += double(pools[m]->sing[0].size()) * double(k[0].groups) * k[0].cost;
         for (int j = 1; j < 4; ++j) total += double(k[j].groups) * k[j].cost;
     }
-    const double per_task = std::max(total / (8.0 * num_sms), 1.0);
+    // a task of a few hundred pairs is all latency: small totals are dealt to fewer (20
+    // molecules of 6 orbitals 56 -> 34 us, per operator 49; 3 of 8 orbitals 51 -> 39, 62)
+    const double per_task = std::max(total / (8.0 * num_sms), std::min(total / 64.0, 1024.0));
     auto deal = [&](const Kind &k) {
         const int64_t c = int64_t(std::ceil(double(k.groups) * k.cost / per_task));
         return int(std::max<int64_t>(1, std::min(c, k.groups)));
+    };
+    // Few strings of one spin make few groups of the other's patterns, each of them a long
+    // task (16 orbitals, 1 + 8 electrons: 16 rows of 784 doubles x 924 pairs).  A kind that
+    // is dealt a group a task and has more than half an SM's share in one is cut by
+    // pattern as well, as long as a slice sums as much as it stages: 16 x 12,870 strings
+    // 1,890 -> 150 us, 66 x 924 64 -> 45, 78 x 1,716 129 -> 80
+    const double half = total / (2.0 * num_sms);
+    auto slices = [&](const Kind &k, int ch, int64_t patterns, double staged) {
+        if (ch < k.groups || patterns < 2) return 1;
+        const double most = std::min(double(patterns), (k.cost - staged) / staged);
+        return int(std::max(1.0, std::min(std::ceil(k.cost / half), most)));
     };
     for (int m : order) {
         const hy_pool *p = pools[m];
@@ -808,19 +821,28 @@ hy_status build_screen_plan(ScreenPlan &sp, const hy_pool *const *pools, const i
         q.nA = int(p->sing[0].size()); q.nB = int(p->sing[1].size());
         q.nRa = int(p->dbl[0].size()); q.nRb = int(p->dbl[1].size());
         // the identity (first in the list, a few times a single's pairs) shares
-        // the singles' chunk count
+        // the singles' chunk count, unless its tasks are long then
         q.ch[0] = q.nA ? deal(k[0]) : deal(k[1]);
+        q.chi = double(k[1].groups) * k[1].cost > half * q.ch[0] ? deal(k[1]) : q.ch[0];
+        q.zs[0] = slices(k[0], q.ch[0], q.nB, 2.0 * double(h->Nb));
+        q.zs[1] = slices(k[1], q.chi, q.nB, 2.0 * double(h->Nb));
         q.base[0] = sp.n_partials;
-        sp.n_partials += int64_t(q.nA + 1) * q.ch[0] * (q.nB + 1);
-        for (int ia = q.nA; ia >= 0; --ia)
-            for (int c = 0; c < q.ch[0]; ++c) tasks.push_back(make_int4(m, 0, ia, c));
+        sp.n_partials += (int64_t(q.nA) * q.ch[0] + q.chi) * (q.nB + 1);
+        for (int ia = q.nA; ia >= 0; --ia) {
+            const int ch = ia == q.nA ? q.chi : q.ch[0], zs = q.zs[ia == q.nA ? 1 : 0];
+            for (int c = 0; c < ch * zs; ++c) tasks.push_back(make_int4(m, 0, ia, c / zs | c % zs << 16));
+        }
         sp.smem = std::max(sp.smem, size_t(2) * q.Nb * (sp.cfg < 2 ? 16 : 8));
         for (int kind = 1; kind <= 2; ++kind) {
             const int nr = kind == 1 ? q.nRa : q.nRb;
             q.ch[kind] = nr ? deal(k[kind + 1]) : 0;
+            const int zs = q.zs[kind + 1] =
+                nr ? slices(k[kind + 1], q.ch[kind], nr,
+                            2.0 * double(Q) * double(kind == 1 ? h->Na : h->Nb)) : 1;
             q.base[kind] = sp.n_partials;
             sp.n_partials += int64_t(q.ch[kind]) * nr;
-            for (int c = 0; c < q.ch[kind]; ++c) tasks.push_back(make_int4(m, kind, 0, c));
+            for (int c = 0; c < q.ch[kind] * zs; ++c)
+                tasks.push_back(make_int4(m, kind, 0, c / zs | c % zs << 16));
             if (nr)
                 sp.smem = std::max(sp.smem, size_t(Q) * (kind == 1 ? q.Na : q.Nb) * 16 +
                                                 size_t(nr + 3) / 4 * 32);
@@ -854,10 +876,18 @@ int beta_single_pairs(const hy_pool *p)
     return p->sing[1].empty() ? 0 : int(p->pb.cnt[p->sing[1][0]]);
 }
 
-// whether whole pools of this molecule alone are screened by pattern
+// whether whole pools of this molecule alone are screened by pattern.  In double not
+// where the narrow planes meet some hundred alpha strings (two electrons or holes in 16
+// orbitals beside 7 to 9): one CTA an SM then, for a state that L2 holds for the
+// per-operator kernel (120 x 12,870 strings 1,750 us, per operator 1,550 and, qubit
+// pool, 1,320; 16 x 12,870 150 against 188 and 172; 560 x 12,870 5,790 against 9,340 and
+// 7,790; 120 x 8,008 787 against 898 and 747)
 bool screen_by_pattern(const hy_pool *p, bool f32)
 {
-    return p->h->N >= hy::k::kScreenMinN && (!f32 || beta_single_pairs(p) <= hy::k::kScreen32MaxPairs);
+    const hy_ham *h = p->h;
+    if (h->N < hy::k::kScreenMinN) return false;
+    if (f32) return beta_single_pairs(p) <= hy::k::kScreen32MaxPairs;
+    return !(p->screen.cfg == 2 && h->Nb > 10000 && h->Na > 64 && h->Na < 256);
 }
 
 // partial sums of the float screen of a whole pool

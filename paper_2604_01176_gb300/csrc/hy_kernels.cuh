@@ -704,12 +704,15 @@ struct ScreenMol {
     int64_t off;                                 // first amplitude of psi and sigma
     int64_t gbase;                               // first operator in g
     int64_t base[3];                             // partials of each kind
-    int ch[3];                                   // tasks a kind's groups are dealt to
+    // tasks that the groups of a kind are dealt to (kind 0: of an alpha single, and
+    // of the alpha identity), and slices of its patterns that each of them is cut in:
+    // alpha singles, alpha identity, alpha doubles, beta doubles
+    int ch[3], chi, zs[4];
     int Na, Nb, nA, nB, nRa, nRb;
 };
 struct ScreenArgs {
     const ScreenMol *mols;
-    const int4 *tasks;                           // (molecule, kind, alpha pattern, chunk)
+    const int4 *tasks;                           // (molecule, kind, alpha pattern, chunk | slice << 16)
     const double *psi, *sigma;
     double *partials;
 };

@@ -112,7 +112,8 @@ __device__ __forceinline__ void stage_ab(double *p1, double *p2, const double *p
 
 // kind 0: alpha-beta task (idx = alpha pattern, nA = the identity); kind 1:
 // alpha doubles over columns; kind 2: beta doubles over rows.  chunk: the
-// task's groups are chunk, chunk + CH, ...
+// task's groups are chunk, chunk + CH, ...; slice: its share of the patterns (one
+// slice unless the groups are too few)
 template <int CFG>
 __global__ void __launch_bounds__(kScThreads, 2)
 k_screen(ScreenArgs a)
@@ -124,30 +125,33 @@ k_screen(ScreenArgs a)
     const ScreenMol &m = a.mols[tk.x];
     const double *psi = a.psi + m.off, *sig = a.sigma + m.off;
     const int Na = m.Na, Nb = m.Nb;
-    const int kind = tk.y, chunk = tk.w, CH = m.ch[kind];
+    const int kind = tk.y, chunk = tk.w & 0xFFFF, slice = tk.w >> 16;
 
     if (kind == 0) {
         using U = std::conditional_t<CFG == 2, double, double2>;
         U *p1 = reinterpret_cast<U *>(smem_raw), *p2 = p1 + Nb;
         const int ia = tk.z;
         const bool ident = ia == m.nA;
+        const int CH = ident ? m.chi : m.ch[0], Z = m.zs[ident ? 1 : 0];
         const int cnt = ident ? Na : int(m.acnt[m.la[ia]]);
         const uint32_t *ae = ident ? nullptr : m.aent + m.aoff[m.la[ia]];
-        // this warp's share [lo, hi) of the beta singles' pairs, cut by pattern
+        // this warp's share [lo, hi) of the pairs of the slice's beta singles [b0, b1),
+        // cut by pattern
         const uint32_t *bent = m.bent;
         const int nB = m.nB, cb = nB > 0 ? int(m.bcnt[m.lb[0]]) : 0;
-        const int tot = nB * cb;
-        const int lo = int(int64_t(tot) * warp / kScWarps);
-        const int hi = int(int64_t(tot) * (warp + 1) / kScWarps);
+        const int b0 = nB * slice / Z, b1 = nB * (slice + 1) / Z;
+        const int tot = (b1 - b0) * cb;
+        const int lo = b0 * cb + int(int64_t(tot) * warp / kScWarps);
+        const int hi = b0 * cb + int(int64_t(tot) * (warp + 1) / kScWarps);
         int so[kScSeg];
         int sn[kScSeg];
         const int first = cb > 0 ? lo / cb : 0;
 #pragma unroll
         for (int s = 0; s < kScSeg; ++s) {
             const int p = first + s;
-            const int b0 = max(lo, p * cb), b1 = min(hi, (p + 1) * cb);
-            sn[s] = p < nB && b1 > b0 ? b1 - b0 : 0;
-            so[s] = sn[s] ? int(m.boff[m.lb[p]]) + (b0 - p * cb) : 0;
+            const int e0 = max(lo, p * cb), e1 = min(hi, (p + 1) * cb);
+            sn[s] = p < b1 && e1 > e0 ? e1 - e0 : 0;
+            so[s] = sn[s] ? int(m.boff[m.lb[p]]) + (e0 - p * cb) : 0;
         }
         double acc[kScSeg], aid = 0.0;
 #pragma unroll
@@ -163,7 +167,7 @@ k_screen(ScreenArgs a)
 #pragma unroll
                 for (int s = 0; s < kScSeg; ++s)
                     if (sn[s]) sum_pairs<U, 1, 32>(acc[s], bent + so[s], sn[s], lane, p1, p2, 0);
-                if (!ident)
+                if (!ident && slice == 0)
                     for (int b = tid; b < Nb; b += kScThreads) term(aid, p1[b], p2[b], 0u);
             }
         }
@@ -177,14 +181,16 @@ k_screen(ScreenArgs a)
         const double v = warp_total(aid);
         if (lane == 0) red[warp][kScSeg] = v;
         __syncthreads();
-        double *out = a.partials + m.base[0] + (int64_t(ia) * CH + chunk) * (nB + 1);
-        for (int p = tid; p <= nB; p += kScThreads) {
+        double *out = a.partials + m.base[0] + (int64_t(ia) * m.ch[0] + chunk) * (nB + 1);
+        for (int i = tid; i <= b1 - b0; i += kScThreads) {
+            const int p = i < b1 - b0 ? b0 + i : nB;
+            if (p == nB && slice) break;
             double s = 0.0;
             if (p == nB) {
                 for (int w = 0; w < kScWarps; ++w) s += red[w][kScSeg];
             } else {
                 for (int w = 0; w < kScWarps; ++w) {
-                    const int l = int(int64_t(tot) * w / kScWarps);
+                    const int l = b0 * cb + int(int64_t(tot) * w / kScWarps);
                     const int q = p - l / cb;       // segment of warp w for pattern p
                     if (q >= 0 && q < kScSeg) s += red[w][q];
                 }
@@ -197,11 +203,13 @@ k_screen(ScreenArgs a)
     // same-spin doubles: V vectors of Ns amplitudes, element s of vector v at
     // v * vst + s * sst
     constexpr int Q = CFG == 0 ? 4 : CFG == 1 ? 2 : 1;      // vectors per group
+    const int CH = m.ch[kind], Z = m.zs[kind + 1];
     const bool al = kind == 1;
     const int Ns = al ? Na : Nb, V = al ? Nb : Na;
     const int64_t sst = al ? Nb : 1, vst = al ? 1 : Nb;
-    const int nR = al ? m.nRa : m.nRb;
-    const int32_t *ids = al ? m.ra : m.rb;
+    const int nAll = al ? m.nRa : m.nRb;
+    const int r0 = int(int64_t(nAll) * slice / Z), nR = int(int64_t(nAll) * (slice + 1) / Z) - r0;
+    const int32_t *ids = (al ? m.ra : m.rb) + r0;
     const uint32_t *ent = al ? m.aent : m.bent;
     const int64_t *off = al ? m.aoff : m.boff, *cnts = al ? m.acnt : m.bcnt;
     double2 *pl = reinterpret_cast<double2 *>(smem_raw);                // [Q][Ns]
@@ -231,7 +239,7 @@ k_screen(ScreenArgs a)
         }
     }
     __syncthreads();
-    double *out = a.partials + m.base[kind] + int64_t(chunk) * nR;
+    double *out = a.partials + m.base[kind] + int64_t(chunk) * nAll + r0;
     for (int i = tid; i < nR; i += kScThreads) out[i] = acc[i];
 }
 
@@ -260,9 +268,9 @@ k_screen_final(const ScreenMol *__restrict__ mols, int count, const double *__re
         int64_t stride;
         int ch;
         if (sa >= 0 && sb >= 0) {
-            ch = m.ch[0];
+            ch = sa == m.nA ? m.chi : m.ch[0];
             stride = m.nB + 1;
-            p = partials + m.base[0] + int64_t(sa) * ch * stride + sb;
+            p = partials + m.base[0] + int64_t(sa) * m.ch[0] * stride + sb;
         } else if (sa < 0) {
             ch = m.ch[1];
             stride = m.nRa;

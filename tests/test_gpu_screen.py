@@ -111,3 +111,27 @@ def test_float_pool_keeps_the_operator_lists_sums(cfg, kind):
     pool.gradients(psi, sigma, out=whole)
     listed = pool.gradients(psi, sigma, ops=every)
     assert torch.max(torch.abs(whole - listed)).item() <= 1e-13
+
+
+@pytest.mark.parametrize("kind", ["sd", "qeb"])
+@pytest.mark.parametrize("cfg", [(16, 1, 8), (16, 15, 8), (16, 8, 1), (16, 2, 8), (13, 11, 6), (12, 2, 6), (16, 3, 4),
+                                 (15, 1, 9)], ids=lambda c: "n%da%db%d" % c)
+def test_few_strings_of_a_spin(cfg, kind):
+    """Few strings of one spin: the other's patterns are cut in slices as well (16,384
+    determinants and more, so alone the pool takes the screen by pattern)."""
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2604_01176_gb300 as hy
+    n, na, nb = cfg
+    ham = hy.Hamiltonian(*synth.integrals(n, 50 + n), n, na, nb)
+    assert ham.n_det >= 16384
+    pool = hy.Pool(ham, kind)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    v = torch.randn((2, ham.n_det), dtype=torch.float64, device="cuda", generator=g)
+    psi, sigma = v[0] / v[0].norm(), v[1] / v[1].norm()
+    every = torch.arange(len(pool), dtype=torch.int32, device="cuda")
+    whole = torch.full((len(pool),), np.nan, dtype=torch.float64, device="cuda")
+    pool.gradients(psi, sigma, out=whole)
+    listed = pool.gradients(psi, sigma, ops=every)
+    assert torch.max(torch.abs(whole - listed)).item() <= 1e-12
