@@ -773,7 +773,11 @@ cudaError_t gemm(const float *A, const float *B, float *C, int M, int N, int Kd,
 // Bound: the weights' way from L2 (0.5 MB a block) and, layer by layer, the
 // launches it replaces: four k_gemm of 1,107 rows 81 us, 34 here (99 with a
 // shared load per product and tiles fetched when needed).
-constexpr int kMlpRows = 8, kMlpTile = 32, kMlpMaxHidden = 512;
+// Beyond 256 units a thread has two, and a block of 8 rows alone takes 43 (288 units)
+// to 95 us (512): up to kMlpWideRows rows the four products, whose time grows with the
+// rows, are quicker (512 units: 8 rows 48 us, 256 rows 90, 384 rows 116; 288 units: 31,
+// 40, 50).  Up to 256 units a block takes 31 us, and the products no less.
+constexpr int kMlpRows = 8, kMlpTile = 32, kMlpMaxHidden = 512, kMlpWideRows = 256;
 
 __host__ __device__ constexpr size_t mlp_smem(int H)
 {
@@ -1192,8 +1196,8 @@ hy_status hy_ranker_predict(hy_ranker *r, const float *feat, int64_t m, float *s
 {
     if (!r || (m > 0 && (!feat || !score)) || m < 0) return rerr(HY_ERR_ARG, "bad arguments");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (r->H >= r->F && r->H <= hy::k::kMlpMaxHidden) {
-        if (m == 0) return HY_OK;
+    if (m == 0) return HY_OK;
+    if (r->H >= r->F && (r->H <= 256 || (r->H <= hy::k::kMlpMaxHidden && m > hy::k::kMlpWideRows))) {
         hy::k::MlpWeights p;
         for (int l = 0; l < 4; ++l) {
             p.w[l] = r->w + r->woff[l];

@@ -61,3 +61,17 @@ def test_two_vectors_share_launches(cfg):
     d1, d2 = hy.touched_weights(ham, psi), hy.touched_weights(ham, sigma)
     w1, w2 = d1[0, 0].item(), d2[0, 0].item()
     assert abs(w1 - 1.0) <= 1e-5 and abs(w2 - 1.0) <= 1e-5
+
+
+@pytest.mark.parametrize("hidden", [257, 384, 512])
+@pytest.mark.parametrize("rows", [1, 255, 256, 257, 300])
+def test_wide_network_few_rows(hidden, rows):
+    """Beyond 256 units, up to 256 rows go through the products and more through the one
+    launch: a row's score is the same bits in either (the first rows of 300 and of 257
+    against the same rows alone)."""
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2604_01176_gb300 as hy
+    r = hy.Ranker(hidden=hidden, seed=3)
+    x = torch.from_numpy(np.random.default_rng(5).standard_normal((300, 16)).astype(np.float32)).cuda()
+    assert torch.equal(r.predict(x[:rows].contiguous()), r.predict(x)[:rows])
