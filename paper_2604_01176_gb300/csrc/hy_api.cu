@@ -80,6 +80,32 @@ struct DevArena {
     }
 };
 
+// several arrays in one allocation and one copy (each allocation and each copy costs
+// about 10 us)
+struct DevPack {
+    std::vector<unsigned char> host;
+    size_t extra = 0;            // bytes behind them that are not copied
+    template <typename T>
+    size_t add(const T *src, size_t count)
+    {
+        const size_t at = (host.size() + 15) / 16 * 16;
+        host.resize(at + count * sizeof(T));
+        if (count) std::memcpy(host.data() + at, src, count * sizeof(T));
+        return at;
+    }
+    template <typename T>
+    size_t add(const std::vector<T> &v) { return add(v.data(), v.size()); }
+    // where the bytes not copied start
+    size_t end() const { return (host.size() + 15) / 16 * 16; }
+    cudaError_t upload(DevArena &ar, unsigned char **base) const
+    {
+        const cudaError_t e = ar.alloc(base, end() + extra);
+        if (e != cudaSuccess || host.empty()) return e;
+        ar.uploaded += int64_t(host.size());
+        return cudaMemcpy(*base, host.data(), host.size(), cudaMemcpyHostToDevice);
+    }
+};
+
 template <typename T>
 struct DevCsr {
     int32_t *ptr = nullptr, *col = nullptr;
@@ -182,6 +208,8 @@ namespace {
 // when a pool is created or a batch given its pools.
 struct ScreenPlan {
     DevArena arena;
+    unsigned char *block = nullptr;     // mols, tasks, partials
+    size_t block_bytes = 0;
     hy::k::ScreenMol *d_mols = nullptr;
     int4 *d_tasks = nullptr;
     double *d_partials = nullptr;
@@ -236,6 +264,7 @@ struct hy_batch {
     int64_t n_tasks64 = 0;
     size_t smem64 = 0;
     int64_t *d_base64 = nullptr, *d_rows64n = nullptr;   // row_energy spans per molecule
+    DevArena tables64;              // all of these
     int *d_counter = nullptr;
     double *d_row_energy = nullptr;
     int64_t *d_base = nullptr, *d_rows = nullptr;
@@ -741,8 +770,13 @@ hy_status energy_t(hy_ham *h, const T *psi, const T *sigma, double *e, cudaStrea
 hy_status build_screen_plan(ScreenPlan &sp, const hy_pool *const *pools, const int64_t *offs,
                             const int64_t *gbase, int count, int num_sms)
 {
-    sp.arena.release();
+    // a plan made anew keeps its memory (what is queued on it ends first)
+    ScreenPlan old = std::move(sp);
     sp = ScreenPlan{};
+    sp.arena = std::move(old.arena);
+    sp.block = old.block;
+    sp.block_bytes = old.block_bytes;
+    if (sp.block) HY_CUDA(cudaDeviceSynchronize(), "screen plan in use");
     int64_t M = 0, nR = 0;
     for (int m = 0; m < count; ++m) {
         M = std::max({M, pools[m]->h->Na, pools[m]->h->Nb});
@@ -850,9 +884,21 @@ hy_status build_screen_plan(ScreenPlan &sp, const hy_pool *const *pools, const i
     }
     sp.count = count;
     sp.n_tasks = int(tasks.size());
-    HY_CUDA(sp.arena.upload(&sp.d_mols, mols.data(), mols.size()), "upload screen plan");
-    HY_CUDA(sp.arena.upload(&sp.d_tasks, tasks.data(), tasks.size()), "upload screen tasks");
-    HY_CUDA(sp.arena.alloc(&sp.d_partials, size_t(sp.n_partials)), "screen partials");
+    DevPack pack;
+    const size_t o_mols = pack.add(mols), o_tasks = pack.add(tasks);
+    pack.extra = size_t(sp.n_partials) * sizeof(double);
+    if (pack.end() + pack.extra > sp.block_bytes) {
+        sp.arena.release();
+        sp.block_bytes = 0;
+        HY_CUDA(sp.arena.alloc(&sp.block, pack.end() + pack.extra), "screen plan");
+        sp.block_bytes = pack.end() + pack.extra;
+    }
+    HY_CUDA(cudaMemcpy(sp.block, pack.host.data(), pack.host.size(), cudaMemcpyHostToDevice), "screen plan");
+    sp.arena.uploaded += int64_t(pack.host.size());
+    unsigned char *d = sp.block;
+    sp.d_mols = reinterpret_cast<hy::k::ScreenMol *>(d + o_mols);
+    sp.d_tasks = reinterpret_cast<int4 *>(d + o_tasks);
+    sp.d_partials = reinterpret_cast<double *>(d + pack.end());
     return HY_OK;
 }
 
@@ -1661,29 +1707,34 @@ hy_status hy_pool_create(const hy_ham *h, hy_pool_kind kind, hy_pool **out)
         if (s == HY_OK && err != cudaSuccess) s = cuda_fail(err, what);
     };
     DevArena &ar = p->arena;
-    up(ar.upload(&p->d_op, p->opd.data(), p->opd.size()), "upload ops");
-    up(ar.upload(&p->d_cons, p->cons.data(), p->cons.size()), "upload constituents");
     up(ar.upload(&p->d_aent, p->pa.entry.data(), p->pa.entry.size()), "upload alpha pairs");
     up(ar.upload(&p->d_bent, p->pb.entry.data(), p->pb.entry.size()), "upload beta pairs");
-    up(ar.upload(&p->d_aoff, p->pa.off.data(), p->pa.off.size()), "upload offsets");
-    up(ar.upload(&p->d_acnt, p->pa.cnt.data(), p->pa.cnt.size()), "upload counts");
-    up(ar.upload(&p->d_boff, p->pb.off.data(), p->pb.off.size()), "upload offsets");
-    up(ar.upload(&p->d_bcnt, p->pb.cnt.data(), p->pb.cnt.size()), "upload counts");
-    {
-        std::vector<int32_t> desc;
-        desc.reserve(p->ops.size() * 11);
-        for (const auto &op : p->ops) desc.insert(desc.end(), op.desc, op.desc + 11);
-        up(ar.upload(&p->d_desc, desc.data(), desc.size()), "upload descriptors");
-        const unsigned long long none = ~0ull;
-        up(ar.upload(&p->d_bad, &none, 1), "upload list-check flag");
-        up(cudaMallocHost(&p->h_bad, sizeof(unsigned long long)), "list-check mirror");
-        if (p->h_bad) *p->h_bad = none;
-    }
+    std::vector<int32_t> desc;
+    desc.reserve(p->ops.size() * 11);
+    for (const auto &op : p->ops) desc.insert(desc.end(), op.desc, op.desc + 11);
+    const unsigned long long none = ~0ull;
+    DevPack pack;
+    std::vector<std::pair<void **, size_t>> at;         // pointers into it
+    auto put = [&](auto **dst, const auto &v) { at.push_back({reinterpret_cast<void **>(dst), pack.add(v)}); };
+    put(&p->d_op, p->opd);
+    put(&p->d_cons, p->cons);
+    put(&p->d_aoff, p->pa.off);
+    put(&p->d_acnt, p->pa.cnt);
+    put(&p->d_boff, p->pb.off);
+    put(&p->d_bcnt, p->pb.cnt);
+    put(&p->d_desc, desc);
+    put(&p->d_bad, std::vector<unsigned long long>{none});
     for (int spin = 0; spin < 2; ++spin) {
-        up(ar.upload(&p->d_sing[spin], p->sing[spin].data(), p->sing[spin].size()), "upload singles");
-        up(ar.upload(&p->d_dbl[spin], p->dbl[spin].data(), p->dbl[spin].size()), "upload doubles");
-        up(ar.upload(&p->d_slot[spin], slot[spin].data(), slot[spin].size()), "upload slots");
+        put(&p->d_sing[spin], p->sing[spin]);
+        put(&p->d_dbl[spin], p->dbl[spin]);
+        put(&p->d_slot[spin], slot[spin]);
     }
+    unsigned char *d = nullptr;
+    up(pack.upload(ar, &d), "upload pool tables");
+    if (s == HY_OK)
+        for (const auto &q : at) *q.first = d + q.second;
+    up(cudaMallocHost(&p->h_bad, sizeof(unsigned long long)), "list-check mirror");
+    if (p->h_bad) *p->h_bad = none;
     if (s == HY_OK) {
         const int64_t zero = 0;
         if (h->N >= hy::k::kScreenMinN) {
@@ -2429,6 +2480,7 @@ hy_status hy_batch_create(const hy_ham *const *hams, int count, hy_batch **out)
         for (int64_t r = 0; r < hams[i]->Na; ++r) tasks.push_back(make_int2(i, int(r)));
     b->n_tasks = int64_t(tasks.size());
     std::vector<int2> tasks64;
+    if (small64) tasks64.reserve(size_t(tb64));
     if (small64)
         for (int i : b->order)
             for (int64_t t = 0; t < rows64[i]; ++t) tasks64.push_back(make_int2(i, int(t)));
@@ -2449,11 +2501,18 @@ hy_status hy_batch_create(const hy_ham *const *hams, int count, hy_batch **out)
     put(&b->d_counter, static_cast<const int *>(nullptr), 1, "batch counter");
     put(&b->d_row_energy, static_cast<const double *>(nullptr), size_t(std::max(tb, tb64)),
         "batch partials");
-    if (small64) {
-        put(&b->d_rows64, r64.data(), r64.size(), "batch tables");
-        put(&b->d_tasks64, tasks64.data(), tasks64.size(), "batch tasks");
-        put(&b->d_base64, base64.data(), base64.size(), "batch tables");
-        put(&b->d_rows64n, rows64.data(), rows64.size(), "batch tables");
+    if (small64 && s == HY_OK) {
+        DevPack pack;
+        const size_t o_mols = pack.add(r64), o_tasks = pack.add(tasks64), o_base = pack.add(base64),
+                     o_rows = pack.add(rows64);
+        unsigned char *d = nullptr;
+        up(pack.upload(b->tables64, &d), "batch tables");
+        if (s == HY_OK) {
+            b->d_rows64 = reinterpret_cast<hy::k::Rows64Mol *>(d + o_mols);
+            b->d_tasks64 = reinterpret_cast<int2 *>(d + o_tasks);
+            b->d_base64 = reinterpret_cast<int64_t *>(d + o_base);
+            b->d_rows64n = reinterpret_cast<int64_t *>(d + o_rows);
+        }
     }
     put(&b->d_base, base.data(), base.size(), "batch tables");
     put(&b->d_rows, rows.data(), rows.size(), "batch tables");
@@ -2474,10 +2533,7 @@ hy_status hy_batch_destroy(hy_batch *b)
     cudaFree(b->d_mols64);
     cudaFree(b->d_mols32);
     cudaFree(b->d_tasks);
-    cudaFree(b->d_rows64);
-    cudaFree(b->d_tasks64);
-    cudaFree(b->d_base64);
-    cudaFree(b->d_rows64n);
+    b->tables64.release();
     cudaFree(b->d_counter);
     cudaFree(b->d_row_energy);
     cudaFree(b->d_base);

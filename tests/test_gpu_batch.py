@@ -166,3 +166,22 @@ def test_batch_gradients_match_oracle_and_lists(batch, dtype):
         b.gradients(psi, sig, ops=O, op_offsets=OF)
     gl2 = b.gradients(psi, sig, ops=O, op_offsets=OF).cpu().numpy()   # the report is cleared
     assert np.abs(gl2 - gl).max() <= ltol * max(1.0, np.abs(g).max())
+
+
+def test_pools_set_again():
+    """A batch given its pools again, and other ones, screens with the last: the plan is
+    made in the same memory."""
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2604_01176_gb300 as hy
+    hams = [hy.Hamiltonian(*synth.integrals(n, 30 + n), n, n // 2, n - n // 2) for n in (4, 7, 9, 6)]
+    batch = hy.Batch(hams)
+    psi = batch.pack([torch.from_numpy(synth.random_state(h.n_det, 1)).cuda() for h in hams])
+    sigma = batch.pack([torch.from_numpy(synth.random_state(h.n_det, 2)).cuda() for h in hams])
+    for kind in ("qeb", "sd", "sd", "qeb"):
+        pools = [hy.Pool(h, kind) for h in hams]
+        batch.set_pools(pools)
+        g = batch.gradients(psi, sigma)
+        refs = [p.gradients(x, y, ops=torch.arange(len(p), dtype=torch.int32, device="cuda"))
+                for p, x, y in zip(pools, batch.unpack(psi), batch.unpack(sigma))]
+        assert torch.max(torch.abs(g - torch.cat(refs))).item() <= 1e-12
