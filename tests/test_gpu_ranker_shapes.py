@@ -75,3 +75,51 @@ def test_wide_network_few_rows(hidden, rows):
     r = hy.Ranker(hidden=hidden, seed=3)
     x = torch.from_numpy(np.random.default_rng(5).standard_normal((300, 16)).astype(np.float32)).cuda()
     assert torch.equal(r.predict(x[:rows].contiguous()), r.predict(x)[:rows])
+
+
+def _touched(D, n, ann, cre):
+    """Weight of one constituent's domain from D, as hyperion.h defines the feature:
+    modes `ann` emptied and `cre` filled, in pairs."""
+    a = [(x, y) for x, y in zip(ann, cre) if x < n]
+    b = [(x - n, y - n) for x, y in zip(ann, cre) if x >= n]
+    if len(a) <= 1 and len(b) <= 1:
+        return max(D[a[0][0] * n + a[0][1] if a else 0, b[0][0] * n + b[0][1] if b else 0], 0.0)
+    if not b:
+        return np.sqrt(np.prod([max(D[x * n + y, 0], 0.0) for x, y in a]))
+    return np.sqrt(np.prod([max(D[0, x * n + y], 0.0) for x, y in b]))
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("cfg", [(3, 1, 2), (6, 3, 3), (9, 5, 4), (12, 6, 6), (16, 3, 4), (16, 8, 2)],
+                         ids=lambda c: "n%da%db%d" % c)
+def test_second_vector_weights(cfg, dtype):
+    """The two features that read both vectors' touched weights, from the shared
+    launches, against 64-bit arithmetic on the weights of each vector from its own call
+    (12,870 alpha strings: blocks of 16 rows and 160 threads).
+
+    Tolerance: the bound and the weight sum at most four float terms of a few roundings
+    each (1e-6 of them), log10 of values of up to 12 adds as much: 5e-6."""
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2604_01176_gb300 as hy
+    n, na, nb = cfg
+    ham = hy.Hamiltonian(*synth.integrals(n, 5), n, na, nb)
+    pool = hy.Pool(ham)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    v = torch.randn((2, ham.n_det), dtype=dtype, device="cuda", generator=g)
+    v[1] *= torch.linspace(0.1, 2.0, ham.n_det, dtype=dtype, device="cuda")     # other weights
+    psi, sigma = v[0].contiguous(), v[1].contiguous()
+    feat = hy.ranker_features(ham, pool, psi, sigma=sigma).cpu().numpy().astype(np.float64)
+    dp, ds = (hy.touched_weights(ham, x).cpu().numpy().astype(np.float64) for x in (psi, sigma))
+    for k, d in enumerate(pool.descriptors()):
+        bound = wsum = 0.0
+        for c in range(d[0]):
+            q = d[1 + 5 * c:6 + 5 * c]
+            cre, ann = [q[1], q[2]][:q[0]], [q[4], q[3]][:q[0]]
+            p, i = _touched(dp, n, ann, cre), _touched(dp, n, cre, ann)
+            sp, si = _touched(ds, n, ann, cre), _touched(ds, n, cre, ann)
+            bound += 2.0 * (np.sqrt(p * si) + np.sqrt(i * sp))
+            wsum += p + i
+        want = (np.log10(bound / np.sqrt(dp[0, 0] * ds[0, 0]) + 1e-12), np.log10(wsum / dp[0, 0] + 1e-12))
+        assert np.abs(feat[k, 10:12] - want).max() <= 5e-6
