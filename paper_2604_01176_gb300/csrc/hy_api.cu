@@ -2211,7 +2211,7 @@ hy_status hy_pool_gradients_sparse(const hy_ham *h, const hy_pool *p, const void
         a.chunks = sparse_chunks(h, n_ops, m);
         a.partials = reinterpret_cast<double *>(static_cast<char *>(hm->ws) + L.partials);
         a.desc = p->d_desc; a.ops = ops_or_null; a.n_ops = n_ops;
-        a.astr = h->d_astr; a.bstr = h->d_bstr; a.binom33 = h->d_binom; a.n = h->n;
+        a.astr = h->d_astr; a.bstr = h->d_bstr; a.n = h->n;
         a.rank16 = h->d_rank16;
         a.Nb = h->Nb; a.g = g_out; a.K = int64_t(p->ops.size()); a.bad = p->d_bad;
         a.qubit = p->qubit;
@@ -3496,7 +3496,7 @@ hy::k::SparseGradArgs<T> sparse_grad_args(const SparseState *s, const void *lam,
     a.list = s->list; a.m = 0; a.d_m = s->cnt; a.cap = s->cap; a.bits = s->bits;
     a.chunks = chunks; a.partials = partials;
     a.desc = p->d_desc; a.ops = ops; a.n_ops = n_ops;
-    a.astr = h->d_astr; a.bstr = h->d_bstr; a.binom33 = h->d_binom; a.n = h->n;
+    a.astr = h->d_astr; a.bstr = h->d_bstr; a.n = h->n;
     a.rank16 = h->d_rank16;
     a.Nb = h->Nb; a.g = g; a.K = int64_t(p->ops.size()); a.bad = p->d_bad;
     a.qubit = p->qubit;

@@ -362,7 +362,7 @@ struct SparseGradArgs {
     const int32_t *desc;     // [K][11] operator descriptors
     const int32_t *ops;      // operator list or nullptr (all)
     int64_t n_ops;
-    const uint32_t *astr, *bstr, *binom33;
+    const uint32_t *astr, *bstr;
     const uint16_t *rank16;  // [1 << n] colex rank of every n-bit string
     int n;
     int64_t Nb;

@@ -184,7 +184,8 @@ k_hpsi_scatter(SparseArgs<T> a)
 // ---------------------------------------------------------------------------
 
 // the runs of the sorted support by alpha string (unordered; the CTA of a run
-// counts its length from the bitmap) and the beta strings present
+// counts its length from the bitmap; or, with `first`, their first rows by string) and
+// the beta strings present
 __global__ void __launch_bounds__(256)
 k_sup_runs(const int64_t *__restrict__ list, const unsigned long long *__restrict__ cnt,
            int64_t cap, int64_t Nb, int64_t *__restrict__ runs, int32_t *__restrict__ ralpha,
@@ -197,11 +198,14 @@ k_sup_runs(const int64_t *__restrict__ list, const unsigned long long *__restric
         const int64_t d = list[t], A = d / Nb;
         flagB[d - A * Nb] = 1;
         if (t == 0 || list[t - 1] / Nb != A) {
+            flagA[A] = 1;
+            if (first) {                    // for k_sup_rows: by alpha string
+                first[A] = int32_t(t);
+                continue;
+            }
             const unsigned long long pos = atomicAdd(ctr + 0, 1ull);
             runs[pos] = t;
             ralpha[pos] = int32_t(A);
-            flagA[A] = 1;
-            if (first) first[A] = int32_t(t);
         }
     }
 }
