@@ -182,6 +182,7 @@ struct hy_ham {
     // workspace (grown on demand; growth synchronises the device)
     void *ws = nullptr;
     size_t ws_bytes = 0;
+    size_t ws_refused = 0;          // the least that an offer_ws found no memory for
     // row groups of a listed state for its touched weights (grown on demand,
     // with a device synchronisation)
     hy::k::TwGroups tw{nullptr, nullptr, nullptr, nullptr, nullptr, 0};
@@ -325,6 +326,19 @@ hy_status ensure_ws(hy_ham *h, size_t bytes)
     }
     h->ws_bytes = bytes;
     return HY_OK;
+}
+
+// The workspace of a call that can do without it: a first call makes what later ones of
+// its handle may need (they may be captured, and cannot allocate then).  Not while this
+// stream is being captured, and not asked for again once there was no memory for it
+void offer_ws(hy_ham *h, size_t bytes, cudaStream_t st)
+{
+    if (bytes <= h->ws_bytes || (h->ws_refused && bytes >= h->ws_refused)) return;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
+        ensure_ws(h, bytes) != HY_OK)
+        h->ws_refused = bytes;
+    cudaGetLastError();
 }
 
 size_t n_partials_needed(const hy_ham *h, int64_t n_ops)
@@ -555,6 +569,7 @@ hy_status apply_h_t(hy_ham *h, const T *psi, T *sigma, cudaStream_t st, int64_t 
     if constexpr (sizeof(T) == sizeof(double)) {
         // one launch where a few partner rows fit an SM twice over
         if (h->d_mbv) {
+            offer_ws(h, ws_layout(h, n_partials_needed(h, 0), sizeof(T)).total, st);
             const double rows_det = double(nr) * double(h->Nb);
             hy::ProfScope prof(HY_PROF_HPSI, st, 2.0 * rows_det * sizeof(T),
                                2.0 * double(hy::ham_connections(h)) * rows_det);
@@ -976,14 +991,15 @@ hy_status grad_t(hy_ham *h, const hy_pool *p, const T *psi, const T *sigma,
                 bytes += 4.0 * nr * nc * sizeof(T);
             }
     hy::ProfScope prof(HY_PROF_SCREEN, st, bytes);
+    const WsLayout L = ws_layout(h, n_partials_needed(h, n_ops), sizeof(T));
     // whole pools by pattern where that is the quicker; lists per operator
     if (!ops && screen_by_pattern(p, sizeof(T) == sizeof(float))) {
+        offer_ws(h, L.total, st);
         if constexpr (sizeof(T) == sizeof(double))
             return screen_run(p->screen, psi, sigma, p->screen.d_partials, g, st);
         else
             return screen32_run(h, p, psi, sigma, p->d_part32, g, st);
     }
-    const WsLayout L = ws_layout(h, n_partials_needed(h, n_ops), sizeof(T));
     hy_status s = ensure_ws(h, L.total);
     if (s != HY_OK) return s;
     hy::k::GradArgs<T> a;
