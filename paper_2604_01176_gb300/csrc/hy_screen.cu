@@ -113,9 +113,10 @@ __device__ __forceinline__ void stage_ab(double *p1, double *p2, const double *p
 // kind 0: alpha-beta task (idx = alpha pattern, nA = the identity); kind 1:
 // alpha doubles over columns; kind 2: beta doubles over rows.  chunk: the
 // task's groups are chunk, chunk + CH, ...; slice: its share of the patterns (one
-// slice unless the groups are too few)
-template <int CFG>
-__global__ void __launch_bounds__(kScThreads, 2)
+// slice unless the groups are too few).  OCC: CTAs that fit an SM's shared memory;
+// one alone has twice the registers (16 orbitals, 8+8: 300 -> 289 ms, 15, 8+7: 58.3 -> 55.4)
+template <int CFG, int OCC>
+__global__ void __launch_bounds__(kScThreads, OCC)
 k_screen(ScreenArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -288,12 +289,12 @@ k_screen_final(const ScreenMol *__restrict__ mols, int count, const double *__re
     if (lane == 0) g[i] = 2.0 * tot;
 }
 
-template <int CFG>
+template <int CFG, int OCC>
 cudaError_t screen_cfg(const ScreenArgs &a, int n_tasks, size_t smem, cudaStream_t st)
 {
-    cudaError_t e = allow_smem(k_screen<CFG>, smem);
+    cudaError_t e = allow_smem(k_screen<CFG, OCC>, smem);
     if (e != cudaSuccess) return e;
-    k_screen<CFG><<<unsigned(n_tasks), kScThreads, smem, st>>>(a);
+    k_screen<CFG, OCC><<<unsigned(n_tasks), kScThreads, smem, st>>>(a);
     hy::count_launch();
     return cudaGetLastError();
 }
@@ -302,9 +303,11 @@ cudaError_t screen_all(const ScreenArgs &a, int cfg, int n_tasks, size_t smem, i
                        int64_t n_ops, double *g, cudaStream_t st)
 {
     if (n_ops == 0) return cudaSuccess;
-    const cudaError_t e = cfg == 0 ? screen_cfg<0>(a, n_tasks, smem, st)
-                        : cfg == 1 ? screen_cfg<1>(a, n_tasks, smem, st)
-                                   : screen_cfg<2>(a, n_tasks, smem, st);
+    const bool two = smem <= 113 * 1024;
+    const cudaError_t e = cfg == 0 ? screen_cfg<0, 2>(a, n_tasks, smem, st)
+                        : cfg == 1 ? (two ? screen_cfg<1, 2>(a, n_tasks, smem, st)
+                                          : screen_cfg<1, 1>(a, n_tasks, smem, st))
+                                   : screen_cfg<2, 1>(a, n_tasks, smem, st);
     if (e != cudaSuccess) return e;
     k_screen_final<<<unsigned((n_ops + 7) / 8), 256, 0, st>>>(a.mols, count, a.partials, n_ops, g);
     hy::count_launch();
