@@ -363,16 +363,17 @@ k_cpl_tc(CplDenseArgs a, int *status, long long spin_limit, int issue)
 // The diagonal slot is one more row of W_J where 64 rows have room for it (all but 8
 // electrons in 16 orbitals: DIAG, summed in FP32 by the builders).  W_J is rounded
 // when it is split and the small products go first (hy_same.cu): the error of the
-// float H|psi> against double, 13 orbitals, 7+6: 2.9e-7 -> 2.3e-7.
+// float H|psi> against double, 11 orbitals, 6+5, 2.2e-7 -> 1.8e-7 (relative, l2).
 // r that no column of a tile holds is skipped.  k_cpl_tc's block-wide barrier
 // per chunk left it at 3,600 clocks per 32 types, 768 of them tensor time.
 // Bound by the hand-over of stages (build, fence, arrive, issue, commit): with
 // gathers, stores or MMAs left out one at a time it loses 0-13 %, with all of them
 // half.  Stages of 8 types (twice the hand-overs) cost 30 %, four groups of four
-// warps, a column's 16 types to a thread, 6-20 %.  Measured, whole float H|psi>:
-// 16 orbitals, 8+8 (66 of 129 ms left of the coupling's) 205 -> 143 ms; 13
-// orbitals, 7+6: 2,989 -> 1,713 us; 11 orbitals, 6+5: 285 -> 174 us; also with few
-// strings: 12 orbitals, 2+2: 62.6 -> 55.9 us.  The diagonal's sums by their own loop,
+// warps, a column's 16 types to a thread, 6-20 %; an issuing warp that meets and
+// elects anew at each stage 8 %.  Measured, whole float H|psi> with the same-spin parts
+// by rows: 16 orbitals, 8+8 (64 of 129 ms left of the coupling's) 205 -> 141 ms; 13
+// orbitals, 7+6: 2,989 -> 1,583 us; 11 orbitals, 6+5: 285 -> 162 us; also with few
+// strings: 12 orbitals, 2+2: 62.6 -> 56 us.  The diagonal's sums by their own loop,
 // all loads at once, gave 11 orbitals 5 % and 13 orbitals 2 % of that.
 // ---------------------------------------------------------------------------
 namespace {

@@ -15,8 +15,8 @@
 // evaluations of 12 operators at 20 qubits: 4,284 us with a launch per pass and
 // one thread summing each gradient's chunks, 2,475 with that sum by a warp and
 // H psi by rows, 1,631 with the chain in one launch on vectors in L2 (3 us a
-// rotation), 1,356 on vectors in shared memory with the pairs of a pass dealt to
-// all SMs (of which H psi 580).
+// rotation), 1,340 on vectors in shared memory with the pairs of a pass dealt to
+// all SMs (of which H psi 564).
 #include <cooperative_groups.h>
 
 #include "hy_kernels.cuh"

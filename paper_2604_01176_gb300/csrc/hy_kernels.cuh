@@ -125,8 +125,8 @@ cudaError_t coupling_tc(const CplDenseArgs &a, int *status, long long spin_limit
 // (same_used, same_fill: place and pack zeroed before, base the sums of count)
 // Strings of each spin from which it is used (of the Hamiltonian, not of the rows at
 // hand: a range of rows gives the full sweep's sums).  Below, a launch costs more
-// than the rows do: 462 strings 184 us by rows, 194 so (whole float H|psi>, 11
-// orbitals, 6+5); 560 strings 286 -> 269, 792 420 -> 387, 1,820 2,211 -> 1,599.
+// than the rows do: 462 strings 162 us by rows, 187 so (whole float H|psi>, 11
+// orbitals, 6+5); 560 strings 271 -> 257, 792 390 -> 369, 1,820 2,082 -> 1,485.
 constexpr int kSameStrings = 512;
 struct SameArgs {
     unsigned char *xpack;       // same_x_bytes of scratch: X as operands

@@ -22,8 +22,9 @@
 //   * warps 0-7 take finished accumulators out (two, each half of tensor memory,
 //     in turn): the tensor cores cut sums off toward zero, so 64 J are added there
 //     and the rest in FP32 registers.  Error of the float H|psi> against double, 14
-//     orbitals, 7+7: 3.3e-7 by rows (k_spmm), 3.2e-7 with 128 J, 2.7e-7 with 64,
-//     2.6e-7 with 32 (5 % slower); hi not rounded to nearest, 128 J: 4.4e-7;
+//     orbitals, 7+7, with the same coupling: 3.3e-7 by rows (k_spmm), 3.2e-7 with 128
+//     J, 2.7e-7 with 64, 2.6e-7 with 32 (5 % slower); hi not rounded to nearest, 128 J:
+//     4.4e-7 (2.1e-7 with 64 J since the coupling rounds too, hy_cpl_tc.cu);
 //   * warp 8 starts the copies;
 //   * warp 9 issues the MMAs in the leading CTA and passes the other one's stages
 //     on to it.
@@ -36,8 +37,8 @@
 // row; else it ends at once (6 of 969 us at 13 orbitals, 7+5, with the looking).
 // Measured: 12,870 strings squared 33.0 -> 12.3 ms a side (71 % of the MMA rate,
 // the rest between stages: 128 KB of L2 reads a pair and 1,536 clocks), 1,716 360 ->
-// 73 us; whole float H|psi>, 16 orbitals, 8+8, 142.9 -> 101.2 ms; 12 orbitals, 6+6,
-// 541 -> 492 us.
+// 73 us; whole float H|psi>, 16 orbitals, 8+8, 140.5 -> 99.0 ms; 13 orbitals, 7+5, 1,389
+// -> 974 us; 12 orbitals, 6+6, 490 -> 444 us.
 #include "hy_kernels.cuh"
 #include "hy_tc.cuh"
 
