@@ -88,7 +88,7 @@ struct DevPack {
     template <typename T>
     size_t add(const T *src, size_t count)
     {
-        const size_t at = (host.size() + 15) / 16 * 16;
+        const size_t at = end();
         host.resize(at + count * sizeof(T));
         if (count) std::memcpy(host.data() + at, src, count * sizeof(T));
         return at;
@@ -96,7 +96,7 @@ struct DevPack {
     template <typename T>
     size_t add(const std::vector<T> &v) { return add(v.data(), v.size()); }
     // where the bytes not copied start
-    size_t end() const { return (host.size() + 15) / 16 * 16; }
+    size_t end() const { return (host.size() + 255) / 256 * 256; }
     cudaError_t upload(DevArena &ar, unsigned char **base) const
     {
         const cudaError_t e = ar.alloc(base, end() + extra);
@@ -215,6 +215,7 @@ struct ScreenPlan {
     int4 *d_tasks = nullptr;
     double *d_partials = nullptr;
     int count = 0, cfg = 0, n_tasks = 0;
+    bool cut = false;               // some tasks are slices of patterns
     int64_t n_partials = 0, n_ops = 0;
     size_t smem = 0;
 };
@@ -835,7 +836,7 @@ hy_status build_screen_plan(ScreenPlan &sp, const hy_pool *const *pools, const i
         for (int j = 1; j < 4; ++j) total += double(k[j].groups) * k[j].cost;
     }
     // a task of a few hundred pairs is all latency: small totals are dealt to fewer (20
-    // molecules of 6 orbitals 56 -> 34 us, per operator 49; 3 of 8 orbitals 51 -> 39, 62)
+    // molecules of 6 orbitals 56 -> 45 us, per operator 49; 3 of 8 orbitals 51 -> 41, 62)
     const double per_task = std::max(total / (8.0 * num_sms), std::min(total / 64.0, 1024.0));
     auto deal = [&](const Kind &k) {
         const int64_t c = int64_t(std::ceil(double(k.groups) * k.cost / per_task));
@@ -843,14 +844,15 @@ hy_status build_screen_plan(ScreenPlan &sp, const hy_pool *const *pools, const i
     };
     // Few strings of one spin make few groups of the other's patterns, each of them a long
     // task (16 orbitals, 1 + 8 electrons: 16 rows of 784 doubles x 924 pairs).  A kind that
-    // is dealt a group a task and has more than half an SM's share in one is cut by
-    // pattern as well, as long as a slice sums as much as it stages: 16 x 12,870 strings
-    // 1,890 -> 150 us, 66 x 924 64 -> 45, 78 x 1,716 129 -> 80
-    const double half = total / (2.0 * num_sms);
+    // is dealt a group a task and has most of an SM's share in one is cut by pattern as
+    // well, as long as a slice sums as much as it stages: 16 x 12,870 strings 1,890 -> 150
+    // us, 66 x 924 64 -> 45, 78 x 1,716 129 -> 80; cut from half a share on, 120 x 252 and 286
+    // x 1,287 lose 5 %
+    const double share = total / num_sms;
     auto slices = [&](const Kind &k, int ch, int64_t patterns, double staged) {
-        if (ch < k.groups || patterns < 2) return 1;
+        if (ch < k.groups || patterns < 2 || k.cost < 0.8 * share) return 1;
         const double most = std::min(double(patterns), (k.cost - staged) / staged);
-        return int(std::max(1.0, std::min(std::ceil(k.cost / half), most)));
+        return int(std::max(1.0, std::min(std::ceil(2.0 * k.cost / share), most)));
     };
     for (int m : order) {
         const hy_pool *p = pools[m];
@@ -870,9 +872,9 @@ hy_status build_screen_plan(ScreenPlan &sp, const hy_pool *const *pools, const i
         q.nA = int(p->sing[0].size()); q.nB = int(p->sing[1].size());
         q.nRa = int(p->dbl[0].size()); q.nRb = int(p->dbl[1].size());
         // the identity (first in the list, a few times a single's pairs) shares
-        // the singles' chunk count, unless its tasks are long then
+        // the singles' chunk count, unless its tasks are of several shares then
         q.ch[0] = q.nA ? deal(k[0]) : deal(k[1]);
-        q.chi = double(k[1].groups) * k[1].cost > half * q.ch[0] ? deal(k[1]) : q.ch[0];
+        q.chi = double(k[1].groups) * k[1].cost > 2.05 * share * q.ch[0] ? deal(k[1]) : q.ch[0];
         q.zs[0] = slices(k[0], q.ch[0], q.nB, 2.0 * double(h->Nb));
         q.zs[1] = slices(k[1], q.chi, q.nB, 2.0 * double(h->Nb));
         q.base[0] = sp.n_partials;
@@ -897,6 +899,8 @@ hy_status build_screen_plan(ScreenPlan &sp, const hy_pool *const *pools, const i
                                                 size_t(nr + 3) / 4 * 32);
         }
     }
+    for (const hy::k::ScreenMol &q : mols)
+        sp.cut = sp.cut || q.chi != q.ch[0] || *std::max_element(q.zs, q.zs + 4) > 1;
     sp.count = count;
     sp.n_tasks = int(tasks.size());
     DevPack pack;
@@ -926,7 +930,7 @@ hy_status screen_run(const ScreenPlan &sp, const double *psi, const double *sigm
     a.psi = psi;
     a.sigma = sigma;
     a.partials = partials;
-    HY_CUDA(hy::k::screen_all(a, sp.cfg, sp.n_tasks, sp.smem, sp.count, sp.n_ops, g, st),
+    HY_CUDA(hy::k::screen_all(a, sp.cfg, sp.cut, sp.n_tasks, sp.smem, sp.count, sp.n_ops, g, st),
             "pool gradients");
     return HY_OK;
 }
@@ -941,8 +945,8 @@ int beta_single_pairs(const hy_pool *p)
 // where the narrow planes meet some hundred alpha strings (two electrons or holes in 16
 // orbitals beside 7 to 9): one CTA an SM then, for a state that L2 holds for the
 // per-operator kernel (120 x 12,870 strings 1,750 us, per operator 1,550 and, qubit
-// pool, 1,320; 16 x 12,870 150 against 188 and 172; 560 x 12,870 5,790 against 9,340 and
-// 7,790; 120 x 8,008 787 against 898 and 747)
+// pool, 1,320; 16 x 12,870 148 against 188 and 172; 560 x 12,870 5,650 against 9,340 and
+// 7,790; 120 x 8,008 770 against 898 and 747)
 bool screen_by_pattern(const hy_pool *p, bool f32)
 {
     const hy_ham *h = p->h;

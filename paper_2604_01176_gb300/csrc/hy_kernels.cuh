@@ -716,7 +716,7 @@ struct ScreenArgs {
     const double *psi, *sigma;
     double *partials;
 };
-cudaError_t screen_all(const ScreenArgs &a, int cfg, int n_tasks, size_t smem, int count,
+cudaError_t screen_all(const ScreenArgs &a, int cfg, bool cut, int n_tasks, size_t smem, int count,
                        int64_t n_ops, double *g, cudaStream_t st);
 
 // Screen of a whole pool on a float state (hy_screen32.cu), CH row chunks as in

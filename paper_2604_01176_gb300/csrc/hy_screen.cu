@@ -113,9 +113,10 @@ __device__ __forceinline__ void stage_ab(double *p1, double *p2, const double *p
 // kind 0: alpha-beta task (idx = alpha pattern, nA = the identity); kind 1:
 // alpha doubles over columns; kind 2: beta doubles over rows.  chunk: the
 // task's groups are chunk, chunk + CH, ...; slice: its share of the patterns (one
-// slice unless the groups are too few).  OCC: CTAs that fit an SM's shared memory;
+// slice unless the groups are too few, CUT: the plan has several somewhere, which
+// costs the other plans 1 to 2 us).  OCC: CTAs that fit an SM's shared memory;
 // one alone has twice the registers (16 orbitals, 8+8: 300 -> 289 ms, 15, 8+7: 58.3 -> 55.4)
-template <int CFG, int OCC>
+template <int CFG, int OCC, bool CUT>
 __global__ void __launch_bounds__(kScThreads, OCC)
 k_screen(ScreenArgs a)
 {
@@ -126,21 +127,27 @@ k_screen(ScreenArgs a)
     const ScreenMol &m = a.mols[tk.x];
     const double *psi = a.psi + m.off, *sig = a.sigma + m.off;
     const int Na = m.Na, Nb = m.Nb;
-    const int kind = tk.y, chunk = tk.w & 0xFFFF, slice = tk.w >> 16;
+    const int kind = tk.y, chunk = CUT ? tk.w & 0xFFFF : tk.w, slice = CUT ? tk.w >> 16 : 0;
+    int CH = m.ch[kind];
 
     if (kind == 0) {
         using U = std::conditional_t<CFG == 2, double, double2>;
         U *p1 = reinterpret_cast<U *>(smem_raw), *p2 = p1 + Nb;
         const int ia = tk.z;
         const bool ident = ia == m.nA;
-        const int CH = ident ? m.chi : m.ch[0], Z = m.zs[ident ? 1 : 0];
+        if (CUT && ident) CH = m.chi;
         const int cnt = ident ? Na : int(m.acnt[m.la[ia]]);
         const uint32_t *ae = ident ? nullptr : m.aent + m.aoff[m.la[ia]];
         // this warp's share [lo, hi) of the pairs of the slice's beta singles [b0, b1),
         // cut by pattern
         const uint32_t *bent = m.bent;
         const int nB = m.nB, cb = nB > 0 ? int(m.bcnt[m.lb[0]]) : 0;
-        const int b0 = nB * slice / Z, b1 = nB * (slice + 1) / Z;
+        int b0 = 0, b1 = nB;
+        if (CUT) {
+            const int Z = m.zs[ident ? 1 : 0];
+            b0 = nB * slice / Z;
+            b1 = nB * (slice + 1) / Z;
+        }
         const int tot = (b1 - b0) * cb;
         const int lo = b0 * cb + int(int64_t(tot) * warp / kScWarps);
         const int hi = b0 * cb + int(int64_t(tot) * (warp + 1) / kScWarps);
@@ -168,7 +175,7 @@ k_screen(ScreenArgs a)
 #pragma unroll
                 for (int s = 0; s < kScSeg; ++s)
                     if (sn[s]) sum_pairs<U, 1, 32>(acc[s], bent + so[s], sn[s], lane, p1, p2, 0);
-                if (!ident && slice == 0)
+                if (!ident && (!CUT || slice == 0))
                     for (int b = tid; b < Nb; b += kScThreads) term(aid, p1[b], p2[b], 0u);
             }
         }
@@ -182,10 +189,10 @@ k_screen(ScreenArgs a)
         const double v = warp_total(aid);
         if (lane == 0) red[warp][kScSeg] = v;
         __syncthreads();
-        double *out = a.partials + m.base[0] + (int64_t(ia) * m.ch[0] + chunk) * (nB + 1);
+        double *out = a.partials + m.base[0] + (int64_t(ia) * (CUT ? m.ch[0] : CH) + chunk) * (nB + 1);
         for (int i = tid; i <= b1 - b0; i += kScThreads) {
             const int p = i < b1 - b0 ? b0 + i : nB;
-            if (p == nB && slice) break;
+            if (CUT && p == nB && slice) break;
             double s = 0.0;
             if (p == nB) {
                 for (int w = 0; w < kScWarps; ++w) s += red[w][kScSeg];
@@ -204,12 +211,16 @@ k_screen(ScreenArgs a)
     // same-spin doubles: V vectors of Ns amplitudes, element s of vector v at
     // v * vst + s * sst
     constexpr int Q = CFG == 0 ? 4 : CFG == 1 ? 2 : 1;      // vectors per group
-    const int CH = m.ch[kind], Z = m.zs[kind + 1];
     const bool al = kind == 1;
     const int Ns = al ? Na : Nb, V = al ? Nb : Na;
     const int64_t sst = al ? Nb : 1, vst = al ? 1 : Nb;
     const int nAll = al ? m.nRa : m.nRb;
-    const int r0 = int(int64_t(nAll) * slice / Z), nR = int(int64_t(nAll) * (slice + 1) / Z) - r0;
+    int r0 = 0, nR = nAll;
+    if (CUT) {
+        const int Z = m.zs[kind + 1];
+        r0 = nAll * slice / Z;
+        nR = nAll * (slice + 1) / Z - r0;
+    }
     const int32_t *ids = (al ? m.ra : m.rb) + r0;
     const uint32_t *ent = al ? m.aent : m.bent;
     const int64_t *off = al ? m.aoff : m.boff, *cnts = al ? m.acnt : m.bcnt;
@@ -290,24 +301,27 @@ k_screen_final(const ScreenMol *__restrict__ mols, int count, const double *__re
 }
 
 template <int CFG, int OCC>
-cudaError_t screen_cfg(const ScreenArgs &a, int n_tasks, size_t smem, cudaStream_t st)
+cudaError_t screen_cfg(const ScreenArgs &a, bool cut, int n_tasks, size_t smem, cudaStream_t st)
 {
-    cudaError_t e = allow_smem(k_screen<CFG, OCC>, smem);
-    if (e != cudaSuccess) return e;
-    k_screen<CFG, OCC><<<unsigned(n_tasks), kScThreads, smem, st>>>(a);
-    hy::count_launch();
-    return cudaGetLastError();
+    auto run = [&](auto *kernel) {
+        const cudaError_t e = allow_smem(kernel, smem);
+        if (e != cudaSuccess) return e;
+        kernel<<<unsigned(n_tasks), kScThreads, smem, st>>>(a);
+        hy::count_launch();
+        return cudaGetLastError();
+    };
+    return cut ? run(k_screen<CFG, OCC, true>) : run(k_screen<CFG, OCC, false>);
 }
 
-cudaError_t screen_all(const ScreenArgs &a, int cfg, int n_tasks, size_t smem, int count,
+cudaError_t screen_all(const ScreenArgs &a, int cfg, bool cut, int n_tasks, size_t smem, int count,
                        int64_t n_ops, double *g, cudaStream_t st)
 {
     if (n_ops == 0) return cudaSuccess;
     const bool two = smem <= 113 * 1024;
-    const cudaError_t e = cfg == 0 ? screen_cfg<0, 2>(a, n_tasks, smem, st)
-                        : cfg == 1 ? (two ? screen_cfg<1, 2>(a, n_tasks, smem, st)
-                                          : screen_cfg<1, 1>(a, n_tasks, smem, st))
-                                   : screen_cfg<2, 1>(a, n_tasks, smem, st);
+    const cudaError_t e = cfg == 0 ? screen_cfg<0, 2>(a, cut, n_tasks, smem, st)
+                        : cfg == 1 ? (two ? screen_cfg<1, 2>(a, cut, n_tasks, smem, st)
+                                          : screen_cfg<1, 1>(a, cut, n_tasks, smem, st))
+                                   : screen_cfg<2, 1>(a, cut, n_tasks, smem, st);
     if (e != cudaSuccess) return e;
     k_screen_final<<<unsigned((n_ops + 7) / 8), 256, 0, st>>>(a.mols, count, a.partials, n_ops, g);
     hy::count_launch();
