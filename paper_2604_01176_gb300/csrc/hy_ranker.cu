@@ -1197,7 +1197,19 @@ hy_status hy_ranker_predict(hy_ranker *r, const float *feat, int64_t m, float *s
     if (!r || (m > 0 && (!feat || !score)) || m < 0) return rerr(HY_ERR_ARG, "bad arguments");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (m == 0) return HY_OK;
-    if (r->H >= r->F && (r->H <= 256 || (r->H <= hy::k::kMlpMaxHidden && m > hy::k::kMlpWideRows))) {
+    bool one = r->H >= r->F && r->H <= hy::k::kMlpMaxHidden, few = false;
+    if (one && r->H > 256) {
+        // few rows through the products, whose buffers the first call makes whatever its
+        // rows; in one launch while there are none (captured first, or no memory)
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (r->act_rows < hy::k::kMlpWideRows && cudaStreamIsCapturing(st, &cap) == cudaSuccess &&
+            cap == cudaStreamCaptureStatusNone)
+            ensure_act(r, hy::k::kMlpWideRows);
+        cudaGetLastError();
+        few = m <= hy::k::kMlpWideRows && r->act_rows >= hy::k::kMlpWideRows;
+        one = !few;
+    }
+    if (one) {
         hy::k::MlpWeights p;
         for (int l = 0; l < 4; ++l) {
             p.w[l] = r->w + r->woff[l];
@@ -1212,7 +1224,7 @@ hy_status hy_ranker_predict(hy_ranker *r, const float *feat, int64_t m, float *s
         hy::count_launch();
         return rcu(cudaGetLastError(), "mlp predict");
     }
-    const int64_t blk = 1 << 14;
+    const int64_t blk = few ? hy::k::kMlpWideRows : 1 << 14;
     RTRY(ensure_act(r, blk));
     for (int64_t o = 0; o < m; o += blk) {
         const int mm = int(m - o < blk ? m - o : blk);

@@ -50,3 +50,24 @@ def test_operator_list_after_a_whole_screen(dtype):
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(g, pool.gradients(psi, sigma, ops=ops))
+
+
+@pytest.mark.parametrize("hidden", [40, 300, 512])
+def test_few_rows_of_a_ranker_after_many(hidden):
+    """A wide network's products have their buffers from the first call, whatever its
+    rows; and a first call may be a captured one."""
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2604_01176_gb300 as hy
+    x = torch.randn((600, 16), device="cuda")
+    few = x[:9].contiguous()
+    for warm in (True, False):
+        r = hy.Ranker(hidden=hidden, seed=3)
+        if warm:
+            r.predict(x)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            out = r.predict(few)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out, r.predict(few))
