@@ -562,15 +562,28 @@ hy_status pack_same(hy_ham *h)
 // sigma rows [r0, r1) (alpha strings) of H psi; sigma holds those rows only.
 // Every output element is formed by the same arithmetic in the same order
 // whatever the range, so shards concatenate to the full sigma bit for bit.
+// own (sigma null then): sigma goes to the workspace's first state buffer, whose
+// place is known only here, once the workspace has its size
 template <typename T>
-hy_status apply_h_t(hy_ham *h, const T *psi, T *sigma, cudaStream_t st, int64_t r0, int64_t r1)
+hy_status apply_h_t(hy_ham *h, const T *psi, T *sigma, cudaStream_t st, int64_t r0, int64_t r1,
+                    T **own = nullptr)
 {
     const int64_t nr = r1 - r0;
     if (nr <= 0) return HY_OK;
+    auto place = [&](const WsLayout &L) {
+        if (own) *own = sigma = reinterpret_cast<T *>(static_cast<char *>(h->ws) + L.buf0);
+    };
     if constexpr (sizeof(T) == sizeof(double)) {
         // one launch where a few partner rows fit an SM twice over
         if (h->d_mbv) {
-            offer_ws(h, ws_layout(h, n_partials_needed(h, 0), sizeof(T)).total, st);
+            const WsLayout L = ws_layout(h, n_partials_needed(h, 0), sizeof(T));
+            if (own) {
+                const hy_status s = ensure_ws(h, L.total);
+                if (s != HY_OK) return s;
+            } else {
+                offer_ws(h, L.total, st);
+            }
+            place(L);
             const double rows_det = double(nr) * double(h->Nb);
             hy::ProfScope prof(HY_PROF_HPSI, st, 2.0 * rows_det * sizeof(T),
                                2.0 * double(hy::ham_connections(h)) * rows_det);
@@ -614,6 +627,7 @@ hy_status apply_h_t(hy_ham *h, const T *psi, T *sigma, cudaStream_t st, int64_t 
         hy_status s = ensure_ws(h, L.total);
         if (s != HY_OK) return s;
     }
+    place(L);
     char *ws = static_cast<char *>(h->ws);
     T *psiT = reinterpret_cast<T *>(ws + L.buf1);
     T *tau = reinterpret_cast<T *>(ws + L.buf2);
@@ -766,12 +780,9 @@ hy_status normalize_t(hy_ham *h, T *psi, cudaStream_t st)
 template <typename T>
 hy_status energy_t(hy_ham *h, const T *psi, const T *sigma, double *e, cudaStream_t st)
 {
-    const WsLayout L = ws_layout(h, n_partials_needed(h, 0), sizeof(T));
-    hy_status s = ensure_ws(h, L.total);
-    if (s != HY_OK) return s;
     if (!sigma) {
-        T *tmp = reinterpret_cast<T *>(static_cast<char *>(h->ws) + L.buf0);
-        s = apply_h_t<T>(h, psi, tmp, st, 0, h->Na);
+        T *tmp = nullptr;
+        const hy_status s = apply_h_t<T>(h, psi, nullptr, st, 0, h->Na, &tmp);
         if (s != HY_OK) return s;
         sigma = tmp;
     }
